@@ -6,13 +6,14 @@
 // shared entries (Sec. 3.2.1) is treated by the variant of fea_scatter:
 //   ATOMIC  FP64 atomic adds, the GPU form of Alg. "no coloring".
 //
-// Tile schedule of one CTA (128 threads, EPC elements):
+// FP64 tiles: pair_tile.cuh.  Tile schedule of one CTA in the FP32 precisions
+// (128 threads, EPC elements):
 //   phase 0  gather the node coordinates of the tile into shared memory
-//   phase 1  one thread per (element, quadrature point): Jacobian, det, J^{-1},
-//            physical gradients g_a and the weight w*detJ (FP64, or FP32 with
-//            an FP64 redo of distorted elements)
-//   phase 2  LPE = n_e * SPLIT lanes per element: lane (a, half) accumulates
-//            the row block A^e_(a, b) for its NB columns b over the points
+//   phase 1  one thread per (element, quadrature point): Jacobian, det, J^{-1}
+//            (FP64, or FP32 with an FP64 redo of distorted elements), physical
+//            gradients g_a and the weight w*detJ
+//   phase 2  n_e lanes per element: lane a accumulates the row block A^e_(a, b)
+//            for every column b over the points
 //   phase 3  the same lane scatters its row block through the rank map.
 #include <cmath>
 #include <cstddef>
@@ -23,6 +24,7 @@
 
 #include "element.cuh"
 #include "fea_internal.cuh"
+#include "pair_tile.cuh"
 #include "sched.cuh"
 
 namespace fea {
@@ -173,86 +175,41 @@ const RefRule& host_rule(int slot) {
 // ---------------------------------------------------------------------------
 // device
 // ---------------------------------------------------------------------------
-struct AsmParams {
-  const double* coords;
-  const int32_t* tconn;     // [n][NN] packed connectivity of the group
-  const int32_t* ids;       // [n] original element ids (nullptr: identity)
-  const int64_t* mapoff;    // [n] node_map offsets (nullptr: id * NN^2)
-  const int32_t* list;      // launch index -> index in the group (nullptr: identity; coloring)
-  int64_t n;                // elements of this launch
-  const int64_t* row_ptr;
-  const int32_t* node_map;
-  double* A;
-  double* b;
-  DevStatus* st;
-  double k0, k2, src;       // diffusion
-  double lam, mu;           // elasticity
-  double f[3];
-  int geo64;                // FP32 tiles: 1 = FP64 geometry for every element, 0 = adaptive
-};
-
-__device__ __forceinline__ int64_t group_index(const AsmParams& P, int64_t et) {
-  return P.list ? (int64_t)P.list[et] : et;
-}
-__device__ __forceinline__ int64_t original_id(const AsmParams& P, int64_t et) {
-  const int64_t g = group_index(P, et);
-  return P.ids ? (int64_t)P.ids[g] : g;
-}
-
-template <int OP, int PREC, int NN, int NQ, int EPC>
+template <int OP, int NN, int NQ, int EPC>
 struct TileSmem {
-  using R = typename std::conditional<PREC == FEA_FP64, double, float>::type;
   double X[EPC][NN][3];     // node coordinates
-  R G[EPC][NQ][NN][3];      // physical gradients
-  R S[EPC][NQ];             // w detJ k(x_q)
-  R W[EPC][NQ];             // w detJ
-  int flag[EPC];            // FP32 mode: element is distorted -> FP64 geometry
+  float G[EPC][NQ][NN][3];  // physical gradients
+  float S[EPC][NQ];         // w detJ k(x_q)
+  float W[EPC][NQ];         // w detJ
+  int flag[EPC];            // adaptive mode: element is distorted -> FP64 geometry
 };
 
-// Tile values of point q from the FP64 Jacobian J' = s J (s a power of two):
-// det J = det'/s^3, grad N_a = J^{-T} grad_xi N_a = s C' grad_xi N_a / det'.
-// FP64 tiles keep FP64; FP32 tiles round the cofactors and the determinant
-// once and form the gradients in FP32.
-// (the point's values from the cofactors C' and det' of J' = s J)
+// Tile values of point q from the cofactors C' and det' of the FP64 Jacobian
+// J' = s J (s a power of two): det J = det'/s^3, grad N_a = J^{-T} grad_xi N_a
+// = s C' grad_xi N_a / det'.  The cofactors and the determinant are rounded
+// once and the gradients formed in FP32.
 template <int OP, int NN, typename Smem>
 __device__ __forceinline__ void geometry_store(Smem& sm, const RefRule& rr, int le, int q, const double (&C)[3][3],
                                                double det, double s, double xq, const AsmParams& P) {
-  using R = std::remove_reference_t<decltype(sm.G[0][0][0][0])>;
-  if constexpr (std::is_same<R, double>::value) {
-    const double wd = rr.w[q] * det * (1.0 / (s * s * s));
-    const double inv = s / det;
+  float Cf[3][3];
 #pragma unroll
-    for (int a = 0; a < NN; ++a)
+  for (int i = 0; i < 3; ++i)
 #pragma unroll
-      for (int i = 0; i < 3; ++i)
-        // g_a,i = sum_j dN_a/dxi_j (J^{-1})_{j i},  (J^{-1})_{j i} = C_{i j} / det
-        sm.G[le][q][a][i] = (rr.dN[q][a][0] * C[i][0] + rr.dN[q][a][1] * C[i][1] + rr.dN[q][a][2] * C[i][2]) * inv;
-    sm.W[le][q] = wd;
-    if constexpr (OP == FEA_OP_DIFFUSION)
-      sm.S[le][q] = wd * (P.k0 + P.k2 * xq * xq);
-    else
-      sm.S[le][q] = wd;
-  } else {
-    float Cf[3][3];
+    for (int j = 0; j < 3; ++j) Cf[i][j] = f64_to_f32_rn(C[i][j]);
+  const float detf = f64_to_f32_rn(det);
+  const float inv = (float)s / detf;
+#pragma unroll
+  for (int a = 0; a < NN; ++a)
 #pragma unroll
     for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) Cf[i][j] = f64_to_f32_rn(C[i][j]);
-    const float detf = f64_to_f32_rn(det);
-    const float inv = (float)s / detf;
-#pragma unroll
-    for (int a = 0; a < NN; ++a)
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-        sm.G[le][q][a][i] = (rr.dNf[q][a][0] * Cf[i][0] + rr.dNf[q][a][1] * Cf[i][1] + rr.dNf[q][a][2] * Cf[i][2]) * inv;
-    const float wdf = rr.wf[q] * detf * (float)(1.0 / (s * s * s));
-    sm.W[le][q] = wdf;
-    if constexpr (OP == FEA_OP_DIFFUSION) {
-      const float x = f64_to_f32_rn(xq);
-      sm.S[le][q] = wdf * (f64_to_f32_rn(P.k0) + f64_to_f32_rn(P.k2) * x * x);
-    } else {
-      sm.S[le][q] = wdf;
-    }
+      sm.G[le][q][a][i] = (rr.dNf[q][a][0] * Cf[i][0] + rr.dNf[q][a][1] * Cf[i][1] + rr.dNf[q][a][2] * Cf[i][2]) * inv;
+  const float wdf = rr.wf[q] * detf * (float)(1.0 / (s * s * s));
+  sm.W[le][q] = wdf;
+  if constexpr (OP == FEA_OP_DIFFUSION) {
+    const float x = f64_to_f32_rn(xq);
+    sm.S[le][q] = wdf * (f64_to_f32_rn(P.k0) + f64_to_f32_rn(P.k2) * x * x);
+  } else {
+    sm.S[le][q] = wdf;
   }
 }
 
@@ -340,26 +297,24 @@ __device__ __forceinline__ bool geometry_fp32(Smem& sm, const RefRule& rr, int l
   return true;
 }
 
-template <int TYPE, int SLOT, int OP, int PREC, int SPLIT>
+template <int TYPE, int SLOT, int OP>
 struct TileCfg {
   static constexpr int NN = nodes_of(TYPE);
   static constexpr int NQ = rule_nq(SLOT);
   static constexpr int D = OP == FEA_OP_DIFFUSION ? 1 : 3;
-  static constexpr int LPE = NN * SPLIT;        // lanes per element
+  static constexpr int LPE = NN;                // lanes per element
   static constexpr int EPW = 32 / LPE;          // elements per warp
   static constexpr int WARPS = 4;
   static constexpr int THREADS = 32 * WARPS;
   static constexpr int EPC = EPW * WARPS;       // elements per CTA
-  static constexpr int NB = NN / SPLIT;         // columns per lane
+  static constexpr int NB = NN;                 // columns per lane
   static constexpr bool kModal = TYPE == FEA_HEX8 && SLOT == kRuleHex8;
-  static_assert(NN % SPLIT == 0, "SPLIT must divide the node count");
   static_assert(!kModal || (EPC * 8 % 32 == 0 && EPC * 8 <= THREADS), "modal hex geometry needs whole warps");
-  using R = typename std::conditional<PREC == FEA_FP64, double, float>::type;
-  using Smem = TileSmem<OP, PREC, NN, NQ, EPC>;
+  using Smem = TileSmem<OP, NN, NQ, EPC>;
 };
 
 // phases 0 and 1 for the tile of elements [e0, e0 + EPC)
-template <class Cfg, int OP, int PREC>
+template <class Cfg, int OP>
 __device__ __forceinline__ void tile_geometry(typename Cfg::Smem& sm, const RefRule& rr, const AsmParams& P,
                                               int64_t e0, int64_t n_end) {
   constexpr int NN = Cfg::NN, NQ = Cfg::NQ, EPC = Cfg::EPC;
@@ -376,7 +331,7 @@ __device__ __forceinline__ void tile_geometry(typename Cfg::Smem& sm, const RefR
   }
   if (threadIdx.x < EPC) sm.flag[threadIdx.x] = 0;
   __syncthreads();
-  const bool all64 = PREC == FEA_FP64 || P.geo64;  // uniform over the grid
+  const bool all64 = P.geo64;  // uniform over the grid
   if constexpr (kModal) {
     if (all64) {
       // trilinear hex in modal form: one lane per (element, corner p = point q);
@@ -431,108 +386,93 @@ __device__ __forceinline__ void tile_geometry(typename Cfg::Smem& sm, const RefR
         cofactors(J, C);
         const double det = J[0][0] * C[0][0] + J[0][1] * C[0][1] + J[0][2] * C[0][2];
         if (!(det > 0.0)) latch_error(P.st, FEA_ERR_INVERTED_ELEMENT, (unsigned long long)original_id(P, et));
-        if constexpr (PREC == FEA_FP64) {
+        // the FP32 roundings of C, det J and x at the points
+        // replace the element's coordinates (read above), and the points'
+        // values follow with one thread per point
+        float xf[NQ];
 #pragma unroll
-          for (int q = 0; q < NQ; ++q) {
-            double xq = sm.X[le][0][0];
+        for (int q = 0; q < NQ; ++q) {
+          double xq = sm.X[le][0][0];
 #pragma unroll
-            for (int a = 1; a < NN; ++a) xq += rr.N[q][a] * d[a][0];
-            geometry_store<OP, NN>(sm, rr, le, q, C, det, 1.0, xq, P);
-          }
-        } else {
-          // FP32 tiles: the FP32 roundings of C, det J and x at the points
-          // replace the element's coordinates (read above), and the points'
-          // values follow with one thread per point
-          float xf[NQ];
-#pragma unroll
-          for (int q = 0; q < NQ; ++q) {
-            double xq = sm.X[le][0][0];
-#pragma unroll
-            for (int a = 1; a < NN; ++a) xq += rr.N[q][a] * d[a][0];
-            xf[q] = OP == FEA_OP_DIFFUSION ? f64_to_f32_rn(xq) : 0.0f;
-          }
-          float* o = reinterpret_cast<float*>(&sm.X[le][0][0]);
-#pragma unroll
-          for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) o[3 * i + j] = f64_to_f32_rn(C[i][j]);
-          o[9] = f64_to_f32_rn(det);
-#pragma unroll
-          for (int q = 0; q < NQ; ++q) o[10 + q] = xf[q];
+          for (int a = 1; a < NN; ++a) xq += rr.N[q][a] * d[a][0];
+          xf[q] = OP == FEA_OP_DIFFUSION ? f64_to_f32_rn(xq) : 0.0f;
         }
+        float* o = reinterpret_cast<float*>(&sm.X[le][0][0]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+          for (int j = 0; j < 3; ++j) o[3 * i + j] = f64_to_f32_rn(C[i][j]);
+        o[9] = f64_to_f32_rn(det);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) o[10 + q] = xf[q];
       }
-      if constexpr (PREC != FEA_FP64) {
-        static_assert(10 + NQ <= NN * 3 * 2, "C, det J and x_q must fit the element's coordinate slot");
-        __syncthreads();
-        for (int t = threadIdx.x; t < EPC * NQ; t += Cfg::THREADS) {
-          const int le = t / NQ, q = t % NQ;
-          if (e0 + le >= n_end) continue;
-          const float* o = reinterpret_cast<const float*>(&sm.X[le][0][0]);
-          float Cf[3][3];
+      static_assert(10 + NQ <= NN * 3 * 2, "C, det J and x_q must fit the element's coordinate slot");
+      __syncthreads();
+      for (int t = threadIdx.x; t < EPC * NQ; t += Cfg::THREADS) {
+        const int le = t / NQ, q = t % NQ;
+        if (e0 + le >= n_end) continue;
+        const float* o = reinterpret_cast<const float*>(&sm.X[le][0][0]);
+        float Cf[3][3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+          for (int j = 0; j < 3; ++j) Cf[i][j] = o[3 * i + j];
+        const float detf = o[9];
+        const float inv = 1.0f / detf;
+#pragma unroll
+        for (int a = 0; a < NN; ++a)
 #pragma unroll
           for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = 0; j < 3; ++j) Cf[i][j] = o[3 * i + j];
-          const float detf = o[9];
-          const float inv = 1.0f / detf;
-#pragma unroll
-          for (int a = 0; a < NN; ++a)
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-              sm.G[le][q][a][i] =
-                  (rr.dNf[q][a][0] * Cf[i][0] + rr.dNf[q][a][1] * Cf[i][1] + rr.dNf[q][a][2] * Cf[i][2]) * inv;
-          const float wdf = rr.wf[q] * detf;
-          sm.W[le][q] = wdf;
-          if constexpr (OP == FEA_OP_DIFFUSION) {
-            const float x = o[10 + q];
-            sm.S[le][q] = wdf * (f64_to_f32_rn(P.k0) + f64_to_f32_rn(P.k2) * x * x);
-          } else {
-            sm.S[le][q] = wdf;
-          }
+            sm.G[le][q][a][i] =
+                (rr.dNf[q][a][0] * Cf[i][0] + rr.dNf[q][a][1] * Cf[i][1] + rr.dNf[q][a][2] * Cf[i][2]) * inv;
+        const float wdf = rr.wf[q] * detf;
+        sm.W[le][q] = wdf;
+        if constexpr (OP == FEA_OP_DIFFUSION) {
+          const float x = o[10 + q];
+          sm.S[le][q] = wdf * (f64_to_f32_rn(P.k0) + f64_to_f32_rn(P.k2) * x * x);
+        } else {
+          sm.S[le][q] = wdf;
         }
       }
       __syncthreads();
       return;
     }
   }
-  // FP64 hex (modal) and tet tiles have returned above
-  if constexpr (!(PREC == FEA_FP64 && (kModal || NN == 4))) {
-    if (all64) {
-      // the differences to node 0 once per element, not once per point
-      for (int t = threadIdx.x; t < EPC * (NN - 1) * 3; t += Cfg::THREADS) {
-        const int le = t / ((NN - 1) * 3), r = t % ((NN - 1) * 3);
-        if (e0 + le < n_end) sm.X[le][1 + r / 3][r % 3] -= sm.X[le][0][r % 3];
-      }
-      __syncthreads();
-    }
-    for (int t = threadIdx.x; t < EPC * NQ; t += Cfg::THREADS) {
-      const int le = t / NQ, q = t % NQ;
-      const int64_t et = e0 + le;
-      if (et >= n_end) continue;
-      if (all64) {
-        geometry_fp64<OP, NN, true>(sm, rr, le, q, original_id(P, et), P);
-      } else {
-        if (!geometry_fp32<OP, NN>(sm, rr, le, q, P)) sm.flag[le] = 1;
-      }
-    }
-    if (!all64) {
-      __syncthreads();
-      for (int t = threadIdx.x; t < EPC * NQ; t += Cfg::THREADS) {
-        const int le = t / NQ, q = t % NQ;
-        const int64_t et = e0 + le;
-        if (et < n_end && sm.flag[le]) geometry_fp64<OP, NN>(sm, rr, le, q, original_id(P, et), P);
-      }
+  if (all64) {
+    // the differences to node 0 once per element, not once per point
+    for (int t = threadIdx.x; t < EPC * (NN - 1) * 3; t += Cfg::THREADS) {
+      const int le = t / ((NN - 1) * 3), r = t % ((NN - 1) * 3);
+      if (e0 + le < n_end) sm.X[le][1 + r / 3][r % 3] -= sm.X[le][0][r % 3];
     }
     __syncthreads();
   }
+  for (int t = threadIdx.x; t < EPC * NQ; t += Cfg::THREADS) {
+    const int le = t / NQ, q = t % NQ;
+    const int64_t et = e0 + le;
+    if (et >= n_end) continue;
+    if (all64) {
+      geometry_fp64<OP, NN, true>(sm, rr, le, q, original_id(P, et), P);
+    } else {
+      if (!geometry_fp32<OP, NN>(sm, rr, le, q, P)) sm.flag[le] = 1;
+    }
+  }
+  if (!all64) {
+    __syncthreads();
+    for (int t = threadIdx.x; t < EPC * NQ; t += Cfg::THREADS) {
+      const int le = t / NQ, q = t % NQ;
+      const int64_t et = e0 + le;
+      if (et < n_end && sm.flag[le]) geometry_fp64<OP, NN>(sm, rr, le, q, original_id(P, et), P);
+    }
+  }
+  __syncthreads();
 }
 
-// phase 2: row block (a, columns b0 .. b0+NB) of element le, and its RHS
+// phase 2: row block of node a of element le, and its RHS
 template <class Cfg, int OP>
 __device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const RefRule& rr, const AsmParams& P,
-                                          int le, int a, int b0, typename Cfg::R (&K)[Cfg::NB][Cfg::D][Cfg::D],
-                                          typename Cfg::R (&rhs)[Cfg::D]) {
-  using R = typename Cfg::R;
+                                          int le, int a, float (&K)[Cfg::NB][Cfg::D][Cfg::D],
+                                          float (&rhs)[Cfg::D]) {
+  using R = float;
   constexpr int NB = Cfg::NB, D = Cfg::D, NQ = Cfg::NQ;
 #pragma unroll
   for (int bb = 0; bb < NB; ++bb)
@@ -551,7 +491,7 @@ __device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const Re
       const R sa0 = s * ga0, sa1 = s * ga1, sa2 = s * ga2;
 #pragma unroll
       for (int bb = 0; bb < NB; ++bb) {
-        const R* gb = sm.G[le][q][b0 + bb];
+        const R* gb = sm.G[le][q][bb];
         K[bb][0][0] += sa0 * gb[0] + sa1 * gb[1] + sa2 * gb[2];
       }
     } else {
@@ -559,7 +499,7 @@ __device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const Re
       const R gm[3] = {s * mu * ga0, s * mu * ga1, s * mu * ga2};
 #pragma unroll
       for (int bb = 0; bb < NB; ++bb) {
-        const R gb[3] = {sm.G[le][q][b0 + bb][0], sm.G[le][q][b0 + bb][1], sm.G[le][q][b0 + bb][2]};
+        const R gb[3] = {sm.G[le][q][bb][0], sm.G[le][q][bb][1], sm.G[le][q][bb][2]};
         const R dot = gm[0] * gb[0] + gm[1] * gb[1] + gm[2] * gb[2];
 #pragma unroll
         for (int c = 0; c < 3; ++c)
@@ -569,19 +509,12 @@ __device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const Re
         for (int c = 0; c < 3; ++c) K[bb][c][c] += dot;
       }
     }
-    if (b0 == 0) {
-      R Nqa;
-      if constexpr (std::is_same<R, double>::value)
-        Nqa = rr.N[q][a];
-      else
-        Nqa = rr.Nf[q][a];
-      const R wN = sm.W[le][q] * Nqa;
-      if constexpr (OP == FEA_OP_DIFFUSION)
-        rhs[0] += wN * (R)P.src;
-      else
+    const R wN = sm.W[le][q] * rr.Nf[q][a];
+    if constexpr (OP == FEA_OP_DIFFUSION)
+      rhs[0] += wN * (R)P.src;
+    else
 #pragma unroll
-        for (int c = 0; c < 3; ++c) rhs[c] += wN * (R)P.f[c];
-    }
+      for (int c = 0; c < 3; ++c) rhs[c] += wN * (R)P.f[c];
   }
 }
 
@@ -610,22 +543,21 @@ struct CoopScatter {
   // hex8 with the 2x2x2 rule (PB = 4, 16-byte staging stores) is the tile it
   // serves; staged in pairs of columns, the tet4 items of the 256-mesh batch
   // made it slower (17.97 against 17.09 ms)
-  static constexpr bool kOn = SC == FEA_SCATTER_ATOMIC && Cfg::D == 3 && Cfg::LPE == Cfg::NN && PB > 0 &&
-                              std::is_same<typename Cfg::R, float>::value && kWarpBytes % 16 == 0 &&
+  static constexpr bool kOn = SC == FEA_SCATTER_ATOMIC && Cfg::D == 3 && PB > 0 && kWarpBytes % 16 == 0 &&
                               (3 * PB) % 4 == 0;
 };
 
 // One tile of EPC elements starting at launch index e0 (elements at or past
-// n_end are skipped): integrate, then scatter each row block (a, b0..b0+NB),
+// n_end are skipped): integrate, then scatter each row block,
 // warp-cooperatively when COOP is set.  Every thread of the CTA must call it;
 // it ends with the shared memory free.
-template <int TYPE, int SLOT, int OP, int PREC, int SPLIT, int SC, bool COOP = false>
-__device__ __forceinline__ void tile_body(typename TileCfg<TYPE, SLOT, OP, PREC, SPLIT>::Smem& sm,
-                                          const RefRule& rr, const AsmParams& P, int64_t e0, int64_t n_end) {
-  using Cfg = TileCfg<TYPE, SLOT, OP, PREC, SPLIT>;
-  using R = typename Cfg::R;
+template <int TYPE, int SLOT, int OP, int SC, bool COOP = false>
+__device__ __forceinline__ void tile_body(typename TileCfg<TYPE, SLOT, OP>::Smem& sm, const RefRule& rr,
+                                          const AsmParams& P, int64_t e0, int64_t n_end) {
+  using Cfg = TileCfg<TYPE, SLOT, OP>;
+  using R = float;
   constexpr int NN = Cfg::NN, D = Cfg::D, NB = Cfg::NB, LPE = Cfg::LPE, EPW = Cfg::EPW;
-  tile_geometry<Cfg, OP, PREC>(sm, rr, P, e0, n_end);
+  tile_geometry<Cfg, OP>(sm, rr, P, e0, n_end);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int lw = lane / LPE;
@@ -643,7 +575,7 @@ __device__ __forceinline__ void tile_body(typename TileCfg<TYPE, SLOT, OP, PREC,
     int64_t node = 0;
     const int32_t* mp = nullptr;
     if (active) {
-      row_block<Cfg, OP>(sm, rr, P, le, a, 0, K, rhs);
+      row_block<Cfg, OP>(sm, rr, P, le, a, K, rhs);
       const int64_t g = group_index(P, et);
       node = P.tconn[g * NN + a];
       const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
@@ -698,17 +630,16 @@ __device__ __forceinline__ void tile_body(typename TileCfg<TYPE, SLOT, OP, PREC,
     return;
   }
   if (lw < EPW && et < n_end) {
-    const int r = lane % LPE;
-    const int a = r % NN, b0 = (r / NN) * NB;
+    const int a = lane % LPE;
 
     R K[NB][D][D], rhs[D];
-    row_block<Cfg, OP>(sm, rr, P, le, a, b0, K, rhs);
+    row_block<Cfg, OP>(sm, rr, P, le, a, K, rhs);
 
     const int64_t g = group_index(P, et);
     const int64_t node = P.tconn[g * NN + a];
     const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
     const int64_t moff = P.mapoff ? P.mapoff[g] : id * NN * NN;
-    const int32_t* mp = P.node_map + moff + a * NN + b0;
+    const int32_t* mp = P.node_map + moff + a * NN;
     int64_t rb[D];
 #pragma unroll
     for (int c = 0; c < D; ++c) rb[c] = P.row_ptr[D * node + c];
@@ -730,13 +661,11 @@ __device__ __forceinline__ void tile_body(typename TileCfg<TYPE, SLOT, OP, PREC,
 #pragma unroll
           for (int cc = 0; cc < D; ++cc) __stcg(P.A + rb[c] + D * k + cc, old[c][cc] + widen(K[bb][c][cc]));
       }
-      if (b0 == 0) {
-        double ob[D];
+      double ob[D];
 #pragma unroll
-        for (int c = 0; c < D; ++c) ob[c] = __ldcg(P.b + D * node + c);
+      for (int c = 0; c < D; ++c) ob[c] = __ldcg(P.b + D * node + c);
 #pragma unroll
-        for (int c = 0; c < D; ++c) __stcg(P.b + D * node + c, ob[c] + widen(rhs[c]));
-      }
+      for (int c = 0; c < D; ++c) __stcg(P.b + D * node + c, ob[c] + widen(rhs[c]));
     } else {
 #pragma unroll
       for (int bb = 0; bb < NB; ++bb) {
@@ -746,13 +675,38 @@ __device__ __forceinline__ void tile_body(typename TileCfg<TYPE, SLOT, OP, PREC,
 #pragma unroll
           for (int cc = 0; cc < D; ++cc) scatter_add<SC>(P.A + rb[c] + D * k + cc, widen(K[bb][c][cc]));
       }
-      if (b0 == 0)
 #pragma unroll
-        for (int c = 0; c < D; ++c) scatter_add<SC>(P.b + D * node + c, widen(rhs[c]));
+      for (int c = 0; c < D; ++c) scatter_add<SC>(P.b + D * node + c, widen(rhs[c]));
     }
   }
   __syncthreads();
 }
+
+// The tile of an element type in a precision: FP64 by node pairs
+// (pair_tile.cuh), else by row blocks.
+template <int TYPE, int SLOT, int OP, int PREC>
+struct Tile {
+  using Cfg = TileCfg<TYPE, SLOT, OP>;
+  using Smem = typename Cfg::Smem;
+  template <int SC, bool COOP>
+  __device__ static __forceinline__ void run(unsigned char* raw, const RefRule& rr, const AsmParams& P, int64_t e0,
+                                             int64_t n_end) {
+    tile_body<TYPE, SLOT, OP, SC, COOP && CoopScatter<Cfg, SC>::kOn>(*reinterpret_cast<Smem*>(raw), rr, P, e0, n_end);
+  }
+  // CTAs per SM its own kernel is compiled for (0: the compiler's choice)
+  static constexpr int min_blocks(int sc) { return sc == FEA_SCATTER_ATOMIC && CoopScatter<Cfg, FEA_SCATTER_ATOMIC>::kOn ? 4 : 0; }
+};
+template <int TYPE, int SLOT, int OP>
+struct Tile<TYPE, SLOT, OP, FEA_FP64> {
+  using Cfg = PairCfg<TYPE, SLOT, OP>;
+  using Smem = typename Cfg::Smem;
+  template <int SC, bool COOP>
+  __device__ static __forceinline__ void run(unsigned char* raw, const RefRule& rr, const AsmParams& P, int64_t e0,
+                                             int64_t n_end) {
+    pair_tile_body<TYPE, SLOT, OP, SC>(*reinterpret_cast<Smem*>(raw), rr, P, e0, n_end);
+  }
+  static constexpr int min_blocks(int) { return 0; }
+};
 
 // Tile kernel: one tile per CTA.  Where the scatter is warp-cooperative its
 // staging needs about 15 more registers than the plain one; at four CTAs per
@@ -762,13 +716,12 @@ __device__ __forceinline__ void tile_body(typename TileCfg<TYPE, SLOT, OP, PREC,
 // bound of 0), and the persistent kernels the plain scatter: there the
 // staging measured slower (8.22 against 7.48 ms; 256 meshes: 19.0 against
 // 18.4 ms).
-template <int TYPE, int SLOT, int OP, int PREC, int SPLIT, int SC>
-__global__ void __launch_bounds__(128, CoopScatter<TileCfg<TYPE, SLOT, OP, PREC, SPLIT>, SC>::kOn ? 4 : 0)
+template <int TYPE, int SLOT, int OP, int PREC, int SC>
+__global__ void __launch_bounds__(128, (Tile<TYPE, SLOT, OP, PREC>::min_blocks(SC)))
     k_assemble_tile(const __grid_constant__ RefRule rr, const __grid_constant__ AsmParams P) {
-  using Cfg = TileCfg<TYPE, SLOT, OP, PREC, SPLIT>;
+  using T = Tile<TYPE, SLOT, OP, PREC>;
   extern __shared__ __align__(16) unsigned char tile_smem[];
-  auto& sm = *reinterpret_cast<typename Cfg::Smem*>(tile_smem);
-  tile_body<TYPE, SLOT, OP, PREC, SPLIT, SC, CoopScatter<Cfg, SC>::kOn>(sm, rr, P, (int64_t)blockIdx.x * Cfg::EPC, P.n);
+  T::template run<SC, true>(tile_smem, rr, P, (int64_t)blockIdx.x * T::Cfg::EPC, P.n);
 }
 
 // ---------------------------------------------------------------------------
@@ -786,52 +739,50 @@ struct PersistAsmArgs {
 
 template <int OP, int PREC>
 struct PersistCfg {
-  static constexpr int S2 = (OP == FEA_OP_ELASTICITY && PREC == FEA_FP64) ? 2 : 1;
   // CTAs per SM the any-type kernel is compiled for.  Its register count is
   // the largest tile body's plus the call sequence (120 for FP32 diffusion),
   // while the light types' own tiles need 46-56; measured on GB300 (4.53 M
   // mixed elements, FP32 diffusion: 4.26 ms with no bound, 4.00 at 5, 3.90 at
   // 6, 3.86 at 8; 256 elasticity meshes, FP32: 19.5 ms with no bound, 18.4
   // at 5, 19.9 at 6, where spills start to cost more than the occupancy
-  // gains).  FP64 keeps the compiler's choice.  FP32 elasticity hex items
+  // gains).  FP64 takes 6 (80 registers; a single tile's kernel needs 40-62,
+  // the compiler's choice here was 116-132).  FP32 elasticity hex items
   // scatter warp-cooperatively (CoopScatter), which needs 4 CTAs per SM: the
   // 256 meshes 18.3 ms plain at 5, 19.3 cooperative at 5, 17.1 at 4, 18.8
   // at 3.  The hex-only kernel (ONLY) keeps the plain scatter: cooperative,
   // without a bound, it measured 8.56 against 7.46 ms on 2.1 M hexes.
-  static constexpr int kMinBlocks = PREC == FEA_FP64 ? 1 : OP == FEA_OP_DIFFUSION ? 8 : 4;
+  static constexpr int kMinBlocks = PREC == FEA_FP64 ? 6 : OP == FEA_OP_DIFFUSION ? 8 : 4;
+  // the hex-only kernel's
+  static constexpr int kMinBlocksHex = PREC == FEA_FP64 ? 6 : 1;
   static constexpr bool kCoop = true;
-  template <int TYPE, int SLOT, int SPLIT>
-  static constexpr size_t bytes() { return sizeof(typename TileCfg<TYPE, SLOT, OP, PREC, SPLIT>::Smem); }
+  template <int TYPE, int SLOT>
+  static constexpr size_t bytes() { return sizeof(typename Tile<TYPE, SLOT, OP, PREC>::Smem); }
   static constexpr size_t mx(size_t a, size_t b) { return a > b ? a : b; }
-  static constexpr size_t smem =
-      mx(mx(mx(bytes<FEA_TET4, kRuleTet1, 1>(), bytes<FEA_TET4, kRuleTet4, 1>()), bytes<FEA_PYR5, kRulePyr8, 1>()),
-         mx(bytes<FEA_PRISM6, kRulePrism6, S2>(), bytes<FEA_HEX8, kRuleHex8, S2>()));
+  static constexpr size_t smem = mx(mx(mx(bytes<FEA_TET4, kRuleTet1>(), bytes<FEA_TET4, kRuleTet4>()),
+                                       bytes<FEA_PYR5, kRulePyr8>()),
+                                    mx(bytes<FEA_PRISM6, kRulePrism6>(), bytes<FEA_HEX8, kRuleHex8>()));
 };
 
-template <int TYPE, int SLOT, int OP, int PREC, int SPLIT, int SC = FEA_SCATTER_ATOMIC, bool COOP = false>
+template <int TYPE, int SLOT, int OP, int PREC, int SC = FEA_SCATTER_ATOMIC, bool COOP = false>
 __device__ __forceinline__ void persist_item(unsigned char* raw, const AsmParams& P, int64_t first, int64_t end) {
-  using Cfg = TileCfg<TYPE, SLOT, OP, PREC, SPLIT>;
-  auto& sm = *reinterpret_cast<typename Cfg::Smem*>(raw);
-  constexpr bool kCoop = COOP && CoopScatter<Cfg, SC>::kOn;
-  for (int64_t e0 = first; e0 < end; e0 += Cfg::EPC)
-    tile_body<TYPE, SLOT, OP, PREC, SPLIT, SC, kCoop>(sm, c_rules[SLOT], P, e0, end);
+  using T = Tile<TYPE, SLOT, OP, PREC>;
+  for (int64_t e0 = first; e0 < end; e0 += T::Cfg::EPC) T::template run<SC, COOP>(raw, c_rules[SLOT], P, e0, end);
 }
 
 // One item of the any-type kernel, not inlined: the switch over five inlined
 // tile bodies made ptxas allocate well above the largest body's registers
 // (FP32 diffusion: 128 against 72), which cut the all-type launch's
 // occupancy; a call keeps the kernel near the largest body (96).
-template <int TYPE, int SLOT, int OP, int PREC, int SPLIT>
+template <int TYPE, int SLOT, int OP, int PREC>
 __device__ __noinline__ void persist_item_call(unsigned char* raw, const AsmParams& P, int64_t first, int64_t end) {
-  persist_item<TYPE, SLOT, OP, PREC, SPLIT, FEA_SCATTER_ATOMIC, PersistCfg<OP, PREC>::kCoop>(raw, P, first, end);
+  persist_item<TYPE, SLOT, OP, PREC, FEA_SCATTER_ATOMIC, PersistCfg<OP, PREC>::kCoop>(raw, P, first, end);
 }
 
 // ONLY >= 0: every item uses that rule slot (a single-type mesh), so the
 // kernel holds one tile body and its register budget; -1: any element type
 template <int OP, int PREC, int ONLY>
-__global__ void __launch_bounds__(128, ONLY < 0 ? PersistCfg<OP, PREC>::kMinBlocks : 1)
+__global__ void __launch_bounds__(128, ONLY < 0 ? PersistCfg<OP, PREC>::kMinBlocks : PersistCfg<OP, PREC>::kMinBlocksHex)
     k_persistent(const __grid_constant__ PersistAsmArgs A) {
-  constexpr int S2 = PersistCfg<OP, PREC>::S2;
   extern __shared__ __align__(16) unsigned char persist_smem[];
   __shared__ int s_item;
   sched_start(A.S);
@@ -845,25 +796,25 @@ __global__ void __launch_bounds__(128, ONLY < 0 ? PersistCfg<OP, PREC>::kMinBloc
     // single mesh: entry t is type t, read at a constant offset of the
     // parameter space; batches: the device table
     if constexpr (ONLY == kRuleHex8) {
-      persist_item<FEA_HEX8, kRuleHex8, OP, PREC, S2>(persist_smem, A.table[FEA_HEX8], first, end);
+      persist_item<FEA_HEX8, kRuleHex8, OP, PREC>(persist_smem, A.table[FEA_HEX8], first, end);
     } else if (A.tab) {
       const AsmParams& P = A.tab[it.entry];
       switch (A.tab_slot[it.entry]) {
-        case kRuleTet1: persist_item_call<FEA_TET4, kRuleTet1, OP, PREC, 1>(persist_smem, P, first, end); break;
-        case kRuleTet4: persist_item_call<FEA_TET4, kRuleTet4, OP, PREC, 1>(persist_smem, P, first, end); break;
-        case kRulePyr8: persist_item_call<FEA_PYR5, kRulePyr8, OP, PREC, 1>(persist_smem, P, first, end); break;
-        case kRulePrism6: persist_item_call<FEA_PRISM6, kRulePrism6, OP, PREC, S2>(persist_smem, P, first, end); break;
-        default: persist_item_call<FEA_HEX8, kRuleHex8, OP, PREC, S2>(persist_smem, P, first, end); break;
+        case kRuleTet1: persist_item_call<FEA_TET4, kRuleTet1, OP, PREC>(persist_smem, P, first, end); break;
+        case kRuleTet4: persist_item_call<FEA_TET4, kRuleTet4, OP, PREC>(persist_smem, P, first, end); break;
+        case kRulePyr8: persist_item_call<FEA_PYR5, kRulePyr8, OP, PREC>(persist_smem, P, first, end); break;
+        case kRulePrism6: persist_item_call<FEA_PRISM6, kRulePrism6, OP, PREC>(persist_smem, P, first, end); break;
+        default: persist_item_call<FEA_HEX8, kRuleHex8, OP, PREC>(persist_smem, P, first, end); break;
       }
     } else {
       switch (A.slot[it.entry]) {
-        case kRuleTet1: persist_item_call<FEA_TET4, kRuleTet1, OP, PREC, 1>(persist_smem, A.table[FEA_TET4], first, end); break;
-        case kRuleTet4: persist_item_call<FEA_TET4, kRuleTet4, OP, PREC, 1>(persist_smem, A.table[FEA_TET4], first, end); break;
-        case kRulePyr8: persist_item_call<FEA_PYR5, kRulePyr8, OP, PREC, 1>(persist_smem, A.table[FEA_PYR5], first, end); break;
+        case kRuleTet1: persist_item_call<FEA_TET4, kRuleTet1, OP, PREC>(persist_smem, A.table[FEA_TET4], first, end); break;
+        case kRuleTet4: persist_item_call<FEA_TET4, kRuleTet4, OP, PREC>(persist_smem, A.table[FEA_TET4], first, end); break;
+        case kRulePyr8: persist_item_call<FEA_PYR5, kRulePyr8, OP, PREC>(persist_smem, A.table[FEA_PYR5], first, end); break;
         case kRulePrism6:
-          persist_item_call<FEA_PRISM6, kRulePrism6, OP, PREC, S2>(persist_smem, A.table[FEA_PRISM6], first, end);
+          persist_item_call<FEA_PRISM6, kRulePrism6, OP, PREC>(persist_smem, A.table[FEA_PRISM6], first, end);
           break;
-        default: persist_item_call<FEA_HEX8, kRuleHex8, OP, PREC, S2>(persist_smem, A.table[FEA_HEX8], first, end); break;
+        default: persist_item_call<FEA_HEX8, kRuleHex8, OP, PREC>(persist_smem, A.table[FEA_HEX8], first, end); break;
       }
     }
     sched_record(A.S, item, it.entry, t0);
@@ -963,7 +914,6 @@ __device__ int mdep_next(const MdepArgs& A, int& cursor) {
 
 template <int OP, int PREC, int ONLY>
 __global__ void __launch_bounds__(128) k_multidep(const __grid_constant__ MdepArgs A) {
-  constexpr int S2 = PersistCfg<OP, PREC>::S2;
   constexpr int MD = FEA_SCATTER_MULTIDEP;
   extern __shared__ __align__(16) unsigned char mdep_smem[];
   __shared__ int s_sub;
@@ -986,14 +936,14 @@ __global__ void __launch_bounds__(128) k_multidep(const __grid_constant__ MdepAr
     for (int64_t c = A.cb_off[k]; c + 1 < A.cb_off[k + 1]; ++c) {
       const int64_t p0 = A.cb[c], p1 = A.cb[c + 1];
       if constexpr (ONLY == kRuleHex8) {
-        persist_item<FEA_HEX8, kRuleHex8, OP, PREC, S2, MD>(mdep_smem, P, p0, p1);
+        persist_item<FEA_HEX8, kRuleHex8, OP, PREC, MD>(mdep_smem, P, p0, p1);
       } else {
         switch (A.slot[w.entry]) {
-          case kRuleTet1: persist_item<FEA_TET4, kRuleTet1, OP, PREC, 1, MD>(mdep_smem, P, p0, p1); break;
-          case kRuleTet4: persist_item<FEA_TET4, kRuleTet4, OP, PREC, 1, MD>(mdep_smem, P, p0, p1); break;
-          case kRulePyr8: persist_item<FEA_PYR5, kRulePyr8, OP, PREC, 1, MD>(mdep_smem, P, p0, p1); break;
-          case kRulePrism6: persist_item<FEA_PRISM6, kRulePrism6, OP, PREC, S2, MD>(mdep_smem, P, p0, p1); break;
-          default: persist_item<FEA_HEX8, kRuleHex8, OP, PREC, S2, MD>(mdep_smem, P, p0, p1); break;
+          case kRuleTet1: persist_item<FEA_TET4, kRuleTet1, OP, PREC, MD>(mdep_smem, P, p0, p1); break;
+          case kRuleTet4: persist_item<FEA_TET4, kRuleTet4, OP, PREC, MD>(mdep_smem, P, p0, p1); break;
+          case kRulePyr8: persist_item<FEA_PYR5, kRulePyr8, OP, PREC, MD>(mdep_smem, P, p0, p1); break;
+          case kRulePrism6: persist_item<FEA_PRISM6, kRulePrism6, OP, PREC, MD>(mdep_smem, P, p0, p1); break;
+          default: persist_item<FEA_HEX8, kRuleHex8, OP, PREC, MD>(mdep_smem, P, p0, p1); break;
         }
       }
     }
@@ -1054,8 +1004,7 @@ static int rule_slot_of(int type, int tet_rule) {
 
 template <int OP, int PREC, int ONLY>
 static int launch_persistent_k(const PersistAsmArgs& args, int n_ctas, bool dry, cudaStream_t s, int* grid_out) {
-  constexpr size_t smem = ONLY == kRuleHex8 ? sizeof(typename TileCfg<FEA_HEX8, kRuleHex8, OP, PREC,
-                                                                       PersistCfg<OP, PREC>::S2>::Smem)
+  constexpr size_t smem = ONLY == kRuleHex8 ? sizeof(typename Tile<FEA_HEX8, kRuleHex8, OP, PREC>::Smem)
                                             : PersistCfg<OP, PREC>::smem;
   auto kern = k_persistent<OP, PREC, ONLY>;
   if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1151,8 +1100,7 @@ int launch_persistent_assemble(const fea_operator* op, fea_mesh* m, const int64_
 
 template <int OP, int PREC, int ONLY>
 static int launch_multidep_k(const MdepArgs& args, int n_ctas, cudaStream_t s) {
-  constexpr size_t smem = ONLY == kRuleHex8 ? sizeof(typename TileCfg<FEA_HEX8, kRuleHex8, OP, PREC,
-                                                                       PersistCfg<OP, PREC>::S2>::Smem)
+  constexpr size_t smem = ONLY == kRuleHex8 ? sizeof(typename Tile<FEA_HEX8, kRuleHex8, OP, PREC>::Smem)
                                             : PersistCfg<OP, PREC>::smem;
   auto kern = k_multidep<OP, PREC, ONLY>;
   if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1226,32 +1174,30 @@ int launch_multidep(const fea_operator* op, fea_mesh* m, const MultidepPlan& pla
 // ---------------------------------------------------------------------------
 // host dispatch
 // ---------------------------------------------------------------------------
-template <int TYPE, int SLOT, int OP, int PREC, int SPLIT, int SC>
+template <int TYPE, int SLOT, int OP, int PREC, int SC>
 static int launch_tile(const AsmParams& P, cudaStream_t s) {
-  using Cfg = TileCfg<TYPE, SLOT, OP, PREC, SPLIT>;
-  const unsigned grid = grid_for(P.n, Cfg::EPC);
-  constexpr size_t smem = sizeof(typename Cfg::Smem);
-  auto kern = k_assemble_tile<TYPE, SLOT, OP, PREC, SPLIT, SC>;
+  using T = Tile<TYPE, SLOT, OP, PREC>;
+  const unsigned grid = grid_for(P.n, T::Cfg::EPC);
+  constexpr size_t smem = sizeof(typename T::Smem);
+  auto kern = k_assemble_tile<TYPE, SLOT, OP, PREC, SC>;
   if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<grid, Cfg::THREADS, smem, s>>>(host_rule(SLOT), P);
+  kern<<<grid, T::Cfg::THREADS, smem, s>>>(host_rule(SLOT), P);
   FEA_CUDA(cudaGetLastError());
   return FEA_OK;
 }
 
 template <int OP, int PREC, int SC>
 static int launch_group_sc(int type, int tet_rule, const AsmParams& P, cudaStream_t s) {
-  // FP64 elasticity splits the columns of hex8 / prism6 over two lanes (register budget)
-  constexpr int S2 = (OP == FEA_OP_ELASTICITY && PREC == FEA_FP64) ? 2 : 1;
   switch (type) {
     case FEA_TET4:
-      return tet_rule ? launch_tile<FEA_TET4, kRuleTet4, OP, PREC, 1, SC>(P, s)
-                      : launch_tile<FEA_TET4, kRuleTet1, OP, PREC, 1, SC>(P, s);
+      return tet_rule ? launch_tile<FEA_TET4, kRuleTet4, OP, PREC, SC>(P, s)
+                      : launch_tile<FEA_TET4, kRuleTet1, OP, PREC, SC>(P, s);
     case FEA_PYR5:
-      return launch_tile<FEA_PYR5, kRulePyr8, OP, PREC, 1, SC>(P, s);
+      return launch_tile<FEA_PYR5, kRulePyr8, OP, PREC, SC>(P, s);
     case FEA_PRISM6:
-      return launch_tile<FEA_PRISM6, kRulePrism6, OP, PREC, S2, SC>(P, s);
+      return launch_tile<FEA_PRISM6, kRulePrism6, OP, PREC, SC>(P, s);
     default:
-      return launch_tile<FEA_HEX8, kRuleHex8, OP, PREC, S2, SC>(P, s);
+      return launch_tile<FEA_HEX8, kRuleHex8, OP, PREC, SC>(P, s);
   }
 }
 
