@@ -1,5 +1,5 @@
-// fea_api.cu -- the C-ABI entry points: errors, mesh upload (element lists
-// per type, packed connectivity, map offsets), pattern calls, assemble, check.
+// fea_api.cu -- the C-ABI entry points: errors, mesh handles, pattern calls,
+// assemble, check.
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -23,35 +23,12 @@ int cuda_fail(cudaError_t e, const char* what) {
   return FEA_ERR_CUDA;
 }
 
-template <typename T>
-static int dalloc(T** p, size_t count) {
-  *p = nullptr;
-  if (count == 0) count = 1;
-  cudaError_t e = cudaMalloc((void**)p, count * sizeof(T));
-  if (e != cudaSuccess) {
-    *p = nullptr;
-    return fail(FEA_ERR_OOM, std::string("cudaMalloc of ") + std::to_string(count * sizeof(T)) +
-                                 " bytes failed: " + cudaGetErrorString(e));
-  }
-  return FEA_OK;
-}
-
-static void free_mesh(fea_mesh* m) {
+void free_mesh(fea_mesh* m) {
   if (!m) return;
-  cudaFree(m->coords);
-  cudaFree(m->conn_off);
-  cudaFree(m->conn);
-  cudaFree(m->map_off);
-  for (auto& g : m->group) {
-    cudaFree(g.ids);
-    cudaFree(g.conn);
-    cudaFree(g.mapoff);
-  }
-  cudaFree(m->status);
-  cudaFree(m->rp_node);
+  cudaFree(m->arena);
+  cudaFree(m->arena_conn);
+  cudaFree(m->graph);
   cudaFree(m->col_node);
-  cudaFree(m->inc_off);
-  cudaFree(m->inc);
   drop_rows_plans(m);
   cudaFree(m->geo[0]);
   cudaFree(m->geo[1]);
@@ -63,138 +40,6 @@ static void free_mesh(fea_mesh* m) {
     delete m->blocks;
   }
   delete m;
-}
-
-#define FEA_TRY(x)                  \
-  do {                              \
-    int _rc = (x);                  \
-    if (_rc != FEA_OK) {            \
-      free_mesh(m);                 \
-      return _rc;                   \
-    }                               \
-  } while (0)
-
-static int upload_mesh(const fea_mesh_desc* d, cudaStream_t s, fea_mesh** out) {
-  if (!d || !out) return fail(FEA_ERR_ARG, "fea_mesh_upload: null argument");
-  *out = nullptr;
-  if (d->n_nodes <= 0 || d->n_elems <= 0) return fail(FEA_ERR_ARG, "fea_mesh_upload: empty mesh");
-  if (d->n_nodes >= (1ll << 31) || d->n_elems >= (1ll << 31))
-    return fail(FEA_ERR_INDEX_OVERFLOW, "fea_mesh_upload: n_nodes and n_elems must be < 2^31");
-  if (!d->coords || !d->types || !d->conn_offsets || !d->conn)
-    return fail(FEA_ERR_ARG, "fea_mesh_upload: null array");
-  const int64_t N = d->n_nodes, E = d->n_elems;
-
-  // host copies of the element arrays (device input is brought back once)
-  std::vector<uint8_t> types(E);
-  std::vector<int64_t> off(E + 1);
-  const uint8_t* ht = d->types;
-  const int64_t* ho = d->conn_offsets;
-  if (d->on_device) {
-    FEA_CUDA(cudaMemcpyAsync(types.data(), d->types, E, cudaMemcpyDeviceToHost, s));
-    FEA_CUDA(cudaMemcpyAsync(off.data(), d->conn_offsets, (E + 1) * 8, cudaMemcpyDeviceToHost, s));
-    FEA_CUDA(cudaStreamSynchronize(s));
-    ht = types.data();
-    ho = off.data();
-  }
-  if (ho[0] != 0) return fail(FEA_ERR_ARG, "fea_mesh_upload: conn_offsets[0] != 0");
-  int64_t count[kNumTypes] = {0, 0, 0, 0};
-  for (int64_t e = 0; e < E; ++e) {
-    int t = ht[e];
-    if (t >= kNumTypes) return fail(FEA_ERR_ARG, "fea_mesh_upload: unknown element type at element " + std::to_string(e));
-    if (ho[e + 1] - ho[e] != kNodesOf[t])
-      return fail(FEA_ERR_ARG, "fea_mesh_upload: conn_offsets does not match the node count of element " +
-                                   std::to_string(e));
-    count[t]++;
-  }
-  const int64_t L = ho[E];
-  std::vector<int32_t> conn(L);
-  if (d->on_device) {
-    FEA_CUDA(cudaMemcpyAsync(conn.data(), d->conn, L * 4, cudaMemcpyDeviceToHost, s));
-    FEA_CUDA(cudaStreamSynchronize(s));
-  } else {
-    std::memcpy(conn.data(), d->conn, L * 4);
-  }
-  for (int64_t t = 0; t < L; ++t)
-    if (conn[t] < 0 || conn[t] >= N)
-      return fail(FEA_ERR_ARG, "fea_mesh_upload: node id out of range at conn[" + std::to_string(t) + "]");
-
-  fea_mesh* m = new fea_mesh();
-  FEA_CUDA(cudaGetDevice(&m->device));
-  m->n_nodes = N;
-  m->n_elems = E;
-  m->conn_len = L;
-  int ntypes = 0, last = -1;
-  for (int t = 0; t < kNumTypes; ++t)
-    if (count[t]) ++ntypes, last = t;
-  m->uniform = (ntypes == 1);
-  m->uniform_type = m->uniform ? last : -1;
-
-  // map offsets: sum of n_e^2 over preceding elements
-  std::vector<int64_t> moff(E + 1);
-  moff[0] = 0;
-  for (int64_t e = 0; e < E; ++e) moff[e + 1] = moff[e] + (ho[e + 1] - ho[e]) * (ho[e + 1] - ho[e]);
-  m->map_len = moff[E];
-
-  FEA_TRY(dalloc(&m->coords, 3 * N));
-  FEA_TRY(dalloc(&m->conn_off, E + 1));
-  FEA_TRY(dalloc(&m->conn, L));
-  FEA_TRY(dalloc(&m->map_off, E + 1));
-  FEA_TRY(dalloc(&m->status, 1));
-  auto cp = [&](void* dst, const void* src, size_t bytes, bool src_dev) -> int {
-    cudaError_t e = cudaMemcpyAsync(dst, src, bytes, src_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s);
-    return e == cudaSuccess ? FEA_OK : cuda_fail(e, "cudaMemcpyAsync");
-  };
-  FEA_TRY(cp(m->coords, d->coords, 3 * N * 8, d->on_device));
-  FEA_TRY(cp(m->conn_off, ho, (E + 1) * 8, false));
-  FEA_TRY(cp(m->conn, conn.data(), L * 4, false));
-  FEA_TRY(cp(m->map_off, moff.data(), (E + 1) * 8, false));
-  DevStatus zero = {0, 0, ~0ull};
-  FEA_TRY(cp(m->status, &zero, sizeof(zero), false));
-
-  // per-type groups in input order (stable), packed connectivity
-  for (int t = 0; t < kNumTypes; ++t) {
-    TypeGroup& g = m->group[t];
-    g.n = count[t];
-    if (!g.n) continue;
-    const int nn = kNodesOf[t];
-    std::vector<int32_t> ids, pc;
-    std::vector<int64_t> mo;
-    pc.reserve(g.n * nn);
-    if (!m->uniform) {
-      ids.reserve(g.n);
-      mo.reserve(g.n);
-    }
-    for (int64_t e = 0; e < E; ++e) {
-      if (ht[e] != t) continue;
-      for (int a = 0; a < nn; ++a) pc.push_back(conn[ho[e] + a]);
-      if (!m->uniform) {
-        ids.push_back((int32_t)e);
-        mo.push_back(moff[e]);
-      }
-    }
-    FEA_TRY(dalloc(&g.conn, g.n * nn));
-    FEA_TRY(cp(g.conn, pc.data(), g.n * nn * 4, false));
-    if (!m->uniform) {
-      FEA_TRY(dalloc(&g.ids, g.n));
-      FEA_TRY(dalloc(&g.mapoff, g.n));
-      FEA_TRY(cp(g.ids, ids.data(), g.n * 4, false));
-      FEA_TRY(cp(g.mapoff, mo.data(), g.n * 8, false));
-    }
-  }
-  cudaError_t e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) {
-    free_mesh(m);
-    return cuda_fail(e, "cudaStreamSynchronize");
-  }
-  {
-    const int rc = init_rule_constants();  // synchronous copy, so never inside a stream capture
-    if (rc) {
-      free_mesh(m);
-      return rc;
-    }
-  }
-  *out = m;
-  return FEA_OK;
 }
 
 }  // namespace fea

@@ -73,7 +73,7 @@ struct MultidepPlan {
 struct TypeGroup {
   int64_t n = 0;            // elements of this type
   int32_t* ids = nullptr;   // [n] original element ids (nullptr: identity, single-type mesh)
-  int32_t* conn = nullptr;  // [n * nodes_of(t)] packed connectivity, local order
+  int32_t* conn = nullptr;  // [n * nodes_of(t)] packed connectivity, local order (single-type mesh: the mesh's)
   int64_t* mapoff = nullptr;// [n] offset of the element's block in node_map (nullptr: id * nn^2)
 };
 
@@ -87,6 +87,9 @@ struct fea_mesh {
   int64_t map_len = 0;
   bool uniform = false;               // one element type, conn_offsets[e] = e * nn
   int uniform_type = -1;
+  // allocations that hold the arrays below and the groups' lists: sized by
+  // nodes and elements, by connectivity, and the node graph's
+  unsigned char *arena = nullptr, *arena_conn = nullptr, *graph = nullptr;
   double* coords = nullptr;           // [3 n_nodes]
   int64_t* conn_off = nullptr;        // [n_elems + 1]
   int32_t* conn = nullptr;            // [conn_len]
@@ -137,7 +140,12 @@ inline unsigned grid_for(int64_t n, int per_block) {
   return (unsigned)(g < 1 ? 1 : g);
 }
 
+// fea_api.cu, upload.cu
+void free_mesh(fea_mesh* m);
+int upload_mesh(const fea_mesh_desc* d, cudaStream_t s, fea_mesh** out);
+
 // pattern.cu
+void scan_tile_sums(int64_t* tile_sums, int64_t n, cudaStream_t s);  // exclusive, in place, one CTA
 int build_node_graph(fea_mesh* m, cudaStream_t s);
 int write_csr_pattern(fea_mesh* m, int ndof, int64_t* row_ptr, int32_t* col_idx, int32_t* node_map,
                       cudaStream_t s);
