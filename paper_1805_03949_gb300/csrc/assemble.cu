@@ -157,6 +157,14 @@ const RefRule& host_rule(int slot) {
         double N[8], dN[8][3];
         ref_shape(rule_type(s), P[q], N, dN);
         R.w[q] = W[q];
+        if (s == kRulePrism6) {
+          for (int j = 0; j < 3; ++j) R.m[q][j] = P[q][j];
+        } else if (s == kRulePyr8) {  // the point of the base square under the collapsed coordinates
+          R.m[q][0] = P[q][0] / (1.0 - P[q][2]);
+          R.m[q][1] = P[q][1] / (1.0 - P[q][2]);
+          R.m[q][2] = R.m[q][0] * R.m[q][1];
+          R.m[q][3] = P[q][2];
+        }
         R.wf[q] = (float)W[q];
         for (int a = 0; a < 8; ++a) {
           R.N[q][a] = N[a];
@@ -223,18 +231,36 @@ __device__ __forceinline__ void geometry_finish(Smem& sm, const RefRule& rr, int
   geometry_store<OP, NN>(sm, rr, le, q, C, det, s, xq, P);
 }
 
-// FP64 geometry of point q of element le, J from the node coordinates (REL:
-// nodes 1 .. NN-1 hold their differences to node 0 already)
-template <int OP, int NN, bool REL = false, typename Smem>
+// FP64 geometry of point q of element le from the combinations RefMap::prep
+// left in sm.X; with pyramids of point q + 4 too, which shares the Jacobian
+template <int OP, int TYPE, int NN, typename Smem>
 __device__ __forceinline__ void geometry_fp64(Smem& sm, const RefRule& rr, int le, int q, int64_t elem_id,
                                               const AsmParams& P) {
+  using Map = RefMap<TYPE>;
+  double J[3][3], C[3][3];
+  Map::jac(sm.X[le], rr.m[q], J);
+  cofactors(J, C);
+  const double det = J[0][0] * C[0][0] + J[0][1] * C[0][1] + J[0][2] * C[0][2];
+  if (!(det > 0.0)) latch_error(P.st, FEA_ERR_INVERTED_ELEMENT, (unsigned long long)elem_id);
+#pragma unroll 1
+  for (int p = q; p < (TYPE == FEA_PYR5 ? 8 : q + 1); p += 4) {
+    double xq = 0.0;
+    if constexpr (OP == FEA_OP_DIFFUSION) xq = Map::x1(sm.X[le], rr.N[p], rr.m[p]);
+    geometry_store<OP, NN>(sm, rr, le, p, C, det, Map::s, xq, P);
+  }
+}
+
+// FP64 geometry of point q of a distorted hex8 from its node coordinates
+template <int OP, typename Smem>
+__device__ __forceinline__ void geometry_fp64_hex(Smem& sm, const RefRule& rr, int le, int q, int64_t elem_id,
+                                                  const AsmParams& P) {
   double J[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
   double xq = sm.X[le][0][0];
 #pragma unroll
-  for (int a = 1; a < NN; ++a) {
-    const double d0 = REL ? sm.X[le][a][0] : sm.X[le][a][0] - sm.X[le][0][0];
-    const double d1 = REL ? sm.X[le][a][1] : sm.X[le][a][1] - sm.X[le][0][1];
-    const double d2 = REL ? sm.X[le][a][2] : sm.X[le][a][2] - sm.X[le][0][2];
+  for (int a = 1; a < 8; ++a) {
+    const double d0 = sm.X[le][a][0] - sm.X[le][0][0];
+    const double d1 = sm.X[le][a][1] - sm.X[le][0][1];
+    const double d2 = sm.X[le][a][2] - sm.X[le][0][2];
     xq += rr.N[q][a] * d0;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
@@ -243,7 +269,7 @@ __device__ __forceinline__ void geometry_fp64(Smem& sm, const RefRule& rr, int l
       J[2][j] += d2 * rr.dN[q][a][j];
     }
   }
-  geometry_finish<OP, NN>(sm, rr, le, q, elem_id, J, 1.0, xq, P);
+  geometry_finish<OP, 8>(sm, rr, le, q, elem_id, J, 1.0, xq, P);
 }
 
 // FP32 geometry on coordinates relative to node 0; returns false when the
@@ -299,6 +325,7 @@ __device__ __forceinline__ bool geometry_fp32(Smem& sm, const RefRule& rr, int l
 
 template <int TYPE, int SLOT, int OP>
 struct TileCfg {
+  static constexpr int kType = TYPE;
   static constexpr int NN = nodes_of(TYPE);
   static constexpr int NQ = rule_nq(SLOT);
   static constexpr int D = OP == FEA_OP_DIFFUSION ? 1 : 3;
@@ -438,30 +465,31 @@ __device__ __forceinline__ void tile_geometry(typename Cfg::Smem& sm, const RefR
       return;
     }
   }
-  if (all64) {
-    // the differences to node 0 once per element, not once per point
-    for (int t = threadIdx.x; t < EPC * (NN - 1) * 3; t += Cfg::THREADS) {
-      const int le = t / ((NN - 1) * 3), r = t % ((NN - 1) * 3);
-      if (e0 + le < n_end) sm.X[le][1 + r / 3][r % 3] -= sm.X[le][0][r % 3];
-    }
-    __syncthreads();
-  }
-  for (int t = threadIdx.x; t < EPC * NQ; t += Cfg::THREADS) {
-    const int le = t / NQ, q = t % NQ;
-    const int64_t et = e0 + le;
-    if (et >= n_end) continue;
-    if (all64) {
-      geometry_fp64<OP, NN, true>(sm, rr, le, q, original_id(P, et), P);
-    } else {
-      if (!geometry_fp32<OP, NN>(sm, rr, le, q, P)) sm.flag[le] = 1;
-    }
-  }
+  // an FP64 point per thread; pyramids two (geometry_fp64)
+  constexpr int kPoints = Cfg::kType == FEA_PYR5 ? 4 : NQ;
   if (!all64) {
-    __syncthreads();
     for (int t = threadIdx.x; t < EPC * NQ; t += Cfg::THREADS) {
       const int le = t / NQ, q = t % NQ;
-      const int64_t et = e0 + le;
-      if (et < n_end && sm.flag[le]) geometry_fp64<OP, NN>(sm, rr, le, q, original_id(P, et), P);
+      if (e0 + le < n_end && !geometry_fp32<OP, NN>(sm, rr, le, q, P)) sm.flag[le] = 1;
+    }
+    __syncthreads();
+  }
+  // FP64: every element, or the distorted ones
+  if constexpr (kModal) {
+    for (int t = threadIdx.x; t < EPC * NQ; t += Cfg::THREADS) {
+      const int le = t / NQ, q = t % NQ;
+      if (e0 + le < n_end && sm.flag[le]) geometry_fp64_hex<OP>(sm, rr, le, q, original_id(P, e0 + le), P);
+    }
+  } else {
+    for (int t = threadIdx.x; t < EPC * 3; t += Cfg::THREADS) {
+      const int le = t / 3;
+      if (e0 + le < n_end && (all64 || sm.flag[le])) RefMap<Cfg::kType>::prep(sm.X[le], t % 3);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < EPC * kPoints; t += Cfg::THREADS) {
+      const int le = t / kPoints, q = t % kPoints;
+      if (e0 + le < n_end && (all64 || sm.flag[le]))
+        geometry_fp64<OP, Cfg::kType, NN>(sm, rr, le, q, original_id(P, e0 + le), P);
     }
   }
   __syncthreads();

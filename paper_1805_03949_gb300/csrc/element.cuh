@@ -33,6 +33,7 @@ struct RefRule {
   double w[8];
   double N[8][8];       // [q][a]
   double dN[8][8][3];   // [q][a][j] = dN_a / dxi_j
+  double m[8][4];       // [q] parameters of the point for RefMap
   float wf[8];
   float Nf[8][8];
   float dNf[8][8][3];
@@ -194,6 +195,95 @@ __device__ __forceinline__ double hex8_modal_x(const double (*c)[3], int q) {
   }
   return acc;
 }
+
+// ---------------------------------------------------------------------------
+// The maps of the other types from a few combinations of the node values,
+// taken once per element and component, instead of a sum over the nodes with
+// tabulated derivatives at every point.  prep(X, i) replaces component i of an
+// element's node values X [NN][3] (coordinates or any nodal field) by its
+// combinations; jac gives J' = s dx/dxi at a point from them, s a power of
+// two; x1 gives component 0 of the field itself (coordinates: before prep the
+// node values were absolute, the combinations are differences).  FP64
+// instructions per element for J and x at every point: prism 330 -> 117,
+// pyramid 348 -> 142 (one J serves two points), both with 8 or 6 points.
+//  tet4    J's columns are the edges x_{j+1} - x_0
+//  prism6  x = [(1 - z) B + (1 + z) T] / 2 with B, T the bottom and top
+//          triangles: columns 0, 1 are linear in z, column 2 in (r, s)
+//  pyr5    with (x, y, z) = (t xi, t eta, 1 - t) the shape functions are t
+//          times the bilinear ones of the base and z: the columns depend on
+//          (xi, eta) only, so the points q and q + 4 share J
+// ---------------------------------------------------------------------------
+template <int TYPE>
+struct RefMap;
+template <>
+struct RefMap<FEA_TET4> {
+  static constexpr double s = 1.0;
+  static __device__ __forceinline__ void prep(double (*X)[3], int i) {
+#pragma unroll
+    for (int a = 1; a < 4; ++a) X[a][i] -= X[0][i];
+  }
+  static __device__ __forceinline__ void jac(const double (*X)[3], const double*, double (&J)[3][3]) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) J[i][j] = X[j + 1][i];
+  }
+  static __device__ __forceinline__ double x1(const double (*X)[3], const double* N, const double*) {
+    return fma(N[3], X[3][0], fma(N[2], X[2][0], fma(N[1], X[1][0], X[0][0])));
+  }
+};
+template <>
+struct RefMap<FEA_PRISM6> {  // m: r, s, z
+  static constexpr double s = 2.0;
+  static __device__ __forceinline__ void prep(double (*X)[3], int i) {
+    const double x0 = X[0][i], x3 = X[3][i];
+    const double e1 = X[1][i] - x0, e2 = X[2][i] - x0, f1 = X[4][i] - x3, f2 = X[5][i] - x3;
+    X[0][i] = e1 + f1;
+    X[1][i] = e2 + f2;
+    X[2][i] = f1 - e1;
+    X[3][i] = f2 - e2;
+    X[4][i] = x3 - x0;
+    X[5][i] = x0 + x3;
+  }
+  static __device__ __forceinline__ void jac(const double (*X)[3], const double* m, double (&J)[3][3]) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      J[i][0] = fma(m[2], X[2][i], X[0][i]);
+      J[i][1] = fma(m[2], X[3][i], X[1][i]);
+      J[i][2] = fma(m[1], X[3][i], fma(m[0], X[2][i], X[4][i]));
+    }
+  }
+  static __device__ __forceinline__ double x1(const double (*X)[3], const double*, const double* m) {
+    const double c = fma(m[1], X[3][0], fma(m[0], X[2][0], X[4][0]));
+    return 0.5 * fma(m[2], c, fma(m[1], X[1][0], fma(m[0], X[0][0], X[5][0])));
+  }
+};
+template <>
+struct RefMap<FEA_PYR5> {  // m: xi, eta, xi eta, z
+  static constexpr double s = 4.0;
+  static __device__ __forceinline__ void prep(double (*X)[3], int i) {
+    const double x0 = X[0][i], x1 = X[1][i], x2 = X[2][i], x3 = X[3][i];
+    const double p = x1 - x0, q = x2 - x3, r = x3 - x0;
+    const double b = p + q, w = fma(2.0, r, b);  // w: the other base nodes' distances to node 0
+    X[0][i] = b;
+    X[1][i] = (x2 - x1) + r;
+    X[2][i] = q - p;
+    X[3][i] = fma(4.0, X[4][i] - x0, -w);
+    X[4][i] = fma(4.0, x0, w);
+  }
+  static __device__ __forceinline__ void jac(const double (*X)[3], const double* m, double (&J)[3][3]) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      J[i][0] = fma(m[1], X[2][i], X[0][i]);
+      J[i][1] = fma(m[0], X[2][i], X[1][i]);
+      J[i][2] = fma(m[2], X[2][i], X[3][i]);
+    }
+  }
+  static __device__ __forceinline__ double x1(const double (*X)[3], const double*, const double* m) {
+    const double base = fma(m[2], X[2][0], fma(m[1], X[1][0], m[0] * X[0][0]));
+    return 0.25 * fma(1.0 - m[3], base, fma(m[3], X[3][0], X[4][0]));
+  }
+};
 
 // FP64 -> FP32, rounded to nearest even, with integer instructions only
 // (IEEE 754 binary64 to binary32).  On GB300 the hardware conversion issues

@@ -199,24 +199,38 @@ __global__ void __launch_bounds__(kGeoThreads) k_geometry(const __grid_constant_
       return;
     }
   }
-  const bool need64 = valid && q < NQ && (all64 || sFlag[le]);
-  if (need64) {
-    double J[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    double xq = sX[le][0][0];
+  if constexpr (kModal) {
+    // adaptive: distorted hexes, from their node coordinates
+    if (valid && sFlag[le]) {
+      double J[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+      double xq = sX[le][0][0];
 #pragma unroll
-    for (int a = 1; a < NN; ++a) {
-      const double d0 = sX[le][a][0] - sX[le][0][0];
-      const double d1 = sX[le][a][1] - sX[le][0][1];
-      const double d2 = sX[le][a][2] - sX[le][0][2];
-      xq += rr.N[q][a] * d0;
+      for (int a = 1; a < NN; ++a) {
+        const double d0 = sX[le][a][0] - sX[le][0][0];
+        const double d1 = sX[le][a][1] - sX[le][0][1];
+        const double d2 = sX[le][a][2] - sX[le][0][2];
+        xq += rr.N[q][a] * d0;
 #pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        J[0][j] += d0 * rr.dN[q][a][j];
-        J[1][j] += d1 * rr.dN[q][a][j];
-        J[2][j] += d2 * rr.dN[q][a][j];
+        for (int j = 0; j < 3; ++j) {
+          J[0][j] += d0 * rr.dN[q][a][j];
+          J[1][j] += d1 * rr.dN[q][a][j];
+          J[2][j] += d2 * rr.dN[q][a][j];
+        }
       }
+      geo_finish<NN, PREC>(rr, P, q, id, J, 1.0, xq, rec);
     }
-    geo_finish<NN, PREC>(rr, P, q, id, J, 1.0, xq, rec);
+  } else {
+    using Map = RefMap<TYPE>;
+    const bool need64 = valid && (all64 || sFlag[le]);
+    if (need64 && lane8 < 3) Map::prep(sX[le], lane8);
+    __syncwarp();  // an element's 8 threads share a warp
+    if (need64 && q < NQ) {
+      double J[3][3];
+      Map::jac(sX[le], rr.m[q], J);
+      double xq = 0.0;
+      if (P.diffusion) xq = Map::x1(sX[le], rr.N[q], rr.m[q]);
+      geo_finish<NN, PREC>(rr, P, q, id, J, Map::s, xq, rec);
+    }
   }
 }
 

@@ -16,8 +16,8 @@
 //  * diffusion: with c_u(q) = C grad_xi N_u (C the cofactors of J) a pair takes
 //    S_q (c_u . c_v), S_q = w k(x_q) / det J, one division per point and no
 //    scaled gradients (k may have either sign, so it stays out of the root);
-//  * a linear tet has one Jacobian: one set of gradients, with the weights of
-//    its points summed first.
+//  * points that share their gradients (a linear tet's all, a pyramid's in
+//    pairs) make one set of gradients, with their weights summed first.
 // Measured on one GB300, before and after: 250,047 hex8, elasticity 8.82 ->
 // 1.95 ms; 162,000 tet4, elasticity 0.776 -> 0.137 ms; 412,500 mixed elements,
 // diffusion 1.53 -> 0.94 ms.
@@ -59,6 +59,7 @@ __device__ __forceinline__ int64_t original_id(const AsmParams& P, int64_t et) {
 
 template <int TYPE, int SLOT, int OP>
 struct PairCfg {
+  static constexpr int kType = TYPE;
   static constexpr int NN = nodes_of(TYPE);
   static constexpr int NQ = rule_nq(SLOT);
   static constexpr int D = OP == FEA_OP_DIFFUSION ? 1 : 3;
@@ -66,8 +67,10 @@ struct PairCfg {
   static constexpr bool kTet = TYPE == FEA_TET4;
   static constexpr int WARPS = 4;
   static constexpr int THREADS = 32 * WARPS;
-  static constexpr int EPC = kTet ? 32 : (THREADS / NQ) & ~3;  // elements per tile
-  static constexpr int NG = kTet ? 1 : NQ;                     // distinct gradient sets of an element
+  static constexpr int EPC = kTet ? 32 : TYPE == FEA_PYR5 ? 32 : (THREADS / NQ) & ~3;  // elements per tile
+  // points that share their gradients: a linear tet's all, a pyramid's q and q + 4 (RefMap)
+  static constexpr int kShare = kTet ? NQ : TYPE == FEA_PYR5 ? 2 : 1;
+  static constexpr int NG = NQ / kShare;                       // gradient sets of an element: q % NG is point q's
   static constexpr int GS = 3 * NN + 1;                        // odd stride: points spread over the banks
   static constexpr int kOff = NN * (NN - 1) / 2;               // off-diagonal pairs
   static_assert(!kHex || EPC * 8 == THREADS, "the modal transform needs whole warps");
@@ -79,8 +82,8 @@ struct PairCfg {
   struct Smem {
     double X[EPC][NN][3];   // node coordinates (hex8: corners in binary order)
     double G[EPC][NG][GS];  // gradients (see above) [point][node][component]
-    double S[EPC][NG];      // diffusion: w k / det J
-    double W[EPC][kTet ? 1 : NQ];  // w det J (tet4: det J)
+    double S[EPC][NG];      // diffusion: w k / det J, summed over the points that share the set
+    double W[EPC][NG];      // w det J (sets shared by points: det J)
     Node nd[EPC][NN];
     int64_t moff[EPC];      // node_map offset of the element
     uint8_t pair[kOff][2];
@@ -120,32 +123,45 @@ __device__ __forceinline__ void pair_add(double* p, int64_t stride, const double
   }
 }
 
-// The values of point q of element le from the cofactors C' and det' of
-// J' = s J: gradients of every slot, S and W.
+// The values of gradient set q of element le from the cofactors C' and det' of
+// J' = s J: gradients of every slot, S (wk = sum of w k over its points) and W.
 template <class Cfg, int OP>
 __device__ __forceinline__ void pair_point(typename Cfg::Smem& sm, const RefRule& rr, int le, int q,
-                                           const double (&C)[3][3], double det, double s, double kq) {
+                                           const double (&C)[3][3], double det, double s, double wk) {
   double* g = sm.G[le][q];
   double F[3][3];
   if constexpr (OP == FEA_OP_DIFFUSION) {
-    sm.S[le][q] = rr.w[q] * kq / (s * det);
+    sm.S[le][q] = wk / (s * det);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
       for (int j = 0; j < 3; ++j) F[i][j] = C[i][j];
   } else {
-    const double r = sqrt(rr.w[q] / s) * rsqrt(det);
+    double w = rr.w[q];
+#pragma unroll
+    for (int k = 1; k < Cfg::kShare; ++k) w += rr.w[q + k * Cfg::NG];
+    const double r = sqrt(w / s) * rsqrt(det);
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
       for (int j = 0; j < 3; ++j) F[i][j] = C[i][j] * r;
   }
-  sm.W[le][q] = rr.w[q] * det * (1.0 / (s * s * s));
+  sm.W[le][q] = (Cfg::kShare == 1 ? rr.w[q] : 1.0) * det * (1.0 / (s * s * s));
+  if constexpr (Cfg::kTet) {
+    // J^{-T} grad_xi N_{j+1} is column j of C / det J; the gradients sum to zero
 #pragma unroll
-  for (int u = 0; u < Cfg::NN; ++u) {
-    const double* d = rr.dN[q][Cfg::kHex ? hex8_corner_node(u) : u];
+    for (int i = 0; i < 3; ++i) {
 #pragma unroll
-    for (int i = 0; i < 3; ++i) g[3 * u + i] = fma(d[2], F[i][2], fma(d[1], F[i][1], d[0] * F[i][0]));
+      for (int j = 0; j < 3; ++j) g[3 * (j + 1) + i] = F[i][j];
+      g[i] = -(F[i][0] + F[i][1] + F[i][2]);
+    }
+  } else {
+#pragma unroll
+    for (int u = 0; u < Cfg::NN; ++u) {
+      const double* d = rr.dN[q][Cfg::kHex ? hex8_corner_node(u) : u];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) g[3 * u + i] = fma(d[2], F[i][2], fma(d[1], F[i][1], d[0] * F[i][0]));
+    }
   }
 }
 
@@ -153,7 +169,8 @@ __device__ __forceinline__ void pair_point(typename Cfg::Smem& sm, const RefRule
 template <class Cfg, int OP, class Params>
 __device__ __forceinline__ void pair_geometry(typename Cfg::Smem& sm, const RefRule& rr, const Params& P, int64_t e0,
                                               int64_t n_end) {
-  constexpr int NN = Cfg::NN, NQ = Cfg::NQ, EPC = Cfg::EPC, D = Cfg::D;
+  constexpr int TYPE = Cfg::kType, NN = Cfg::NN, NG = Cfg::NG, EPC = Cfg::EPC, D = Cfg::D;
+  static_assert(EPC * 3 <= Cfg::THREADS, "a thread per element and component");
   for (int p = threadIdx.x; p < Cfg::kOff; p += Cfg::THREADS) {
     int u = 0, r = p;
     while (r >= NN - 1 - u) r -= NN - 1 - u++;
@@ -196,71 +213,29 @@ __device__ __forceinline__ void pair_geometry(typename Cfg::Smem& sm, const RefR
         const double x = hex8_modal_x(sm.X[le], p);
         kq = P.k0 + P.k2 * x * x;
       }
-      pair_point<Cfg, OP>(sm, rr, le, p, C, det, 8.0, kq);
-    }
-  } else if constexpr (Cfg::kTet) {
-    if (t < EPC && e0 + t < n_end) {
-      const double(&X)[NN][3] = sm.X[t];
-      // column j of J is the edge x_{j+1} - x_0, and J^{-T} grad_xi N_{j+1} is
-      // column j of C / det J; the gradients sum to zero
-      double J[3][3], C[3][3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) J[i][j] = X[j + 1][i] - X[0][i];
-      cofactors(J, C);
-      const double det = J[0][0] * C[0][0] + J[0][1] * C[0][1] + J[0][2] * C[0][2];
-      if (!(det > 0.0)) latch_error(P.st, FEA_ERR_INVERTED_ELEMENT, (unsigned long long)original_id(P, e0 + t));
-      double r = 1.0;
-      if constexpr (OP == FEA_OP_DIFFUSION) {
-        double wk = 0.0;
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-          double x = X[0][0];
-#pragma unroll
-          for (int a = 1; a < NN; ++a) x = fma(rr.N[q][a], J[0][a - 1], x);
-          wk = fma(rr.w[q], P.k0 + P.k2 * x * x, wk);
-        }
-        sm.S[t][0] = wk / det;
-      } else {
-        double w = 0.0;
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) w += rr.w[q];
-        r = sqrt(w) * rsqrt(det);
-      }
-      sm.W[t][0] = det;
-      double* g = sm.G[t][0];
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const double a = C[i][0] * r, b = C[i][1] * r, c = C[i][2] * r;
-        g[3 + i] = a;
-        g[6 + i] = b;
-        g[9 + i] = c;
-        g[i] = -(a + b + c);
-      }
+      pair_point<Cfg, OP>(sm, rr, le, p, C, det, 8.0, rr.w[p] * kq);
     }
   } else {
-    const int le = t / NQ, q = t % NQ;
-    if (t < EPC * NQ && e0 + le < n_end) {
-      const double(&X)[NN][3] = sm.X[le];
-      double J[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}}, C[3][3], x = X[0][0];
-#pragma unroll
-      for (int a = 1; a < NN; ++a) {
-        double d[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) d[i] = X[a][i] - X[0][i];
-        if constexpr (OP == FEA_OP_DIFFUSION) x = fma(rr.N[q][a], d[0], x);
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-          for (int j = 0; j < 3; ++j) J[i][j] = fma(d[i], rr.dN[q][a][j], J[i][j]);
-      }
+    using Map = RefMap<TYPE>;
+    if (t < EPC * 3 && e0 + t / 3 < n_end) Map::prep(sm.X[t / 3], t % 3);
+    __syncthreads();
+    const int le = t / NG, q = t % NG;
+    if (t < EPC * NG && e0 + le < n_end) {
+      double J[3][3], C[3][3];
+      Map::jac(sm.X[le], rr.m[q], J);
       cofactors(J, C);
       const double det = J[0][0] * C[0][0] + J[0][1] * C[0][1] + J[0][2] * C[0][2];
       if (!(det > 0.0)) latch_error(P.st, FEA_ERR_INVERTED_ELEMENT, (unsigned long long)original_id(P, e0 + le));
-      double kq = 0.0;
-      if constexpr (OP == FEA_OP_DIFFUSION) kq = P.k0 + P.k2 * x * x;
-      pair_point<Cfg, OP>(sm, rr, le, q, C, det, 1.0, kq);
+      double wk = 0.0;
+      if constexpr (OP == FEA_OP_DIFFUSION) {
+#pragma unroll
+        for (int k = 0; k < Cfg::kShare; ++k) {
+          const int p = q + k * NG;
+          const double x = Map::x1(sm.X[le], rr.N[p], rr.m[p]);
+          wk = fma(rr.w[p], P.k0 + P.k2 * x * x, wk);
+        }
+      }
+      pair_point<Cfg, OP>(sm, rr, le, q, C, det, Map::s, wk);
     }
   }
   __syncthreads();
@@ -272,9 +247,16 @@ __device__ __forceinline__ double pair_beta(const typename Cfg::Smem& sm, const 
   const int a = Cfg::node_of(u);
   double s = 0.0;
 #pragma unroll
-  for (int q = 0; q < Cfg::NQ; ++q)
-    s = Cfg::kTet ? fma(rr.w[q], rr.N[q][a], s) : fma(sm.W[le][Cfg::kTet ? 0 : q], rr.N[q][a], s);
-  return Cfg::kTet ? s * sm.W[le][0] : s;
+  for (int g = 0; g < Cfg::NG; ++g) {
+    double n = rr.N[g][a];
+    if constexpr (Cfg::kShare > 1) {
+      n *= rr.w[g];
+#pragma unroll
+      for (int k = 1; k < Cfg::kShare; ++k) n = fma(rr.w[g + k * Cfg::NG], rr.N[g + k * Cfg::NG][a], n);
+    }
+    s = fma(sm.W[le][g], n, s);
+  }
+  return s;
 }
 
 // One task: the entry block of the nodes in slots u and v of element le, into
