@@ -19,28 +19,34 @@
 // in the tile precision (FP32 for FEA_FP32_INTEGRATE: the return map and D_ep
 // stay FP64, the D_ep B products are FP32; FP64 otherwise), accumulated into
 // A and b in FP64 by atomics (ATOMIC) or plain read-modify-writes (COLOR).
+//
+// The Gauss-point update is bound by the number of its FP64 instructions (a
+// warp instruction holds the SM's FP64 unit for 16 cycles; ncu of the element
+// loop: unit 87 % busy, issue slots 12 %), so:
+//  * the displacement gradient of every type is Ju C^T / det from the
+//    displacement field's reference Jacobian Ju (RefMap, or the modal
+//    transform), only its symmetric part is formed, and the committed plastic
+//    strain is subtracted in the same FMAs;
+//  * a point clearly inside the yield surface is told by the squared norm: no
+//    square root (a point near the surface takes the root and the same test
+//    as a yielding one, so ties fall as before);
+//  * reciprocals of det J, of the Newton slope and of the norm are rcp64, and
+//    constant divisors are the host's factors;
+//  * the element loop forms no tile factors (they go nowhere there).
+// 499,200 hex8, element loop, one GB300: 2.24 -> 1.63 ms; 373,248 hex8, FP32
+// assembly: 2.20 -> 1.96 ms.
 #include <cmath>
 #include <cstring>
 #include <type_traits>
 
 #include "element.cuh"
 #include "fea_internal.cuh"
+#include "pairs.cuh"
 #include "sched.cuh"
 
 namespace fea {
 
-struct J2Params {
-  const double* coords;
-  const int32_t* tconn;   // [n][NN] packed connectivity of the type group
-  const int32_t* ids;     // group index -> original id (nullptr: identity)
-  const int64_t* mapoff;  // group index -> node_map offset (nullptr: id * NN^2)
-  const int32_t* list;    // launch index -> group index (nullptr: identity; coloring)
-  int64_t n;
-  const int64_t* row_ptr;
-  const int32_t* node_map;
-  double* A;
-  double* b;
-  DevStatus* st;
+struct J2Params : ElemParams {
   const double* u;
   const double* state_in;
   double* state_out;
@@ -49,55 +55,55 @@ struct J2Params {
   double* stress_out;     // element loop: [E][8][6] Cauchy stress per point slot (may be nullptr)
   double lam, mu, kappa;
   double s0, sinf, delta, hard, tol_g, tol_step;
-  double mu2_3;           // 2 mu / 3: the factor 2 mu theta / 3 of an elastic point (theta = 1)
+  double mu2, mu2_3;      // 2 mu, 2 mu / 3
+  double gp0, gp1;        // dg/d(dgamma) = gp0 + gp1 exp(-delta a)
+  double inv3mu;          // 1 / (3 mu)
   int max_iter;
 };
 
-template <int TYPE, int SLOT, int PREC, int SPLIT>
+// FP32 tiles: lane a of an element's NN lanes holds its row block.
+template <int TYPE, int SLOT>
 struct J2Cfg {
+  static constexpr int kType = TYPE;
   static constexpr int NN = nodes_of(TYPE);
   static constexpr int NQ = rule_nq(SLOT);
-  static constexpr int LPE = NN * SPLIT;
+  static constexpr int LPE = NN;
   static constexpr int EPW = 32 / LPE;
   static constexpr int WARPS = 4;
   static constexpr int THREADS = 32 * WARPS;
   static constexpr int EPC = EPW * WARPS;
-  static constexpr int NB = NN / SPLIT;
-  static constexpr bool kModal = TYPE == FEA_HEX8 && SLOT == kRuleHex8;
-  static_assert(NN % SPLIT == 0, "SPLIT must divide the node count");
-  static_assert(!kModal || (EPC * 8 % 32 == 0 && EPC * 8 <= THREADS), "modal hex geometry needs whole warps");
-  using R = typename std::conditional<PREC == FEA_FP64, double, float>::type;
-  struct Smem {
+  static constexpr int NB = NN;
+  static constexpr bool kHex = TYPE == FEA_HEX8;
+  static_assert(!kHex || (EPC * 8 % 32 == 0 && EPC * 8 <= THREADS), "modal hex geometry needs whole warps");
+  // what the Gauss-point update of the element loop needs
+  struct Fields {
     double X[EPC][NN][3];
     double U[EPC][NN][3];
-    R G[EPC][NQ][NN][3];  // grad N_a
-    R H[EPC][NQ][NN][3];  // h_a = n grad N_a
-    R C[EPC][NQ][4];      // W, W lam', W mu', W beta
-    R S[EPC][NQ][6];      // W sigma (xx, yy, zz, xy, yz, xz)
+  };
+  struct Smem : Fields {
+    float G[EPC][NQ][NN][3];  // grad N_a
+    float H[EPC][NQ][NN][3];  // h_a = n grad N_a
+    float C[EPC][NQ][4];      // W, W lam', W mu', W beta
+    float S[EPC][NQ][6];      // W sigma (xx, yy, zz, xy, yz, xz)
   };
 };
 
-__device__ __forceinline__ int64_t j2_group_index(const J2Params& P, int64_t et) {
-  return P.list ? (int64_t)P.list[et] : et;
-}
-
-// Radial return at one point (all FP64).  eps, eps_p_n: tensor components.
+// Radial return at one point (all FP64): trial strain e = eps - eps_p_n.
 struct J2Point {
   double sig[6], n[6], ep[6];
   double theta, theta_bar, alpha;
   int iters, yielded, ok;
 };
 
-__device__ __forceinline__ void j2_return(const J2Params& P, const double eps[6], const double epn[6], double an,
+__device__ __forceinline__ void j2_return(const J2Params& P, const double e[6], const double epn[6], double an,
                                           J2Point& r) {
   const double r23 = 0.81649658092772603273;  // sqrt(2/3)
-  double e[6], s[6];
-#pragma unroll
-  for (int i = 0; i < 6; ++i) e[i] = eps[i] - epn[i];
   const double tr = e[0] + e[1] + e[2];
+  const double m = -P.mu2_3 * tr;  // the volumetric part of 2 mu e
+  double s[6];
 #pragma unroll
-  for (int i = 0; i < 6; ++i) s[i] = 2.0 * P.mu * (e[i] - (i < 3 ? tr / 3.0 : 0.0));
-  const double norm = sqrt(s[0] * s[0] + s[1] * s[1] + s[2] * s[2] + 2.0 * (s[3] * s[3] + s[4] * s[4] + s[5] * s[5]));
+  for (int i = 0; i < 6; ++i) s[i] = i < 3 ? fma(P.mu2, e[i], m) : P.mu2 * e[i];
+  const double n2 = fma(2.0, fma(s[5], s[5], fma(s[4], s[4], s[3] * s[3])), fma(s[2], s[2], fma(s[1], s[1], s[0] * s[0])));
   const double dsy = P.sinf - P.s0;
   // sigma_y(alpha_n); at alpha_n = 0 (a point that never yielded) it is s0
   // exactly, and the exp is not taken
@@ -107,21 +113,28 @@ __device__ __forceinline__ void j2_return(const J2Params& P, const double eps[6]
   r.theta_bar = 0.0;
   r.iters = 0;
   r.ok = 1;
+  r.yielded = 0;
+  r.alpha = an;
 #pragma unroll
   for (int i = 0; i < 6; ++i) r.n[i] = 0.0;
-  if (norm - r23 * sy_n <= 0.0) {
 #pragma unroll
-    for (int i = 0; i < 6; ++i) r.ep[i] = epn[i];
-    r.alpha = an;
-    r.yielded = 0;
-  } else {
+  for (int i = 0; i < 6; ++i) r.ep[i] = epn[i];
+  const double thr = r23 * sy_n;
+  double norm = 0.0;
+  // clearly elastic (thr > 0 and the norm below it by more than rounding): no root
+  bool plastic = !(thr > 0.0 && n2 < 0.999999 * (thr * thr));
+  if (plastic) {
+    norm = sqrt(n2);
+    plastic = !(norm - thr <= 0.0);
+  }
+  if (plastic) {
     double dg = 0.0, ex = 1.0;
     int it = 0, ok = 0;
     bool ex_final = false;  // ex belongs to the final dg (no step after it)
     for (;;) {
-      const double a = an + r23 * dg;
+      const double a = fma(r23, dg, an);
       ex = exp(-P.delta * a);
-      const double g = norm - 2.0 * P.mu * dg - r23 * (P.s0 + P.hard * a + dsy * (1.0 - ex));
+      const double g = norm - P.mu2 * dg - r23 * (P.s0 + P.hard * a + dsy * (1.0 - ex));
       if (fabs(g) <= P.tol_g * sy_n) {
         ok = 1;
         ex_final = true;
@@ -131,8 +144,7 @@ __device__ __forceinline__ void j2_return(const J2Params& P, const double eps[6]
         ex_final = true;
         break;
       }
-      const double gp = -2.0 * P.mu - (2.0 / 3.0) * (P.hard + dsy * P.delta * ex);
-      const double step = -g / gp;
+      const double step = -g * rcp64(fma(P.gp1, ex, P.gp0));
       dg += step;
       ++it;
       if (fabs(step) <= P.tol_step) {
@@ -142,97 +154,34 @@ __device__ __forceinline__ void j2_return(const J2Params& P, const double eps[6]
     }
     r.iters = it;
     r.ok = ok;
-    const double a = an + r23 * dg;
+    const double a = fma(r23, dg, an);
     // exp(-delta a) at the final dg: the loop's last value when it stopped at
     // the residual test or the iteration limit (the same a), else a new one
     const double slope = P.hard + dsy * P.delta * (ex_final ? ex : exp(-P.delta * a));
-    const double inv = 1.0 / norm;
+    const double inv = rcp64(norm);
 #pragma unroll
     for (int i = 0; i < 6; ++i) r.n[i] = s[i] * inv;
-    r.theta = 1.0 - 2.0 * P.mu * dg * inv;
-    r.theta_bar = 1.0 / (1.0 + slope / (3.0 * P.mu)) - (1.0 - r.theta);
+    r.theta = fma(-P.mu2 * dg, inv, 1.0);
+    r.theta_bar = rcp64(fma(slope, P.inv3mu, 1.0)) - (1.0 - r.theta);
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-      s[i] -= 2.0 * P.mu * dg * r.n[i];
-      r.ep[i] = epn[i] + dg * r.n[i];
+      s[i] *= r.theta;
+      r.ep[i] = fma(dg, r.n[i], epn[i]);
     }
     r.alpha = a;
     r.yielded = 1;
   }
+  const double p = P.kappa * tr;
 #pragma unroll
-  for (int i = 0; i < 6; ++i) r.sig[i] = s[i] + (i < 3 ? P.kappa * tr : 0.0);
+  for (int i = 0; i < 6; ++i) r.sig[i] = i < 3 ? s[i] + p : s[i];
 }
 
-// Phase 1 of point q of element le: FP64 geometry, strain and return map;
-// writes the per-point factors of the tile precision into shared memory.
-// J' = s J is the reference Jacobian scaled by a power of two.  MODAL (hex8,
-// FP32 tiles): Ju' = s Ju is the displacement field's reference Jacobian from
-// the modal transform of the nodal displacements, and the displacement
-// gradient is Ju J^-1 = Ju' C'^T / det' in FP64 (27 + 9 operations), so the
-// shape-function gradients are only needed in the tile precision: formed in
-// FP32 from C' and det' rounded once each, as the elasticity tile forms them.
-template <class Cfg, bool MODAL = false>
-__device__ __forceinline__ void j2_point(typename Cfg::Smem& sm, const RefRule& rr, const J2Params& P, int le, int q,
-                                         int64_t et, double (&J)[3][3], double s, const double (*Ju)[3] = nullptr) {
-  using R = typename Cfg::R;
-  constexpr int NN = Cfg::NN;
-  const int64_t g = j2_group_index(P, et);
-  const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
-  double C[3][3];
-  cofactors(J, C);
-  const double det = J[0][0] * C[0][0] + J[0][1] * C[0][1] + J[0][2] * C[0][2];
-  if (!(det > 0.0)) {
-    latch_error(P.st, FEA_ERR_INVERTED_ELEMENT, (unsigned long long)id);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) sm.C[le][q][k] = R(0);
-#pragma unroll
-    for (int k = 0; k < 6; ++k) sm.S[le][q][k] = R(0);
-#pragma unroll
-    for (int a = 0; a < NN; ++a)
-#pragma unroll
-      for (int i = 0; i < 3; ++i) sm.G[le][q][a][i] = sm.H[le][q][a][i] = R(0);
-    return;
-  }
-  // the displacement gradient H_ij = sum_a u_a,i g_a,j (FP64) and the
-  // gradients g_a in the tile precision
-  double Hu[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-  R gt[NN][3];
-  if constexpr (MODAL) {
-    static_assert(!std::is_same<R, double>::value, "the modal strain path forms FP32 gradients");
-    const double rdet = 1.0 / det;
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) Hu[i][j] = (Ju[i][0] * C[j][0] + Ju[i][1] * C[j][1] + Ju[i][2] * C[j][2]) * rdet;
-    float Cf[3][3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) Cf[i][j] = f64_to_f32_rn(C[i][j]);
-    const float invf = (float)s / f64_to_f32_rn(det);
-#pragma unroll
-    for (int a = 0; a < NN; ++a)
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-        gt[a][i] = (rr.dNf[q][a][0] * Cf[i][0] + rr.dNf[q][a][1] * Cf[i][1] + rr.dNf[q][a][2] * Cf[i][2]) * invf;
-  } else {
-    const double inv = s / det;
-#pragma unroll
-    for (int a = 0; a < NN; ++a) {
-      double gd[3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-        gd[i] = (rr.dN[q][a][0] * C[i][0] + rr.dN[q][a][1] * C[i][1] + rr.dN[q][a][2] * C[i][2]) * inv;
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Hu[i][j] = fma(sm.U[le][a][i], gd[j], Hu[i][j]);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) gt[a][i] = to_tile<R>(gd[i]);
-    }
-  }
-  const double eps[6] = {Hu[0][0], Hu[1][1], Hu[2][2], 0.5 * (Hu[0][1] + Hu[1][0]), 0.5 * (Hu[1][2] + Hu[2][1]),
-                         0.5 * (Hu[0][2] + Hu[2][0])};
+// The Gauss-point update of point q of the element with original id `id`:
+// strain from the displacement field's reference Jacobian Ju' = s Ju and the
+// cofactors C' and determinant of J' = s J, return map from the committed
+// state, and its results to the state, flag and stress arrays.
+__device__ __forceinline__ void j2_update(const J2Params& P, int64_t id, int q, const double (&C)[3][3], double rdet,
+                                          const double (&Ju)[3][3], J2Point& r) {
   double epn[6] = {0, 0, 0, 0, 0, 0}, an = 0.0;
   const int64_t slot = id * 8 + q;
   if (P.state_in) {
@@ -241,8 +190,16 @@ __device__ __forceinline__ void j2_point(typename Cfg::Smem& sm, const RefRule& 
     for (int i = 0; i < 6; ++i) epn[i] = sp[i];
     an = sp[6];
   }
-  J2Point r;
-  j2_return(P, eps, epn, an, r);
+  // e = sym(Ju' C'^T) / det' - eps_p_n: the displacement gradient is Ju J^-1
+  double e[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const int i = k < 3 ? k : k == 4 ? 1 : 0, j = k < 3 ? k : k == 3 ? 1 : 2;
+    double h = fma(Ju[i][2], C[j][2], fma(Ju[i][1], C[j][1], Ju[i][0] * C[j][0]));
+    if (k >= 3) h = fma(Ju[j][2], C[i][2], fma(Ju[j][1], C[i][1], fma(Ju[j][0], C[i][0], h)));
+    e[k] = fma(h, k < 3 ? rdet : 0.5 * rdet, -epn[k]);
+  }
+  j2_return(P, e, epn, an, r);
   if (!r.ok) latch_error(P.st, FEA_ERR_NO_CONVERGENCE, (unsigned long long)id);
   if (P.state_out) {
     double* sp = P.state_out + slot * 7;
@@ -256,46 +213,108 @@ __device__ __forceinline__ void j2_point(typename Cfg::Smem& sm, const RefRule& 
 #pragma unroll
     for (int i = 0; i < 6; ++i) P.stress_out[slot * 6 + i] = r.sig[i];
   }
-  const double W = rr.w[q] * det * (1.0 / (s * s * s));
-  sm.C[le][q][0] = to_tile<R>(W);
-  // 2 mu theta / 3, from the host's 2 mu / 3 at an elastic point (the same
-  // value: theta = 1 there), so that point takes no FP64 division
-  const double mu2t_3 = r.yielded ? 2.0 * P.mu * r.theta / 3.0 : P.mu2_3;
-  sm.C[le][q][1] = to_tile<R>(W * (P.kappa - mu2t_3));
-  sm.C[le][q][2] = to_tile<R>(W * P.mu * r.theta);
-  sm.C[le][q][3] = to_tile<R>(W * 2.0 * P.mu * r.theta_bar);
+}
+
+// Cofactors and determinant of J' at point q; det' <= 0 latches the element.
+__device__ __forceinline__ bool j2_jacobian(const J2Params& P, int64_t id, const double (&J)[3][3], double (&C)[3][3],
+                                            double* det) {
+  cofactors(J, C);
+  *det = J[0][0] * C[0][0] + J[0][1] * C[0][1] + J[0][2] * C[0][2];
+  if (*det > 0.0) return true;
+  latch_error(P.st, FEA_ERR_INVERTED_ELEMENT, (unsigned long long)id);
+  return false;
+}
+
+// Phase 1 of point q of element le of an FP32 tile: the update, then
+// (SCATTER) the point's factors in FP32 into shared memory.  Hex gradients are
+// formed in FP32 from C' and det' rounded once each, as the elasticity tile
+// forms them; the other types' in FP64 and rounded.
+template <class Cfg, bool SCATTER, class Smem>
+__device__ __forceinline__ void j2_point(Smem& sm, const RefRule& rr, const J2Params& P, int le, int q, int64_t et,
+                                         const double (&J)[3][3], const double (&Ju)[3][3], double s) {
+  constexpr int NN = Cfg::NN;
+  const int64_t id = original_id(P, et);
+  double C[3][3], det;
+  const bool ok = j2_jacobian(P, id, J, C, &det);
+  if (!ok) {
+    if constexpr (SCATTER) {
 #pragma unroll
-  for (int k = 0; k < 6; ++k) sm.S[le][q][k] = to_tile<R>(W * r.sig[k]);
-  // h_a = n g_a in the tile precision (n = 0 at elastic points)
-  const R n0 = to_tile<R>(r.n[0]), n1 = to_tile<R>(r.n[1]), n2 = to_tile<R>(r.n[2]), n3 = to_tile<R>(r.n[3]),
-          n4 = to_tile<R>(r.n[4]), n5 = to_tile<R>(r.n[5]);
+      for (int k = 0; k < 4; ++k) sm.C[le][q][k] = 0.0f;
 #pragma unroll
-  for (int a = 0; a < NN; ++a) {
-    const R g0 = gt[a][0], g1 = gt[a][1], g2 = gt[a][2];
-    sm.G[le][q][a][0] = g0;
-    sm.G[le][q][a][1] = g1;
-    sm.G[le][q][a][2] = g2;
-    sm.H[le][q][a][0] = n0 * g0 + n3 * g1 + n5 * g2;
-    sm.H[le][q][a][1] = n3 * g0 + n1 * g1 + n4 * g2;
-    sm.H[le][q][a][2] = n5 * g0 + n4 * g1 + n2 * g2;
+      for (int k = 0; k < 6; ++k) sm.S[le][q][k] = 0.0f;
+#pragma unroll
+      for (int a = 0; a < NN; ++a)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) sm.G[le][q][a][i] = sm.H[le][q][a][i] = 0.0f;
+    }
+    return;
+  }
+  J2Point r;
+  const double rdet = rcp64(det);
+  j2_update(P, id, q, C, rdet, Ju, r);
+  if constexpr (SCATTER) {
+    const double W = rr.w[q] * det * (1.0 / (s * s * s));
+    sm.C[le][q][0] = f64_to_f32_rn(W);
+    sm.C[le][q][1] = f64_to_f32_rn(W * (P.kappa - (r.yielded ? P.mu2_3 * r.theta : P.mu2_3)));
+    sm.C[le][q][2] = f64_to_f32_rn(W * P.mu * r.theta);
+    sm.C[le][q][3] = r.yielded ? f64_to_f32_rn(W * P.mu2 * r.theta_bar) : 0.0f;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) sm.S[le][q][k] = f64_to_f32_rn(W * r.sig[k]);
+    float gt[NN][3];
+    if constexpr (Cfg::kHex) {
+      float Cf[3][3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) Cf[i][j] = f64_to_f32_rn(C[i][j]);
+      const float invf = (float)s / f64_to_f32_rn(det);
+#pragma unroll
+      for (int a = 0; a < NN; ++a)
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+          gt[a][i] = (rr.dNf[q][a][0] * Cf[i][0] + rr.dNf[q][a][1] * Cf[i][1] + rr.dNf[q][a][2] * Cf[i][2]) * invf;
+    } else {
+      const double inv = s * rdet;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const double c0 = C[i][0] * inv, c1 = C[i][1] * inv, c2 = C[i][2] * inv;
+#pragma unroll
+        for (int a = 0; a < NN; ++a)
+          gt[a][i] = f64_to_f32_rn(fma(rr.dN[q][a][2], c2, fma(rr.dN[q][a][1], c1, rr.dN[q][a][0] * c0)));
+      }
+    }
+    // h_a = n g_a (n = 0 at elastic points)
+    float n[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) n[k] = r.yielded ? f64_to_f32_rn(r.n[k]) : 0.0f;
+#pragma unroll
+    for (int a = 0; a < NN; ++a) {
+      const float g0 = gt[a][0], g1 = gt[a][1], g2 = gt[a][2];
+      sm.G[le][q][a][0] = g0;
+      sm.G[le][q][a][1] = g1;
+      sm.G[le][q][a][2] = g2;
+      sm.H[le][q][a][0] = n[0] * g0 + n[3] * g1 + n[5] * g2;
+      sm.H[le][q][a][1] = n[3] * g0 + n[1] * g1 + n[4] * g2;
+      sm.H[le][q][a][2] = n[5] * g0 + n[4] * g1 + n[2] * g2;
+    }
   }
 }
 
-// One tile of EPC elements from launch index e0 (elements at or past n_end
-// are skipped).  Every thread of the CTA calls it; it ends with a barrier.
-// SCATTER = false is the element-wise loop: the Gauss-point update only.
-template <int TYPE, int SLOT, int PREC, int SPLIT, int SC, bool SCATTER = true>
-__device__ __forceinline__ void j2_tile_body(typename J2Cfg<TYPE, SLOT, PREC, SPLIT>::Smem& sm, const RefRule& rr,
-                                             const J2Params& P, int64_t e0, int64_t n_end) {
-  using Cfg = J2Cfg<TYPE, SLOT, PREC, SPLIT>;
-  using R = typename Cfg::R;
+// One FP32 tile of EPC elements from launch index e0 (elements at or past
+// n_end are skipped).  Every thread of the CTA calls it; it ends with a
+// barrier.  SCATTER = false is the element-wise loop: the Gauss-point update
+// only.
+template <int TYPE, int SLOT, int SC, bool SCATTER, class Smem>
+__device__ __forceinline__ void j2_tile_body(Smem& sm, const RefRule& rr, const J2Params& P, int64_t e0,
+                                             int64_t n_end) {
+  using Cfg = J2Cfg<TYPE, SLOT>;
   constexpr int NN = Cfg::NN, NQ = Cfg::NQ, EPC = Cfg::EPC, NB = Cfg::NB, LPE = Cfg::LPE, EPW = Cfg::EPW;
   // phase 0: coordinates and displacements of the tile's nodes
   for (int t = threadIdx.x; t < EPC * NN; t += Cfg::THREADS) {
     const int le = t / NN, a = t % NN;
     const int64_t et = e0 + le;
     if (et < n_end) {
-      const int64_t node = P.tconn[j2_group_index(P, et) * NN + a];
+      const int64_t node = P.tconn[group_index(P, et) * NN + a];
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
         sm.X[le][a][i] = P.coords[3 * node + i];
@@ -305,179 +324,259 @@ __device__ __forceinline__ void j2_tile_body(typename J2Cfg<TYPE, SLOT, PREC, SP
   }
   __syncthreads();
   // phase 1: one thread per (element, point)
-  if constexpr (Cfg::kModal) {
-    const int t = threadIdx.x;
-    if (t < EPC * 8) {
-      const int le = t >> 3, p = t & 7;
-      const int64_t et = e0 + le;
-      const bool valid = et < n_end;
-      const int a = hex8_corner_node(p);
-      // FP32 tiles take the displacements to modal form as well (the strain
-      // then needs no FP64 gradients); sm.U holds modal coefficients after
-      constexpr bool kModalU = PREC != FEA_FP64;
-      double v[3], vu[3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        v[i] = valid ? sm.X[le][a][i] : 0.0;
-        vu[i] = valid ? sm.U[le][a][i] : 0.0;
-      }
-      hex8_modal(v);
-      if constexpr (kModalU) hex8_modal(vu);
-      __syncwarp();
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        sm.X[le][p][i] = v[i];
-        if constexpr (kModalU) sm.U[le][p][i] = vu[i];
-      }
-      __syncwarp();
-      // every lane forms its Jacobians (the lanes of an element exchange
-      // columns); the valid ones use them
-      double J[3][3], Ju[3][3];
-      hex8_jacobian_pairs(sm.X[le], p, J);
-      if constexpr (kModalU) hex8_jacobian_pairs(sm.U[le], p, Ju);
-      if (valid) {
-        if constexpr (kModalU)
-          j2_point<Cfg, true>(sm, rr, P, le, p, et, J, 8.0, Ju);
-        else
-          j2_point<Cfg>(sm, rr, P, le, p, et, J, 8.0);
-      }
-    }
-  } else {
-    for (int t = threadIdx.x; t < EPC * NQ; t += Cfg::THREADS) {
-      const int le = t / NQ, q = t % NQ;
-      const int64_t et = e0 + le;
-      if (et >= n_end) continue;
-      double J[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-#pragma unroll
-      for (int a = 1; a < NN; ++a) {
-        const double d0 = sm.X[le][a][0] - sm.X[le][0][0];
-        const double d1 = sm.X[le][a][1] - sm.X[le][0][1];
-        const double d2 = sm.X[le][a][2] - sm.X[le][0][2];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          J[0][j] += d0 * rr.dN[q][a][j];
-          J[1][j] += d1 * rr.dN[q][a][j];
-          J[2][j] += d2 * rr.dN[q][a][j];
-        }
-      }
-      j2_point<Cfg>(sm, rr, P, le, q, et, J, 1.0);
-    }
-  }
+  field_points<TYPE, NQ, EPC, Cfg::THREADS>(
+      sm, rr, e0, n_end, [](int p) { return hex8_corner_node(p); },
+      [&](int le, int q, int64_t et, const double(&J)[3][3], const double(&Ju)[3][3], double s) {
+        j2_point<Cfg, SCATTER>(sm, rr, P, le, q, et, J, Ju, s);
+      });
   __syncthreads();
+  if constexpr (!SCATTER) return;
 
-  // phase 2: lane (a, half) accumulates the row block (a, b0 .. b0 + NB)
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int lw = lane / LPE;
-  const int le = warp * EPW + lw;
-  const int64_t et = e0 + le;
-  if (SCATTER && lw < EPW && et < n_end) {
-    const int r = lane % LPE;
-    const int a = r % NN, b0 = (r / NN) * NB;
-    R K[NB][3][3], rhs[3] = {R(0), R(0), R(0)};
+  // phase 2: lane a accumulates its row block
+  if constexpr (SCATTER) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int lw = lane / LPE;
+    const int le = warp * EPW + lw;
+    const int64_t et = e0 + le;
+    if (lw < EPW && et < n_end) {
+      const int a = lane % LPE;
+      float K[NB][3][3], rhs[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
-    for (int bb = 0; bb < NB; ++bb)
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] = R(0);
-#pragma unroll 1
-    for (int q = 0; q < NQ; ++q) {
-      const R wl = sm.C[le][q][1], wm = sm.C[le][q][2], wb = sm.C[le][q][3];
-      const R ga[3] = {sm.G[le][q][a][0], sm.G[le][q][a][1], sm.G[le][q][a][2]};
-      const R gl[3] = {wl * ga[0], wl * ga[1], wl * ga[2]};
-      const R gm[3] = {wm * ga[0], wm * ga[1], wm * ga[2]};
-      const R hb[3] = {wb * sm.H[le][q][a][0], wb * sm.H[le][q][a][1], wb * sm.H[le][q][a][2]};
-#pragma unroll
-      for (int bb = 0; bb < NB; ++bb) {
-        const R gb[3] = {sm.G[le][q][b0 + bb][0], sm.G[le][q][b0 + bb][1], sm.G[le][q][b0 + bb][2]};
-        const R hh[3] = {sm.H[le][q][b0 + bb][0], sm.H[le][q][b0 + bb][1], sm.H[le][q][b0 + bb][2]};
-        const R dot = gm[0] * gb[0] + gm[1] * gb[1] + gm[2] * gb[2];
+      for (int bb = 0; bb < NB; ++bb)
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
-          for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] += gl[c] * gb[cc] + gm[cc] * gb[c] - hb[c] * hh[cc];
+          for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] = 0.0f;
+#pragma unroll 1
+      for (int q = 0; q < NQ; ++q) {
+        const float wl = sm.C[le][q][1], wm = sm.C[le][q][2], wb = sm.C[le][q][3];
+        const float ga[3] = {sm.G[le][q][a][0], sm.G[le][q][a][1], sm.G[le][q][a][2]};
+        const float gl[3] = {wl * ga[0], wl * ga[1], wl * ga[2]};
+        const float gm[3] = {wm * ga[0], wm * ga[1], wm * ga[2]};
+        const float hb[3] = {wb * sm.H[le][q][a][0], wb * sm.H[le][q][a][1], wb * sm.H[le][q][a][2]};
 #pragma unroll
-        for (int c = 0; c < 3; ++c) K[bb][c][c] += dot;
-      }
-      if (b0 == 0) {
-        const R* S = sm.S[le][q];
+        for (int bb = 0; bb < NB; ++bb) {
+          const float gb[3] = {sm.G[le][q][bb][0], sm.G[le][q][bb][1], sm.G[le][q][bb][2]};
+          const float hh[3] = {sm.H[le][q][bb][0], sm.H[le][q][bb][1], sm.H[le][q][bb][2]};
+          const float dot = gm[0] * gb[0] + gm[1] * gb[1] + gm[2] * gb[2];
+#pragma unroll
+          for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] += gl[c] * gb[cc] + gm[cc] * gb[c] - hb[c] * hh[cc];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) K[bb][c][c] += dot;
+        }
+        const float* S = sm.S[le][q];
         rhs[0] += S[0] * ga[0] + S[3] * ga[1] + S[5] * ga[2];
         rhs[1] += S[3] * ga[0] + S[1] * ga[1] + S[4] * ga[2];
         rhs[2] += S[5] * ga[0] + S[4] * ga[1] + S[2] * ga[2];
       }
-    }
-    const int64_t g = j2_group_index(P, et);
-    const int64_t node = P.tconn[g * NN + a];
-    const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
-    const int64_t moff = P.mapoff ? P.mapoff[g] : id * NN * NN;
-    const int32_t* mp = P.node_map + moff + a * NN + b0;
-    int64_t rb[3];
+      const int64_t g = group_index(P, et);
+      const int64_t node = P.tconn[g * NN + a];
+      const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
+      const int64_t moff = P.mapoff ? P.mapoff[g] : id * NN * NN;
+      const int32_t* mp = P.node_map + moff + a * NN;
+      int64_t rb[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) rb[c] = P.row_ptr[3 * node + c];
+      for (int c = 0; c < 3; ++c) rb[c] = P.row_ptr[3 * node + c];
 #pragma unroll
-    for (int bb = 0; bb < NB; ++bb) {
-      const int64_t k = mp[bb];
+      for (int bb = 0; bb < NB; ++bb) {
+        const int64_t k = mp[bb];
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
+        for (int c = 0; c < 3; ++c)
 #pragma unroll
-        for (int cc = 0; cc < 3; ++cc) scatter_add<SC>(P.A + rb[c] + 3 * k + cc, widen(K[bb][c][cc]));
-    }
-    if (b0 == 0)
+          for (int cc = 0; cc < 3; ++cc) scatter_add<SC>(P.A + rb[c] + 3 * k + cc, widen(K[bb][c][cc]));
+      }
 #pragma unroll
       for (int c = 0; c < 3; ++c) scatter_add<SC>(P.b + 3 * node + c, widen(rhs[c]));
+    }
+    __syncthreads();
   }
+}
+
+// ---------------------------------------------------------------------------
+// FP64 tiles, by node pairs (pairs.cuh).  With g^_a = sqrt(W) g_a, h^_a = n g^_a
+// and eta = 1 - theta (0 at an elastic point), mu' = mu (1 - eta) and
+// lam' = lam + 2 mu eta / 3, so
+//   A^e_ab = lam M + mu M^T + mu tr(M) I + 2/3 mu N - mu N^T - mu tr(N) I - B,
+//   M = sum_q g^_a (x) g^_b,  N = sum_q eta g^_a (x) g^_b,  B = sum_q beta h^_a (x) h^_b:
+// an elastic point takes the 9 products of M, a plastic one 24 more, where a
+// row block took 36 per ordered pair and point.
+// ---------------------------------------------------------------------------
+template <int TYPE, int SLOT>
+struct J2PairCfg : PairShape<TYPE, SLOT, 3, pair_epc(rule_nq(SLOT))> {
+  using Base = PairShape<TYPE, SLOT, 3, pair_epc(rule_nq(SLOT))>;
+  struct Smem : Base::Nodes {
+    double U[Base::EPC][Base::NN][3];
+    double G[Base::EPC][Base::NQ][Base::GS];  // g^
+    double H[Base::EPC][Base::NQ][Base::GS];  // h^ (plastic points)
+    double C[Base::EPC][Base::NQ][2];         // eta, beta (0, 0 at an elastic point)
+    double S[Base::EPC][Base::NQ][6];         // sqrt(W) sigma
+  };
+};
+
+template <class Cfg>
+__device__ __forceinline__ void j2_pair_point(typename Cfg::Smem& sm, const RefRule& rr, const J2Params& P, int le,
+                                              int q, int64_t et, const double (&J)[3][3], const double (&Ju)[3][3],
+                                              double s) {
+  constexpr int NN = Cfg::NN;
+  const int64_t id = original_id(P, et);
+  double C[3][3], det;
+  double *g = sm.G[le][q], *h = sm.H[le][q];
+  if (!j2_jacobian(P, id, J, C, &det)) {
+#pragma unroll
+    for (int k = 0; k < 3 * NN; ++k) g[k] = h[k] = 0.0;
+    sm.C[le][q][0] = sm.C[le][q][1] = 0.0;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) sm.S[le][q][k] = 0.0;
+    return;
+  }
+  J2Point r;
+  const double rdet = rcp64(det);
+  j2_update(P, id, q, C, rdet, Ju, r);
+  const double root = sqrt(rr.w[q] * det * (1.0 / (s * s * s))), inv = root * (s * rdet);
+  sm.C[le][q][0] = 1.0 - r.theta;
+  sm.C[le][q][1] = P.mu2 * r.theta_bar;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) sm.S[le][q][k] = root * r.sig[k];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) C[i][j] *= inv;
+#pragma unroll
+  for (int u = 0; u < NN; ++u) {
+    const double* d = rr.dN[q][Cfg::node_of(u)];
+    double v[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) g[3 * u + i] = v[i] = fma(d[2], C[i][2], fma(d[1], C[i][1], d[0] * C[i][0]));
+    if (r.yielded) {
+      h[3 * u] = fma(r.n[5], v[2], fma(r.n[3], v[1], r.n[0] * v[0]));
+      h[3 * u + 1] = fma(r.n[4], v[2], fma(r.n[1], v[1], r.n[3] * v[0]));
+      h[3 * u + 2] = fma(r.n[2], v[2], fma(r.n[4], v[1], r.n[5] * v[0]));
+    }
+  }
+}
+
+template <class Cfg, int SC, bool DIAG>
+__device__ __forceinline__ void j2_pair_task(const typename Cfg::Smem& sm, const J2Params& P, int le, int u, int v) {
+  const typename Cfg::Node nu = sm.nd[le][u], nv = sm.nd[le][v];
+  int64_t kuv, kvu;
+  pair_ranks<Cfg>(sm, P, le, u, v, &kuv, &kvu);
+  double M[3][3], N[3][3], B[3][3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) M[c][k] = N[c][k] = B[c][k] = 0.0;
+  double f[1][3] = {{0.0, 0.0, 0.0}};
+#pragma unroll 1
+  for (int q = 0; q < Cfg::NQ; ++q) {
+    const double *a = sm.G[le][q] + 3 * u, *b = sm.G[le][q] + 3 * v;
+    const double eta = sm.C[le][q][0], beta = sm.C[le][q][1];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int k = DIAG ? c : 0; k < 3; ++k) M[c][k] = fma(a[c], b[k], M[c][k]);
+    if (eta != 0.0 || beta != 0.0) {
+      const double *ha = sm.H[le][q] + 3 * u, *hb = sm.H[le][q] + 3 * v;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const double x = eta * a[c], y = beta * ha[c];
+#pragma unroll
+        for (int k = DIAG ? c : 0; k < 3; ++k) {
+          N[c][k] = fma(x, b[k], N[c][k]);
+          B[c][k] = fma(y, hb[k], B[c][k]);
+        }
+      }
+    }
+    if constexpr (DIAG) {
+      const double* S = sm.S[le][q];
+      f[0][0] = fma(S[5], a[2], fma(S[3], a[1], fma(S[0], a[0], f[0][0])));
+      f[0][1] = fma(S[4], a[2], fma(S[1], a[1], fma(S[3], a[0], f[0][1])));
+      f[0][2] = fma(S[2], a[2], fma(S[4], a[1], fma(S[5], a[0], f[0][2])));
+    }
+  }
+  const double tr = P.mu * ((M[0][0] + M[1][1] + M[2][2]) - (N[0][0] + N[1][1] + N[2][2]));
+  double K[3][3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const bool low = DIAG && k < c;  // M, N and B are symmetric on the diagonal
+      const double mt = DIAG ? (low ? M[k][c] : M[c][k]) : M[k][c], nt = DIAG ? (low ? N[k][c] : N[c][k]) : N[k][c];
+      K[c][k] = low ? K[k][c]
+                    : fma(P.lam, M[c][k], fma(P.mu, mt - nt, fma(P.mu2_3, N[c][k], c == k ? tr - B[c][k] : -B[c][k])));
+    }
+  pair_block<SC, DIAG>(P, nu, nv, kuv, kvu, K);
+  if constexpr (DIAG) pair_add<SC>(P.b + 3 * (int64_t)nu.id, 0, f);
+}
+
+template <int TYPE, int SLOT, int SC>
+__device__ __forceinline__ void j2_pair_body(typename J2PairCfg<TYPE, SLOT>::Smem& sm, const RefRule& rr,
+                                             const J2Params& P, int64_t e0, int64_t n_end) {
+  using Cfg = J2PairCfg<TYPE, SLOT>;
+  pair_nodes<Cfg>(sm, P, e0, n_end, P.u, sm.U);
+  __syncthreads();
+  field_points<TYPE, Cfg::NQ, Cfg::EPC, Cfg::THREADS>(
+      sm, rr, e0, n_end, [](int p) { return p; },
+      [&](int le, int q, int64_t et, const double(&J)[3][3], const double(&Ju)[3][3], double s) {
+        j2_pair_point<Cfg>(sm, rr, P, le, q, et, J, Ju, s);
+      });
+  __syncthreads();
+  pair_rounds<Cfg>(
+      sm, e0, n_end, [&](int le, int u, int v) { j2_pair_task<Cfg, SC, false>(sm, P, le, u, v); },
+      [&](int le, int u) { j2_pair_task<Cfg, SC, true>(sm, P, le, u, u); });
   __syncthreads();
 }
 
-template <int TYPE, int SLOT, int PREC, int SPLIT, int SC>
+// The tile of an element type in a precision; POINTS: the element loop's.
+template <int TYPE, int SLOT, int PREC, bool POINTS = false>
+struct J2Tile {
+  using Cfg = J2Cfg<TYPE, SLOT>;
+  using Smem = std::conditional_t<POINTS, typename Cfg::Fields, typename Cfg::Smem>;
+  template <int SC>
+  __device__ static __forceinline__ void run(unsigned char* raw, const RefRule& rr, const J2Params& P, int64_t e0,
+                                             int64_t n_end) {
+    j2_tile_body<TYPE, SLOT, SC, !POINTS>(*reinterpret_cast<Smem*>(raw), rr, P, e0, n_end);
+  }
+};
+template <int TYPE, int SLOT>
+struct J2Tile<TYPE, SLOT, FEA_FP64, false> {
+  using Cfg = J2PairCfg<TYPE, SLOT>;
+  using Smem = typename Cfg::Smem;
+  template <int SC>
+  __device__ static __forceinline__ void run(unsigned char* raw, const RefRule& rr, const J2Params& P, int64_t e0,
+                                             int64_t n_end) {
+    j2_pair_body<TYPE, SLOT, SC>(*reinterpret_cast<Smem*>(raw), rr, P, e0, n_end);
+  }
+};
+
+// one tile per CTA
+template <int TYPE, int SLOT, int PREC, int SC, bool POINTS>
 __global__ void __launch_bounds__(128) k_j2_tile(const __grid_constant__ RefRule rr, const __grid_constant__ J2Params P) {
-  using Cfg = J2Cfg<TYPE, SLOT, PREC, SPLIT>;
+  using T = J2Tile<TYPE, SLOT, PREC, POINTS>;
   extern __shared__ __align__(16) unsigned char j2_smem_raw[];
-  j2_tile_body<TYPE, SLOT, PREC, SPLIT, SC>(*reinterpret_cast<typename Cfg::Smem*>(j2_smem_raw), rr, P,
-                                            (int64_t)blockIdx.x * Cfg::EPC, P.n);
+  T::template run<SC>(j2_smem_raw, rr, P, (int64_t)blockIdx.x * T::Cfg::EPC, P.n);
 }
 
-// element-wise loop: one tile of Gauss-point updates per CTA
-template <int TYPE, int SLOT>
-__global__ void __launch_bounds__(128) k_j2_points(const __grid_constant__ RefRule rr, const __grid_constant__ J2Params P) {
-  using Cfg = J2Cfg<TYPE, SLOT, FEA_FP32_INTEGRATE, 1>;
-  extern __shared__ __align__(16) unsigned char j2_smem_raw[];
-  j2_tile_body<TYPE, SLOT, FEA_FP32_INTEGRATE, 1, FEA_SCATTER_ATOMIC, false>(
-      *reinterpret_cast<typename Cfg::Smem*>(j2_smem_raw), rr, P, (int64_t)blockIdx.x * Cfg::EPC, P.n);
-}
-
-template <int TYPE, int SLOT>
-static int launch_j2_points(const J2Params& P, cudaStream_t s) {
-  using Cfg = J2Cfg<TYPE, SLOT, FEA_FP32_INTEGRATE, 1>;
-  constexpr size_t smem = sizeof(typename Cfg::Smem);
-  auto kern = k_j2_points<TYPE, SLOT>;
-  if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<grid_for(P.n, Cfg::EPC), Cfg::THREADS, smem, s>>>(host_rule(SLOT), P);
-  FEA_CUDA(cudaGetLastError());
-  return FEA_OK;
-}
-
-template <int TYPE, int SLOT, int PREC, int SPLIT, int SC>
+template <int TYPE, int SLOT, int PREC, int SC, bool POINTS = false>
 static int launch_j2(const J2Params& P, cudaStream_t s) {
-  using Cfg = J2Cfg<TYPE, SLOT, PREC, SPLIT>;
-  constexpr size_t smem = sizeof(typename Cfg::Smem);
+  using T = J2Tile<TYPE, SLOT, PREC, POINTS>;
+  constexpr size_t smem = sizeof(typename T::Smem);
   static_assert(smem <= 227 * 1024, "J2 tile exceeds shared memory");
-  auto kern = k_j2_tile<TYPE, SLOT, PREC, SPLIT, SC>;
+  auto kern = k_j2_tile<TYPE, SLOT, PREC, SC, POINTS>;
   if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const unsigned grid = grid_for(P.n, Cfg::EPC);
-  kern<<<grid, Cfg::THREADS, smem, s>>>(host_rule(SLOT), P);
+  kern<<<grid_for(P.n, T::Cfg::EPC), T::Cfg::THREADS, smem, s>>>(host_rule(SLOT), P);
   FEA_CUDA(cudaGetLastError());
   return FEA_OK;
 }
 
-template <int PREC, int SC>
+template <int PREC, int SC, bool POINTS = false>
 static int launch_j2_type(int type, const J2Params& P, cudaStream_t s) {
-  constexpr int S2 = PREC == FEA_FP64 ? 2 : 1;  // FP64 splits the columns of hex8 / prism6 over two lanes
   switch (type) {
-    case FEA_TET4: return launch_j2<FEA_TET4, kRuleTet4, PREC, 1, SC>(P, s);
-    case FEA_PYR5: return launch_j2<FEA_PYR5, kRulePyr8, PREC, 1, SC>(P, s);
-    case FEA_PRISM6: return launch_j2<FEA_PRISM6, kRulePrism6, PREC, S2, SC>(P, s);
-    default: return launch_j2<FEA_HEX8, kRuleHex8, PREC, S2, SC>(P, s);
+    case FEA_TET4: return launch_j2<FEA_TET4, kRuleTet4, PREC, SC, POINTS>(P, s);
+    case FEA_PYR5: return launch_j2<FEA_PYR5, kRulePyr8, PREC, SC, POINTS>(P, s);
+    case FEA_PRISM6: return launch_j2<FEA_PRISM6, kRulePrism6, PREC, SC, POINTS>(P, s);
+    default: return launch_j2<FEA_HEX8, kRuleHex8, PREC, SC, POINTS>(P, s);
   }
 }
 
@@ -500,28 +599,32 @@ struct PersistJ2Args {
   SchedArgs S;
 };
 
-template <int PREC>
+template <int PREC, bool POINTS>
 struct PersistJ2Cfg {
-  static constexpr int S2 = PREC == FEA_FP64 ? 2 : 1;
-  template <int TYPE, int SLOT, int SPLIT>
-  static constexpr size_t bytes() { return sizeof(typename J2Cfg<TYPE, SLOT, PREC, SPLIT>::Smem); }
+  template <int TYPE, int SLOT>
+  static constexpr size_t bytes() { return sizeof(typename J2Tile<TYPE, SLOT, PREC, POINTS>::Smem); }
   static constexpr size_t mx(size_t a, size_t b) { return a > b ? a : b; }
-  static constexpr size_t smem = mx(mx(bytes<FEA_TET4, kRuleTet4, 1>(), bytes<FEA_PYR5, kRulePyr8, 1>()),
-                                    mx(bytes<FEA_PRISM6, kRulePrism6, S2>(), bytes<FEA_HEX8, kRuleHex8, S2>()));
+  static constexpr size_t smem = mx(mx(bytes<FEA_TET4, kRuleTet4>(), bytes<FEA_PYR5, kRulePyr8>()),
+                                    mx(bytes<FEA_PRISM6, kRulePrism6>(), bytes<FEA_HEX8, kRuleHex8>()));
 };
 
-template <int TYPE, int SLOT, int PREC, int SPLIT, bool SCATTER>
+template <int TYPE, int SLOT, int PREC, bool POINTS>
 __device__ __forceinline__ void persist_j2_item(unsigned char* raw, const J2Params& P, int64_t first, int64_t end) {
-  using Cfg = J2Cfg<TYPE, SLOT, PREC, SPLIT>;
-  auto& sm = *reinterpret_cast<typename Cfg::Smem*>(raw);
-  for (int64_t e0 = first; e0 < end; e0 += Cfg::EPC)
-    j2_tile_body<TYPE, SLOT, PREC, SPLIT, FEA_SCATTER_ATOMIC, SCATTER>(sm, c_rules_j2[SLOT], P, e0, end);
+  using T = J2Tile<TYPE, SLOT, PREC, POINTS>;
+  for (int64_t e0 = first; e0 < end; e0 += T::Cfg::EPC)
+    T::template run<FEA_SCATTER_ATOMIC>(raw, c_rules_j2[SLOT], P, e0, end);
+}
+
+// One item of the any-type kernel, not inlined: four inlined tile bodies take
+// 213 registers in FP32 where the largest needs 126.
+template <int TYPE, int SLOT, int PREC, bool POINTS>
+__device__ __noinline__ void persist_j2_call(unsigned char* raw, const J2Params& P, int64_t first, int64_t end) {
+  persist_j2_item<TYPE, SLOT, PREC, POINTS>(raw, P, first, end);
 }
 
 // ONLY == kRuleHex8: a mesh of hexes only (one tile body); -1: any type
-template <int PREC, int ONLY, bool SCATTER>
-__global__ void __launch_bounds__(128) k_persistent_j2(const __grid_constant__ PersistJ2Args A) {
-  constexpr int S2 = PersistJ2Cfg<PREC>::S2;
+template <int PREC, int ONLY, bool POINTS>
+__global__ void __launch_bounds__(128, PREC == FEA_FP64 ? 3 : 4) k_persistent_j2(const __grid_constant__ PersistJ2Args A) {
   extern __shared__ __align__(16) unsigned char persist_j2_smem[];
   __shared__ int s_item;
   sched_start(A.S);
@@ -534,15 +637,15 @@ __global__ void __launch_bounds__(128) k_persistent_j2(const __grid_constant__ P
     const int64_t first = it.first, end = (int64_t)it.first + it.count;
     // entry t is type t: the parameters are read at constant offsets
     if constexpr (ONLY == kRuleHex8) {
-      persist_j2_item<FEA_HEX8, kRuleHex8, PREC, S2, SCATTER>(persist_j2_smem, A.table[FEA_HEX8], first, end);
+      persist_j2_item<FEA_HEX8, kRuleHex8, PREC, POINTS>(persist_j2_smem, A.table[FEA_HEX8], first, end);
     } else {
       switch (A.slot[it.entry]) {
-        case kRulePyr8: persist_j2_item<FEA_PYR5, kRulePyr8, PREC, 1, SCATTER>(persist_j2_smem, A.table[FEA_PYR5], first, end); break;
+        case kRulePyr8: persist_j2_call<FEA_PYR5, kRulePyr8, PREC, POINTS>(persist_j2_smem, A.table[FEA_PYR5], first, end); break;
         case kRulePrism6:
-          persist_j2_item<FEA_PRISM6, kRulePrism6, PREC, S2, SCATTER>(persist_j2_smem, A.table[FEA_PRISM6], first, end);
+          persist_j2_call<FEA_PRISM6, kRulePrism6, PREC, POINTS>(persist_j2_smem, A.table[FEA_PRISM6], first, end);
           break;
-        case kRuleHex8: persist_j2_item<FEA_HEX8, kRuleHex8, PREC, S2, SCATTER>(persist_j2_smem, A.table[FEA_HEX8], first, end); break;
-        default: persist_j2_item<FEA_TET4, kRuleTet4, PREC, 1, SCATTER>(persist_j2_smem, A.table[FEA_TET4], first, end); break;
+        case kRuleHex8: persist_j2_call<FEA_HEX8, kRuleHex8, PREC, POINTS>(persist_j2_smem, A.table[FEA_HEX8], first, end); break;
+        default: persist_j2_call<FEA_TET4, kRuleTet4, PREC, POINTS>(persist_j2_smem, A.table[FEA_TET4], first, end); break;
       }
     }
     sched_record(A.S, item, it.entry, t0);
@@ -584,23 +687,27 @@ static J2Params j2_base_params(const fea_operator* op, fea_mesh* m, const int64_
   P.lam = E * nu / ((1.0 + nu) * (1.0 - 2.0 * nu));
   P.mu = E / (2.0 * (1.0 + nu));
   P.kappa = P.lam + 2.0 * P.mu / 3.0;
+  P.mu2 = 2.0 * P.mu;
   P.mu2_3 = 2.0 * P.mu / 3.0;
+  P.inv3mu = 1.0 / (3.0 * P.mu);
   P.s0 = op->sigma0;
   P.sinf = op->sigma_inf;
   P.delta = op->delta;
   P.hard = op->hardening;
   P.tol_g = op->tol_g;
   P.tol_step = op->tol_step;
+  P.gp0 = -2.0 * P.mu - (2.0 / 3.0) * P.hard;
+  P.gp1 = -(2.0 / 3.0) * (P.sinf - P.s0) * P.delta;
   P.max_iter = op->max_iter;
   return P;
 }
 
-template <int PREC, int ONLY, bool SCATTER = true>
+template <int PREC, int ONLY, bool POINTS = false>
 static int launch_persistent_j2_t(const PersistJ2Args& args, int n_ctas, bool dry, cudaStream_t s, int* grid_out) {
   constexpr size_t smem = ONLY == kRuleHex8
-                              ? sizeof(typename J2Cfg<FEA_HEX8, kRuleHex8, PREC, PersistJ2Cfg<PREC>::S2>::Smem)
-                              : PersistJ2Cfg<PREC>::smem;
-  auto kern = k_persistent_j2<PREC, ONLY, SCATTER>;
+                              ? sizeof(typename J2Tile<FEA_HEX8, kRuleHex8, PREC, POINTS>::Smem)
+                              : PersistJ2Cfg<PREC, POINTS>::smem;
+  auto kern = k_persistent_j2<PREC, ONLY, POINTS>;
   if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int grid = n_ctas;
   if (grid <= 0) {
@@ -644,8 +751,8 @@ int launch_persistent_j2(const fea_operator* op, fea_mesh* m, const int64_t* row
   for (int t = 0; t < kNumTypes; ++t)
     if (t != FEA_HEX8 && m->group[t].n) hex_only = false;
   if (points_only)  // the element-wise loop: Gauss-point updates only
-    return hex_only ? launch_persistent_j2_t<FEA_FP32_INTEGRATE, kRuleHex8, false>(args, n_ctas, dry, s, grid_out)
-                    : launch_persistent_j2_t<FEA_FP32_INTEGRATE, -1, false>(args, n_ctas, dry, s, grid_out);
+    return hex_only ? launch_persistent_j2_t<FEA_FP32_INTEGRATE, kRuleHex8, true>(args, n_ctas, dry, s, grid_out)
+                    : launch_persistent_j2_t<FEA_FP32_INTEGRATE, -1, true>(args, n_ctas, dry, s, grid_out);
   if (op->precision == FEA_FP64)
     return hex_only ? launch_persistent_j2_t<FEA_FP64, kRuleHex8>(args, n_ctas, dry, s, grid_out)
                     : launch_persistent_j2_t<FEA_FP64, -1>(args, n_ctas, dry, s, grid_out);
@@ -734,12 +841,7 @@ int element_loop_j2(const fea_operator* op, fea_mesh* m, double* stress, cudaStr
     P.mapoff = g.mapoff;
     P.list = nullptr;
     P.n = g.n;
-    switch (t) {
-      case FEA_TET4: rc = launch_j2_points<FEA_TET4, kRuleTet4>(P, s); break;
-      case FEA_PYR5: rc = launch_j2_points<FEA_PYR5, kRulePyr8>(P, s); break;
-      case FEA_PRISM6: rc = launch_j2_points<FEA_PRISM6, kRulePrism6>(P, s); break;
-      default: rc = launch_j2_points<FEA_HEX8, kRuleHex8>(P, s); break;
-    }
+    rc = launch_j2_type<FEA_FP32_INTEGRATE, FEA_SCATTER_ATOMIC, true>(t, P, s);
     if (rc) return rc;
     if (2 + launched < nev) FEA_CUDA(cudaEventRecord(ev[2 + launched], s));
     ++launched;

@@ -17,155 +17,159 @@
 // F^-T, ln J and P.  The gradient products (h_a and the blocks) run in the
 // tile precision (FP32 for FEA_FP32_INTEGRATE) and are added into A and b in
 // FP64, by atomics (ATOMIC) or plain read-modify-writes (COLOR).
+//
+// Both precisions are bound by the number of FP64 instructions (pairs.cuh).
+// F - I = Ju C^T / det of every type from the displacement field's reference
+// Jacobian Ju (RefMap, or the modal transform), reciprocals by rcp64, and FP64
+// tiles form the node pairs of the symmetric element matrix: with
+// g^_a = sqrt(W) g_a and h^_a = sqrt(W) h_a,
+//   A^e_ab = lam M + N^T + (mu D + m sum_q W N_a N_b) I,
+//   M = sum_q h^_a (x) h^_b,  N = sum_q (mu - lam ln J) h^_a (x) h^_b,
+//   D = sum_q g^_a . g^_b,
+// 24 products per pair and point where a row block took 28 per ordered pair.
+// 65,559 hex8, FP64, one GB300: 2.81 -> 1.29 ms.
 #include <cmath>
 #include <cstring>
 #include <type_traits>
 
 #include "element.cuh"
 #include "fea_internal.cuh"
+#include "pairs.cuh"
 
 namespace fea {
 
-struct NHParams {
-  const double* coords;
-  const int32_t* tconn;   // [n][NN] packed connectivity of the type group
-  const int32_t* ids;     // group index -> original id (nullptr: identity)
-  const int64_t* mapoff;  // group index -> node_map offset (nullptr: id * NN^2)
-  const int32_t* list;    // launch index -> group index (nullptr: identity; coloring)
-  int64_t n;
-  const int64_t* row_ptr;
-  const int32_t* node_map;
-  double* A;
-  double* b;
-  DevStatus* st;
+struct NHParams : ElemParams {
   const double* u;
   double lam, mu, mass;
 };
 
-template <int TYPE, int SLOT, int PREC, int SPLIT>
+// FP32 tiles: lane a of an element's NN lanes holds its row block.
+template <int TYPE, int SLOT>
 struct NHCfg {
   static constexpr int NN = nodes_of(TYPE);
   static constexpr int NQ = rule_nq(SLOT);
-  static constexpr int LPE = NN * SPLIT;
+  static constexpr int LPE = NN;
   static constexpr int EPW = 32 / LPE;
   static constexpr int WARPS = 4;
   static constexpr int THREADS = 32 * WARPS;
   static constexpr int EPC = EPW * WARPS;
-  static constexpr int NB = NN / SPLIT;
-  static constexpr bool kModal = TYPE == FEA_HEX8 && SLOT == kRuleHex8;
-  static_assert(NN % SPLIT == 0, "SPLIT must divide the node count");
-  static_assert(!kModal || (EPC * 8 % 32 == 0 && EPC * 8 <= THREADS), "modal hex geometry needs whole warps");
-  using R = typename std::conditional<PREC == FEA_FP64, double, float>::type;
+  static constexpr int NB = NN;
+  static constexpr bool kHex = TYPE == FEA_HEX8;
+  static_assert(!kHex || (EPC * 8 % 32 == 0 && EPC * 8 <= THREADS), "modal hex geometry needs whole warps");
   struct Smem {
     double X[EPC][NN][3];
     double U[EPC][NN][3];
-    R G[EPC][NQ][NN][3];  // g_a = grad0 N_a
-    R H[EPC][NQ][NN][3];  // h_a = F^-T g_a
-    R C[EPC][NQ][4];      // W mu, W lam, W (mu - lam ln J), W m
-    R S[EPC][NQ][9];      // W P, row-major
+    float G[EPC][NQ][NN][3];  // g_a = grad0 N_a
+    float H[EPC][NQ][NN][3];  // h_a = F^-T g_a
+    float C[EPC][NQ][4];      // W mu, W lam, W (mu - lam ln J), W m
+    float S[EPC][NQ][9];      // W P, row-major
   };
 };
 
-__device__ __forceinline__ int64_t nh_group_index(const NHParams& P, int64_t et) {
-  return P.list ? (int64_t)P.list[et] : et;
-}
+// The kinematics of one point (FP64), from the Jacobian J' = s J0 (s a power
+// of two) and Ju' = s Ju of the displacement field: C' and det' of J', F^-T,
+// ln J and W P.  False (and latched) if the element is inverted in the
+// reference configuration or by the deformation.
+struct NHPoint {
+  double C[3][3], Fit[3][3], WP[3][3];
+  double rdet, W, lnJ;
+};
 
-// Phase 1 of point q of element le (FP64): J' = s J0 is the reference
-// Jacobian scaled by a power of two s; writes the point's factors in the
-// tile precision into shared memory.  MODAL (hex8, FP32 tiles): Ju' = s Ju
-// is the displacement field's reference Jacobian from the modal transform of
-// the nodal displacements, so F - I = Ju' C'^T / det' in FP64 and the
-// reference gradients are formed in FP32 from C' and det' rounded once.
-template <class Cfg, bool MODAL = false>
-__device__ __forceinline__ void nh_point(typename Cfg::Smem& sm, const RefRule& rr, const NHParams& P, int le, int q,
-                                         int64_t et, double (&J)[3][3], double s, const double (*Ju)[3] = nullptr) {
-  using R = typename Cfg::R;
-  constexpr int NN = Cfg::NN;
-  const int64_t g = nh_group_index(P, et);
-  const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
-  double C[3][3];
-  cofactors(J, C);
-  const double det = J[0][0] * C[0][0] + J[0][1] * C[0][1] + J[0][2] * C[0][2];
-  R gt[NN][3];  // g_a in the tile precision
-  double F[3][3] = {{1, 0, 0}, {0, 1, 0}, {0, 0, 1}};
-  double Fc[3][3], detF = 0.0;
+__device__ __forceinline__ bool nh_kinematics(const NHParams& P, int64_t id, double w, const double (&J)[3][3],
+                                              const double (&Ju)[3][3], double s, NHPoint& r) {
+  cofactors(J, r.C);
+  const double det = J[0][0] * r.C[0][0] + J[0][1] * r.C[0][1] + J[0][2] * r.C[0][2];
+  double F[3][3], Fc[3][3], detF = 0.0;
   if (det > 0.0) {
-    if constexpr (MODAL) {
-      static_assert(!std::is_same<R, double>::value, "the modal path forms FP32 gradients");
-      const double rdet = 1.0 / det;
+    r.rdet = rcp64(det);
 #pragma unroll
-      for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < 3; ++i)
 #pragma unroll
-        for (int j = 0; j < 3; ++j) F[i][j] += (Ju[i][0] * C[j][0] + Ju[i][1] * C[j][1] + Ju[i][2] * C[j][2]) * rdet;
-      float Cf[3][3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int j = 0; j < 3; ++j) Cf[i][j] = f64_to_f32_rn(C[i][j]);
-      const float invf = (float)s / f64_to_f32_rn(det);
-#pragma unroll
-      for (int a = 0; a < NN; ++a)
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-          gt[a][i] = (rr.dNf[q][a][0] * Cf[i][0] + rr.dNf[q][a][1] * Cf[i][1] + rr.dNf[q][a][2] * Cf[i][2]) * invf;
-    } else {
-      const double inv = s / det;
-#pragma unroll
-      for (int a = 0; a < NN; ++a) {
-        double gd[3];
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-          gd[i] = (rr.dN[q][a][0] * C[i][0] + rr.dN[q][a][1] * C[i][1] + rr.dN[q][a][2] * C[i][2]) * inv;
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-          for (int j = 0; j < 3; ++j) F[i][j] = fma(sm.U[le][a][i], gd[j], F[i][j]);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) gt[a][i] = to_tile<R>(gd[i]);
+      for (int j = 0; j < 3; ++j) {
+        const double h = fma(Ju[i][2], r.C[j][2], fma(Ju[i][1], r.C[j][1], Ju[i][0] * r.C[j][0]));
+        F[i][j] = i == j ? fma(h, r.rdet, 1.0) : h * r.rdet;
       }
-    }
     cofactors(F, Fc);  // cof F = det F * F^-T
     detF = F[0][0] * Fc[0][0] + F[0][1] * Fc[0][1] + F[0][2] * Fc[0][2];
   }
   if (!(det > 0.0) || !(detF > 0.0)) {
-    // inverted in the reference configuration or by the deformation
     latch_error(P.st, FEA_ERR_INVERTED_ELEMENT, (unsigned long long)id);
+    return false;
+  }
+  const double rJ = rcp64(detF);
+  r.lnJ = log(detF);
+  r.W = w * det * (1.0 / (s * s * s));
+  // P = mu (F - F^-T) + lam ln J F^-T
+  const double a = r.W * P.mu, b = fma(r.W * P.lam, r.lnJ, -a);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) sm.C[le][q][k] = R(0);
+  for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int k = 0; k < 9; ++k) sm.S[le][q][k] = R(0);
+    for (int j = 0; j < 3; ++j) {
+      r.Fit[i][j] = Fc[i][j] * rJ;
+      r.WP[i][j] = fma(b, r.Fit[i][j], a * F[i][j]);
+    }
+  return true;
+}
+
+// Phase 1 of point q of element le of an FP32 tile.  Hex gradients are formed
+// in FP32 from C' and det' rounded once, the other types' in FP64 and rounded.
+template <class Cfg>
+__device__ __forceinline__ void nh_point(typename Cfg::Smem& sm, const RefRule& rr, const NHParams& P, int le, int q,
+                                         int64_t et, const double (&J)[3][3], const double (&Ju)[3][3], double s) {
+  constexpr int NN = Cfg::NN;
+  NHPoint r;
+  if (!nh_kinematics(P, original_id(P, et), rr.w[q], J, Ju, s, r)) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) sm.C[le][q][k] = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) sm.S[le][q][k] = 0.0f;
 #pragma unroll
     for (int a = 0; a < NN; ++a)
 #pragma unroll
-      for (int i = 0; i < 3; ++i) sm.G[le][q][a][i] = sm.H[le][q][a][i] = R(0);
+      for (int i = 0; i < 3; ++i) sm.G[le][q][a][i] = sm.H[le][q][a][i] = 0.0f;
     return;
   }
-  const double rJ = 1.0 / detF;
-  double Fit[3][3];  // F^-T
+  sm.C[le][q][0] = f64_to_f32_rn(r.W * P.mu);
+  sm.C[le][q][1] = f64_to_f32_rn(r.W * P.lam);
+  sm.C[le][q][2] = f64_to_f32_rn(r.W * (P.mu - P.lam * r.lnJ));
+  sm.C[le][q][3] = f64_to_f32_rn(r.W * P.mass);
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) Fit[i][j] = Fc[i][j] * rJ;
-  const double lnJ = log(detF);
-  const double W = rr.w[q] * det * (1.0 / (s * s * s));
-  sm.C[le][q][0] = to_tile<R>(W * P.mu);
-  sm.C[le][q][1] = to_tile<R>(W * P.lam);
-  sm.C[le][q][2] = to_tile<R>(W * (P.mu - P.lam * lnJ));
-  sm.C[le][q][3] = to_tile<R>(W * P.mass);
+    for (int j = 0; j < 3; ++j) sm.S[le][q][3 * i + j] = f64_to_f32_rn(r.WP[i][j]);
+  float gt[NN][3];  // g_a
+  if constexpr (Cfg::kHex) {
+    const double det = J[0][0] * r.C[0][0] + J[0][1] * r.C[0][1] + J[0][2] * r.C[0][2];
+    float Cf[3][3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) Cf[i][j] = f64_to_f32_rn(r.C[i][j]);
+    const float invf = (float)s / f64_to_f32_rn(det);
+#pragma unroll
+    for (int a = 0; a < NN; ++a)
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+        gt[a][i] = (rr.dNf[q][a][0] * Cf[i][0] + rr.dNf[q][a][1] * Cf[i][1] + rr.dNf[q][a][2] * Cf[i][2]) * invf;
+  } else {
+    const double inv = s * r.rdet;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const double c0 = r.C[i][0] * inv, c1 = r.C[i][1] * inv, c2 = r.C[i][2] * inv;
+#pragma unroll
+      for (int a = 0; a < NN; ++a)
+        gt[a][i] = f64_to_f32_rn(fma(rr.dN[q][a][2], c2, fma(rr.dN[q][a][1], c1, rr.dN[q][a][0] * c0)));
+    }
+  }
+  // h_a = F^-T g_a in FP32, like the other gradient products
+  float Ft[3][3];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j)
-      sm.S[le][q][3 * i + j] = to_tile<R>(W * (P.mu * (F[i][j] - Fit[i][j]) + P.lam * lnJ * Fit[i][j]));
-  // h_a = F^-T g_a in the tile precision, like the other gradient products
-  R Ft[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) Ft[i][j] = to_tile<R>(Fit[i][j]);
+    for (int j = 0; j < 3; ++j) Ft[i][j] = f64_to_f32_rn(r.Fit[i][j]);
 #pragma unroll
   for (int a = 0; a < NN; ++a) {
-    const R g0 = gt[a][0], g1 = gt[a][1], g2 = gt[a][2];
+    const float g0 = gt[a][0], g1 = gt[a][1], g2 = gt[a][2];
     sm.G[le][q][a][0] = g0;
     sm.G[le][q][a][1] = g1;
     sm.G[le][q][a][2] = g2;
@@ -174,20 +178,19 @@ __device__ __forceinline__ void nh_point(typename Cfg::Smem& sm, const RefRule& 
   }
 }
 
-// One tile of EPC elements from launch index e0 (elements at or past n_end
-// are skipped).  Every thread of the CTA calls it; it ends with a barrier.
-template <int TYPE, int SLOT, int PREC, int SPLIT, int SC>
-__device__ __forceinline__ void nh_tile_body(typename NHCfg<TYPE, SLOT, PREC, SPLIT>::Smem& sm, const RefRule& rr,
+// One FP32 tile of EPC elements from launch index e0 (elements at or past
+// n_end are skipped).  Every thread of the CTA calls it; it ends with a barrier.
+template <int TYPE, int SLOT, int SC>
+__device__ __forceinline__ void nh_tile_body(typename NHCfg<TYPE, SLOT>::Smem& sm, const RefRule& rr,
                                              const NHParams& P, int64_t e0, int64_t n_end) {
-  using Cfg = NHCfg<TYPE, SLOT, PREC, SPLIT>;
-  using R = typename Cfg::R;
+  using Cfg = NHCfg<TYPE, SLOT>;
   constexpr int NN = Cfg::NN, NQ = Cfg::NQ, EPC = Cfg::EPC, NB = Cfg::NB, LPE = Cfg::LPE, EPW = Cfg::EPW;
   // phase 0: coordinates and displacements of the tile's nodes
   for (int t = threadIdx.x; t < EPC * NN; t += Cfg::THREADS) {
     const int le = t / NN, a = t % NN;
     const int64_t et = e0 + le;
     if (et < n_end) {
-      const int64_t node = P.tconn[nh_group_index(P, et) * NN + a];
+      const int64_t node = P.tconn[group_index(P, et) * NN + a];
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
         sm.X[le][a][i] = P.coords[3 * node + i];
@@ -197,104 +200,40 @@ __device__ __forceinline__ void nh_tile_body(typename NHCfg<TYPE, SLOT, PREC, SP
   }
   __syncthreads();
   // phase 1: one thread per (element, point)
-  if constexpr (Cfg::kModal) {
-    const int t = threadIdx.x;
-    if (t < EPC * 8) {
-      const int le = t >> 3, p = t & 7;
-      const int64_t et = e0 + le;
-      const bool valid = et < n_end;
-      const int a = hex8_corner_node(p);
-      // FP32 tiles take the displacements to modal form as well (F then
-      // needs no FP64 gradients); sm.U holds modal coefficients after
-      constexpr bool kModalU = PREC != FEA_FP64;
-      double v[3], vu[3];
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        v[i] = valid ? sm.X[le][a][i] : 0.0;
-        vu[i] = valid ? sm.U[le][a][i] : 0.0;
-      }
-      hex8_modal(v);
-      if constexpr (kModalU) hex8_modal(vu);
-      __syncwarp();
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        sm.X[le][p][i] = v[i];
-        if constexpr (kModalU) sm.U[le][p][i] = vu[i];
-      }
-      __syncwarp();
-      // every lane forms its Jacobians (the lanes of an element exchange
-      // columns); the valid ones use them
-      double J[3][3], Ju[3][3];
-      hex8_jacobian_pairs(sm.X[le], p, J);
-      if constexpr (kModalU) hex8_jacobian_pairs(sm.U[le], p, Ju);
-      if (valid) {
-        if constexpr (kModalU)
-          nh_point<Cfg, true>(sm, rr, P, le, p, et, J, 8.0, Ju);
-        else
-          nh_point<Cfg>(sm, rr, P, le, p, et, J, 8.0);
-      }
-    }
-  } else {
-    for (int t = threadIdx.x; t < EPC * NQ; t += Cfg::THREADS) {
-      const int le = t / NQ, q = t % NQ;
-      const int64_t et = e0 + le;
-      if (et >= n_end) continue;
-      double J[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-#pragma unroll
-      for (int a = 1; a < NN; ++a) {
-        const double d0 = sm.X[le][a][0] - sm.X[le][0][0];
-        const double d1 = sm.X[le][a][1] - sm.X[le][0][1];
-        const double d2 = sm.X[le][a][2] - sm.X[le][0][2];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          J[0][j] += d0 * rr.dN[q][a][j];
-          J[1][j] += d1 * rr.dN[q][a][j];
-          J[2][j] += d2 * rr.dN[q][a][j];
-        }
-      }
-      nh_point<Cfg>(sm, rr, P, le, q, et, J, 1.0);
-    }
-  }
+  field_points<TYPE, NQ, EPC, Cfg::THREADS>(
+      sm, rr, e0, n_end, [](int p) { return hex8_corner_node(p); },
+      [&](int le, int q, int64_t et, const double(&J)[3][3], const double(&Ju)[3][3], double s) {
+        nh_point<Cfg>(sm, rr, P, le, q, et, J, Ju, s);
+      });
   __syncthreads();
 
-  // phase 2: lane (a, half) accumulates the row block (a, b0 .. b0 + NB)
+  // phase 2: lane a accumulates its row block
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int lw = lane / LPE;
   const int le = warp * EPW + lw;
   const int64_t et = e0 + le;
   if (lw < EPW && et < n_end) {
-    const int r = lane % LPE;
-    const int a = r % NN, b0 = (r / NN) * NB;
-    R K[NB][3][3], rhs[3] = {R(0), R(0), R(0)};
+    const int a = lane % LPE;
+    float K[NB][3][3], rhs[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int bb = 0; bb < NB; ++bb)
 #pragma unroll
       for (int c = 0; c < 3; ++c)
 #pragma unroll
-        for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] = R(0);
+        for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] = 0.0f;
 #pragma unroll 1
     for (int q = 0; q < NQ; ++q) {
-      const R wm = sm.C[le][q][0], wl = sm.C[le][q][1], wp = sm.C[le][q][2], wn = sm.C[le][q][3];
-      const R ga[3] = {sm.G[le][q][a][0], sm.G[le][q][a][1], sm.G[le][q][a][2]};
-      const R gm[3] = {wm * ga[0], wm * ga[1], wm * ga[2]};
-      const R hl[3] = {wl * sm.H[le][q][a][0], wl * sm.H[le][q][a][1], wl * sm.H[le][q][a][2]};
-      const R hp[3] = {wp * sm.H[le][q][a][0], wp * sm.H[le][q][a][1], wp * sm.H[le][q][a][2]};
-      R Nqa;
-      if constexpr (PREC == FEA_FP64)
-        Nqa = rr.N[q][a];
-      else
-        Nqa = rr.Nf[q][a];
-      const R mn = wn * Nqa;
+      const float wm = sm.C[le][q][0], wl = sm.C[le][q][1], wp = sm.C[le][q][2], wn = sm.C[le][q][3];
+      const float ga[3] = {sm.G[le][q][a][0], sm.G[le][q][a][1], sm.G[le][q][a][2]};
+      const float gm[3] = {wm * ga[0], wm * ga[1], wm * ga[2]};
+      const float hl[3] = {wl * sm.H[le][q][a][0], wl * sm.H[le][q][a][1], wl * sm.H[le][q][a][2]};
+      const float hp[3] = {wp * sm.H[le][q][a][0], wp * sm.H[le][q][a][1], wp * sm.H[le][q][a][2]};
+      const float mn = wn * rr.Nf[q][a];
 #pragma unroll
       for (int bb = 0; bb < NB; ++bb) {
-        const R gb[3] = {sm.G[le][q][b0 + bb][0], sm.G[le][q][b0 + bb][1], sm.G[le][q][b0 + bb][2]};
-        const R hb[3] = {sm.H[le][q][b0 + bb][0], sm.H[le][q][b0 + bb][1], sm.H[le][q][b0 + bb][2]};
-        R Nqb;
-        if constexpr (PREC == FEA_FP64)
-          Nqb = rr.N[q][b0 + bb];
-        else
-          Nqb = rr.Nf[q][b0 + bb];
-        const R diag = gm[0] * gb[0] + gm[1] * gb[1] + gm[2] * gb[2] + mn * Nqb;
+        const float gb[3] = {sm.G[le][q][bb][0], sm.G[le][q][bb][1], sm.G[le][q][bb][2]};
+        const float hb[3] = {sm.H[le][q][bb][0], sm.H[le][q][bb][1], sm.H[le][q][bb][2]};
+        const float diag = gm[0] * gb[0] + gm[1] * gb[1] + gm[2] * gb[2] + mn * rr.Nf[q][bb];
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -302,17 +241,15 @@ __device__ __forceinline__ void nh_tile_body(typename NHCfg<TYPE, SLOT, PREC, SP
 #pragma unroll
         for (int c = 0; c < 3; ++c) K[bb][c][c] += diag;
       }
-      if (b0 == 0) {
-        const R* S = sm.S[le][q];
+      const float* S = sm.S[le][q];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) rhs[c] += S[3 * c] * ga[0] + S[3 * c + 1] * ga[1] + S[3 * c + 2] * ga[2];
-      }
+      for (int c = 0; c < 3; ++c) rhs[c] += S[3 * c] * ga[0] + S[3 * c + 1] * ga[1] + S[3 * c + 2] * ga[2];
     }
-    const int64_t g = nh_group_index(P, et);
+    const int64_t g = group_index(P, et);
     const int64_t node = P.tconn[g * NN + a];
     const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
     const int64_t moff = P.mapoff ? P.mapoff[g] : id * NN * NN;
-    const int32_t* mp = P.node_map + moff + a * NN + b0;
+    const int32_t* mp = P.node_map + moff + a * NN;
     int64_t rb[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) rb[c] = P.row_ptr[3 * node + c];
@@ -324,27 +261,162 @@ __device__ __forceinline__ void nh_tile_body(typename NHCfg<TYPE, SLOT, PREC, SP
 #pragma unroll
         for (int cc = 0; cc < 3; ++cc) scatter_add<SC>(P.A + rb[c] + 3 * k + cc, widen(K[bb][c][cc]));
     }
-    if (b0 == 0)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) scatter_add<SC>(P.b + 3 * node + c, widen(rhs[c]));
+    for (int c = 0; c < 3; ++c) scatter_add<SC>(P.b + 3 * node + c, widen(rhs[c]));
   }
   __syncthreads();
 }
 
-template <int TYPE, int SLOT, int PREC, int SPLIT, int SC>
-__global__ void __launch_bounds__(128) k_nh_tile(const __grid_constant__ RefRule rr, const __grid_constant__ NHParams P) {
-  using Cfg = NHCfg<TYPE, SLOT, PREC, SPLIT>;
-  extern __shared__ __align__(16) unsigned char nh_smem_raw[];
-  nh_tile_body<TYPE, SLOT, PREC, SPLIT, SC>(*reinterpret_cast<typename Cfg::Smem*>(nh_smem_raw), rr, P,
-                                            (int64_t)blockIdx.x * Cfg::EPC, P.n);
+// ---------------------------------------------------------------------------
+// FP64 tiles, by node pairs
+// ---------------------------------------------------------------------------
+template <int TYPE, int SLOT>
+struct NHPairCfg : PairShape<TYPE, SLOT, 3, pair_epc(rule_nq(SLOT))> {
+  using Base = PairShape<TYPE, SLOT, 3, pair_epc(rule_nq(SLOT))>;
+  struct Smem : Base::Nodes {
+    double U[Base::EPC][Base::NN][3];
+    double G[Base::EPC][Base::NQ][Base::GS];  // g^
+    double H[Base::EPC][Base::NQ][Base::GS];  // h^
+    double C[Base::EPC][Base::NQ][2];         // mu - lam ln J, W m
+    double S[Base::EPC][Base::NQ][9];         // sqrt(W) P, row-major
+  };
+};
+
+template <class Cfg>
+__device__ __forceinline__ void nh_pair_point(typename Cfg::Smem& sm, const RefRule& rr, const NHParams& P, int le,
+                                              int q, int64_t et, const double (&J)[3][3], const double (&Ju)[3][3],
+                                              double s) {
+  constexpr int NN = Cfg::NN;
+  NHPoint r;
+  double *g = sm.G[le][q], *h = sm.H[le][q];
+  if (!nh_kinematics(P, original_id(P, et), rr.w[q], J, Ju, s, r)) {
+#pragma unroll
+    for (int k = 0; k < 3 * NN; ++k) g[k] = h[k] = 0.0;
+    sm.C[le][q][0] = sm.C[le][q][1] = 0.0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) sm.S[le][q][k] = 0.0;
+    return;
+  }
+  const double rroot = rsqrt(r.W), inv = r.W * rroot * (s * r.rdet);
+  sm.C[le][q][0] = fma(-P.lam, r.lnJ, P.mu);
+  sm.C[le][q][1] = r.W * P.mass;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      sm.S[le][q][3 * i + j] = r.WP[i][j] * rroot;
+      r.C[i][j] *= inv;
+    }
+#pragma unroll
+  for (int u = 0; u < NN; ++u) {
+    const double* d = rr.dN[q][Cfg::node_of(u)];
+    double v[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) g[3 * u + i] = v[i] = fma(d[2], r.C[i][2], fma(d[1], r.C[i][1], d[0] * r.C[i][0]));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) h[3 * u + i] = fma(r.Fit[i][2], v[2], fma(r.Fit[i][1], v[1], r.Fit[i][0] * v[0]));
+  }
 }
 
-template <int TYPE, int SLOT, int PREC, int SPLIT, int SC>
+template <class Cfg, int SC, bool DIAG>
+__device__ __forceinline__ void nh_pair_task(const typename Cfg::Smem& sm, const RefRule& rr, const NHParams& P,
+                                             int le, int u, int v) {
+  const typename Cfg::Node nu = sm.nd[le][u], nv = sm.nd[le][v];
+  int64_t kuv, kvu;
+  pair_ranks<Cfg>(sm, P, le, u, v, &kuv, &kvu);
+  const int au = Cfg::node_of(u), av = Cfg::node_of(v);
+  double M[3][3], N[3][3], dot = 0.0, mass = 0.0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) M[c][k] = N[c][k] = 0.0;
+  double f[1][3] = {{0.0, 0.0, 0.0}};
+#pragma unroll 1
+  for (int q = 0; q < Cfg::NQ; ++q) {
+    const double *a = sm.G[le][q] + 3 * u, *b = sm.G[le][q] + 3 * v;
+    const double *ha = sm.H[le][q] + 3 * u, *hb = sm.H[le][q] + 3 * v;
+    const double p = sm.C[le][q][0];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double y = p * ha[c];
+      dot = fma(a[c], b[c], dot);
+#pragma unroll
+      for (int k = DIAG ? c : 0; k < 3; ++k) {
+        M[c][k] = fma(ha[c], hb[k], M[c][k]);
+        N[c][k] = fma(y, hb[k], N[c][k]);
+      }
+    }
+    if (P.mass != 0.0) mass = fma(sm.C[le][q][1] * rr.N[q][au], rr.N[q][av], mass);
+    if constexpr (DIAG) {
+      const double* S = sm.S[le][q];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) f[0][c] = fma(S[3 * c + 2], a[2], fma(S[3 * c + 1], a[1], fma(S[3 * c], a[0], f[0][c])));
+    }
+  }
+  const double d = fma(P.mu, dot, mass);
+  double K[3][3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const bool low = DIAG && k < c;  // M and N are symmetric on the diagonal
+      const double nt = DIAG ? (low ? N[k][c] : N[c][k]) : N[k][c];
+      K[c][k] = low ? K[k][c] : fma(P.lam, M[c][k], c == k ? nt + d : nt);
+    }
+  pair_block<SC, DIAG>(P, nu, nv, kuv, kvu, K);
+  if constexpr (DIAG) pair_add<SC>(P.b + 3 * (int64_t)nu.id, 0, f);
+}
+
+template <int TYPE, int SLOT, int SC>
+__device__ __forceinline__ void nh_pair_body(typename NHPairCfg<TYPE, SLOT>::Smem& sm, const RefRule& rr,
+                                             const NHParams& P, int64_t e0, int64_t n_end) {
+  using Cfg = NHPairCfg<TYPE, SLOT>;
+  pair_nodes<Cfg>(sm, P, e0, n_end, P.u, sm.U);
+  __syncthreads();
+  field_points<TYPE, Cfg::NQ, Cfg::EPC, Cfg::THREADS>(
+      sm, rr, e0, n_end, [](int p) { return p; },
+      [&](int le, int q, int64_t et, const double(&J)[3][3], const double(&Ju)[3][3], double s) {
+        nh_pair_point<Cfg>(sm, rr, P, le, q, et, J, Ju, s);
+      });
+  __syncthreads();
+  pair_rounds<Cfg>(
+      sm, e0, n_end, [&](int le, int u, int v) { nh_pair_task<Cfg, SC, false>(sm, rr, P, le, u, v); },
+      [&](int le, int u) { nh_pair_task<Cfg, SC, true>(sm, rr, P, le, u, u); });
+  __syncthreads();
+}
+
+// the tile of an element type in a precision
+template <int TYPE, int SLOT, int PREC>
+struct NHTile {
+  using Cfg = NHCfg<TYPE, SLOT>;
+  template <int SC>
+  __device__ static __forceinline__ void run(typename Cfg::Smem& sm, const RefRule& rr, const NHParams& P, int64_t e0) {
+    nh_tile_body<TYPE, SLOT, SC>(sm, rr, P, e0, P.n);
+  }
+};
+template <int TYPE, int SLOT>
+struct NHTile<TYPE, SLOT, FEA_FP64> {
+  using Cfg = NHPairCfg<TYPE, SLOT>;
+  template <int SC>
+  __device__ static __forceinline__ void run(typename Cfg::Smem& sm, const RefRule& rr, const NHParams& P, int64_t e0) {
+    nh_pair_body<TYPE, SLOT, SC>(sm, rr, P, e0, P.n);
+  }
+};
+
+template <int TYPE, int SLOT, int PREC, int SC>
+__global__ void __launch_bounds__(128, PREC == FEA_FP64 ? 0 : 4) k_nh_tile(const __grid_constant__ RefRule rr, const __grid_constant__ NHParams P) {
+  using T = NHTile<TYPE, SLOT, PREC>;
+  extern __shared__ __align__(16) unsigned char nh_smem_raw[];
+  T::template run<SC>(*reinterpret_cast<typename T::Cfg::Smem*>(nh_smem_raw), rr, P,
+                      (int64_t)blockIdx.x * T::Cfg::EPC);
+}
+
+template <int TYPE, int SLOT, int PREC, int SC>
 static int launch_nh(const NHParams& P, cudaStream_t s) {
-  using Cfg = NHCfg<TYPE, SLOT, PREC, SPLIT>;
+  using Cfg = typename NHTile<TYPE, SLOT, PREC>::Cfg;
   constexpr size_t smem = sizeof(typename Cfg::Smem);
   static_assert(smem <= 227 * 1024, "finite-strain tile exceeds shared memory");
-  auto kern = k_nh_tile<TYPE, SLOT, PREC, SPLIT, SC>;
+  auto kern = k_nh_tile<TYPE, SLOT, PREC, SC>;
   if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kern<<<grid_for(P.n, Cfg::EPC), Cfg::THREADS, smem, s>>>(host_rule(SLOT), P);
   FEA_CUDA(cudaGetLastError());
@@ -353,12 +425,11 @@ static int launch_nh(const NHParams& P, cudaStream_t s) {
 
 template <int PREC, int SC>
 static int launch_nh_type(int type, const NHParams& P, cudaStream_t s) {
-  constexpr int S2 = PREC == FEA_FP64 ? 2 : 1;  // FP64 splits the columns of hex8 / prism6 over two lanes
   switch (type) {
-    case FEA_TET4: return launch_nh<FEA_TET4, kRuleTet4, PREC, 1, SC>(P, s);
-    case FEA_PYR5: return launch_nh<FEA_PYR5, kRulePyr8, PREC, 1, SC>(P, s);
-    case FEA_PRISM6: return launch_nh<FEA_PRISM6, kRulePrism6, PREC, S2, SC>(P, s);
-    default: return launch_nh<FEA_HEX8, kRuleHex8, PREC, S2, SC>(P, s);
+    case FEA_TET4: return launch_nh<FEA_TET4, kRuleTet4, PREC, SC>(P, s);
+    case FEA_PYR5: return launch_nh<FEA_PYR5, kRulePyr8, PREC, SC>(P, s);
+    case FEA_PRISM6: return launch_nh<FEA_PRISM6, kRulePrism6, PREC, SC>(P, s);
+    default: return launch_nh<FEA_HEX8, kRuleHex8, PREC, SC>(P, s);
   }
 }
 
