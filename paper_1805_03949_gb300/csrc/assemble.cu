@@ -22,6 +22,7 @@
 #include <mutex>
 #include <type_traits>
 
+#include "coop_scatter.cuh"
 #include "element.cuh"
 #include "fea_internal.cuh"
 #include "pair_tile.cuh"
@@ -186,7 +187,7 @@ const RefRule& host_rule(int slot) {
 template <int OP, int NN, int NQ, int EPC>
 struct TileSmem {
   double X[EPC][NN][3];     // node coordinates
-  float G[EPC][NQ][NN][3];  // physical gradients
+  float G[EPC][NQ][grad_stride(NN)];  // physical gradients [point][node][component]
   float S[EPC][NQ];         // w detJ k(x_q)
   float W[EPC][NQ];         // w detJ
   int flag[EPC];            // adaptive mode: element is distorted -> FP64 geometry
@@ -210,7 +211,7 @@ __device__ __forceinline__ void geometry_store(Smem& sm, const RefRule& rr, int 
   for (int a = 0; a < NN; ++a)
 #pragma unroll
     for (int i = 0; i < 3; ++i)
-      sm.G[le][q][a][i] = (rr.dNf[q][a][0] * Cf[i][0] + rr.dNf[q][a][1] * Cf[i][1] + rr.dNf[q][a][2] * Cf[i][2]) * inv;
+      sm.G[le][q][3 * a + i] = (rr.dNf[q][a][0] * Cf[i][0] + rr.dNf[q][a][1] * Cf[i][1] + rr.dNf[q][a][2] * Cf[i][2]) * inv;
   const float wdf = rr.wf[q] * detf * (float)(1.0 / (s * s * s));
   sm.W[le][q] = wdf;
   if constexpr (OP == FEA_OP_DIFFUSION) {
@@ -311,7 +312,7 @@ __device__ __forceinline__ bool geometry_fp32(Smem& sm, const RefRule& rr, int l
   for (int a = 0; a < NN; ++a)
 #pragma unroll
     for (int i = 0; i < 3; ++i)
-      sm.G[le][q][a][i] = (rr.dNf[q][a][0] * C[i][0] + rr.dNf[q][a][1] * C[i][1] + rr.dNf[q][a][2] * C[i][2]) * inv;
+      sm.G[le][q][3 * a + i] = (rr.dNf[q][a][0] * C[i][0] + rr.dNf[q][a][1] * C[i][1] + rr.dNf[q][a][2] * C[i][2]) * inv;
   const float wd = rr.wf[q] * det;
   sm.W[le][q] = wd;
   if constexpr (OP == FEA_OP_DIFFUSION) {
@@ -450,7 +451,7 @@ __device__ __forceinline__ void tile_geometry(typename Cfg::Smem& sm, const RefR
         for (int a = 0; a < NN; ++a)
 #pragma unroll
           for (int i = 0; i < 3; ++i)
-            sm.G[le][q][a][i] =
+            sm.G[le][q][3 * a + i] =
                 (rr.dNf[q][a][0] * Cf[i][0] + rr.dNf[q][a][1] * Cf[i][1] + rr.dNf[q][a][2] * Cf[i][2]) * inv;
         const float wdf = rr.wf[q] * detf;
         sm.W[le][q] = wdf;
@@ -514,12 +515,13 @@ __device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const Re
 #pragma unroll 1
   for (int q = 0; q < NQ; ++q) {
     const R s = sm.S[le][q];
-    const R ga0 = sm.G[le][q][a][0], ga1 = sm.G[le][q][a][1], ga2 = sm.G[le][q][a][2];
+    const R* ga = sm.G[le][q] + 3 * a;
+    const R ga0 = ga[0], ga1 = ga[1], ga2 = ga[2];
     if constexpr (OP == FEA_OP_DIFFUSION) {
       const R sa0 = s * ga0, sa1 = s * ga1, sa2 = s * ga2;
 #pragma unroll
       for (int bb = 0; bb < NB; ++bb) {
-        const R* gb = sm.G[le][q][bb];
+        const R* gb = sm.G[le][q] + 3 * bb;
         K[bb][0][0] += sa0 * gb[0] + sa1 * gb[1] + sa2 * gb[2];
       }
     } else {
@@ -527,7 +529,8 @@ __device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const Re
       const R gm[3] = {s * mu * ga0, s * mu * ga1, s * mu * ga2};
 #pragma unroll
       for (int bb = 0; bb < NB; ++bb) {
-        const R gb[3] = {sm.G[le][q][bb][0], sm.G[le][q][bb][1], sm.G[le][q][bb][2]};
+        const R* g = sm.G[le][q] + 3 * bb;
+        const R gb[3] = {g[0], g[1], g[2]};
         const R dot = gm[0] * gb[0] + gm[1] * gb[1] + gm[2] * gb[2];
 #pragma unroll
         for (int c = 0; c < 3; ++c)
@@ -546,34 +549,10 @@ __device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const Re
   }
 }
 
-// Warp-cooperative reduction of FP32 elasticity row blocks.  A lane's row
-// block holds, for each row c and column node b, three consecutive entries of
-// A (24 bytes); one lane per entry scatters each warp-wide reduction over 32
-// rows, while three neighbouring lanes on one 24-byte run and ten runs from
-// one or two rows make each reduction touch about a third of the sectors
-// (measured on GB300 with A in L2: 192 G reductions/s scattered, 443 G/s in
-// runs of three).  The lanes hand their entries to the warp through the
-// gradient table's shared memory, which row_block no longer needs: per warp
-// the row starts (rbs), the column positions (ks, -1 for an idle lane) and PB
-// columns' entries at a time (vals).
+// the cooperative scatter of a tile, staged in the gradients of each warp's elements
 template <class Cfg, int SC>
-struct CoopScatter {
-  using Smem = typename Cfg::Smem;
-  static constexpr int NB = Cfg::NB;
-  static constexpr size_t kWarpBytes = sizeof(((Smem*)nullptr)->G) / Cfg::WARPS;
-  static constexpr size_t kValsOff = 256 + 4 * 32 * NB;  // after rbs[32] and ks[32][NB]
-  static constexpr int pb() {
-    for (int p = NB; p > 0; --p)
-      if (NB % p == 0 && kValsOff + 4 * 32 * 3 * p <= kWarpBytes) return p;
-    return 0;
-  }
-  static constexpr int PB = pb();
-  // hex8 with the 2x2x2 rule (PB = 4, 16-byte staging stores) is the tile it
-  // serves; staged in pairs of columns, the tet4 items of the 256-mesh batch
-  // made it slower (17.97 against 17.09 ms)
-  static constexpr bool kOn = SC == FEA_SCATTER_ATOMIC && Cfg::D == 3 && PB > 0 && kWarpBytes % 16 == 0 &&
-                              (3 * PB) % 4 == 0;
-};
+using TileCoop =
+    CoopScatter<Cfg::NN, Cfg::D == 3 ? SC : (int)FEA_SCATTER_COLOR, sizeof(((typename Cfg::Smem*)nullptr)->G) / Cfg::WARPS>;
 
 // One tile of EPC elements starting at launch index e0 (elements at or past
 // n_end are skipped): integrate, then scatter each row block,
@@ -592,68 +571,14 @@ __device__ __forceinline__ void tile_body(typename TileCfg<TYPE, SLOT, OP>::Smem
   const int le = warp * EPW + lw;
   const int64_t et = e0 + le;
   if constexpr (COOP) {
-    static_assert(CoopScatter<Cfg, SC>::kOn, "no cooperative scatter for this tile");
-    using CS = CoopScatter<Cfg, SC>;
-    constexpr int PB = CS::PB;
+    using CS = TileCoop<Cfg, SC>;
+    static_assert(CS::kOn, "no cooperative scatter for this tile");
     static_assert(offsetof(typename Cfg::Smem, G) % 16 == 0, "staged entries need 16-byte rows");
     const bool active = lw < EPW && et < n_end;
     const int a = lane % LPE;
     R K[NB][D][D], rhs[D];
-    int64_t rb[D] = {};
-    int64_t node = 0;
-    const int32_t* mp = nullptr;
-    if (active) {
-      row_block<Cfg, OP>(sm, rr, P, le, a, K, rhs);
-      const int64_t g = group_index(P, et);
-      node = P.tconn[g * NN + a];
-      const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
-      mp = P.node_map + (P.mapoff ? P.mapoff[g] : id * NN * NN) + a * NN;
-#pragma unroll
-      for (int c = 0; c < D; ++c) rb[c] = P.row_ptr[D * node + c];
-    }
-    __syncthreads();  // every row_block has read the gradient table
-    unsigned char* wb = reinterpret_cast<unsigned char*>(&sm.G[0][0][0][0]) + warp * CS::kWarpBytes;
-    int64_t* rbs = reinterpret_cast<int64_t*>(wb);
-    int32_t* ks = reinterpret_cast<int32_t*>(wb + 256);
-    float* vals = reinterpret_cast<float*>(wb + CS::kValsOff);
-#pragma unroll
-    for (int bb = 0; bb < NB; ++bb) ks[lane * NB + bb] = active ? mp[bb] : -1;
-    // run j of a round: lanes 3j .. 3j+2 (lanes 30 and 31 rest)
-    const int run = lane / 3, m = lane - 3 * run;
-    constexpr int kRuns = 32 * PB, kRounds = (kRuns + 9) / 10;
-#pragma unroll
-    for (int c = 0; c < D; ++c) {
-      __syncwarp();
-      rbs[lane] = rb[c];
-#pragma unroll
-      for (int part = 0; part < NB / PB; ++part) {
-        __syncwarp();
-        float4* v4 = reinterpret_cast<float4*>(vals + lane * PB * 3);
-#pragma unroll
-        for (int i = 0; i < 3 * PB / 4; ++i) {
-          float t[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int f = 4 * i + u;
-            t[u] = K[part * PB + f / 3][c][f % 3];
-          }
-          v4[i] = make_float4(t[0], t[1], t[2], t[3]);
-        }
-        __syncwarp();
-#pragma unroll 2
-        for (int r = 0; r < kRounds; ++r) {
-          const int ch = 10 * r + run;  // run ch: lane ch / PB, column part * PB + ch % PB
-          if (run < 10 && ch < kRuns) {
-            const int s = ch / PB, j = ch - PB * s;
-            const int32_t k = ks[s * NB + part * PB + j];
-            if (k >= 0) red_add(P.A + rbs[s] + 3 * (int64_t)k + m, widen(vals[3 * ch + m]));
-          }
-        }
-      }
-    }
-    if (active)
-#pragma unroll
-      for (int c = 0; c < D; ++c) red_add(P.b + D * node + c, widen(rhs[c]));
+    if (active) row_block<Cfg, OP>(sm, rr, P, le, a, K, rhs);
+    CS::run(reinterpret_cast<unsigned char*>(sm.G[warp * EPW]), P, active, active ? group_index(P, et) : 0, a, K, rhs);
     __syncthreads();
     return;
   }
@@ -719,10 +644,10 @@ struct Tile {
   template <int SC, bool COOP>
   __device__ static __forceinline__ void run(unsigned char* raw, const RefRule& rr, const AsmParams& P, int64_t e0,
                                              int64_t n_end) {
-    tile_body<TYPE, SLOT, OP, SC, COOP && CoopScatter<Cfg, SC>::kOn>(*reinterpret_cast<Smem*>(raw), rr, P, e0, n_end);
+    tile_body<TYPE, SLOT, OP, SC, COOP && TileCoop<Cfg, SC>::kOn>(*reinterpret_cast<Smem*>(raw), rr, P, e0, n_end);
   }
   // CTAs per SM its own kernel is compiled for (0: the compiler's choice)
-  static constexpr int min_blocks(int sc) { return sc == FEA_SCATTER_ATOMIC && CoopScatter<Cfg, FEA_SCATTER_ATOMIC>::kOn ? 4 : 0; }
+  static constexpr int min_blocks(int sc) { return sc == FEA_SCATTER_ATOMIC && TileCoop<Cfg, FEA_SCATTER_ATOMIC>::kOn ? 4 : 0; }
 };
 template <int TYPE, int SLOT, int OP>
 struct Tile<TYPE, SLOT, OP, FEA_FP64> {

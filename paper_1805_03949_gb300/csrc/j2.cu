@@ -39,6 +39,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "coop_scatter.cuh"
 #include "element.cuh"
 #include "fea_internal.cuh"
 #include "pairs.cuh"
@@ -81,8 +82,8 @@ struct J2Cfg {
     double U[EPC][NN][3];
   };
   struct Smem : Fields {
-    float G[EPC][NQ][NN][3];  // grad N_a
-    float H[EPC][NQ][NN][3];  // h_a = n grad N_a
+    float G[EPC][NQ][grad_stride(NN)];  // grad N_a [point][node][component]
+    float H[EPC][NQ][grad_stride(NN)];  // h_a = n grad N_a
     float C[EPC][NQ][4];      // W, W lam', W mu', W beta
     float S[EPC][NQ][6];      // W sigma (xx, yy, zz, xy, yz, xz)
   };
@@ -245,7 +246,7 @@ __device__ __forceinline__ void j2_point(Smem& sm, const RefRule& rr, const J2Pa
 #pragma unroll
       for (int a = 0; a < NN; ++a)
 #pragma unroll
-        for (int i = 0; i < 3; ++i) sm.G[le][q][a][i] = sm.H[le][q][a][i] = 0.0f;
+        for (int i = 0; i < 3; ++i) sm.G[le][q][3 * a + i] = sm.H[le][q][3 * a + i] = 0.0f;
     }
     return;
   }
@@ -290,12 +291,13 @@ __device__ __forceinline__ void j2_point(Smem& sm, const RefRule& rr, const J2Pa
 #pragma unroll
     for (int a = 0; a < NN; ++a) {
       const float g0 = gt[a][0], g1 = gt[a][1], g2 = gt[a][2];
-      sm.G[le][q][a][0] = g0;
-      sm.G[le][q][a][1] = g1;
-      sm.G[le][q][a][2] = g2;
-      sm.H[le][q][a][0] = n[0] * g0 + n[3] * g1 + n[5] * g2;
-      sm.H[le][q][a][1] = n[3] * g0 + n[1] * g1 + n[4] * g2;
-      sm.H[le][q][a][2] = n[5] * g0 + n[4] * g1 + n[2] * g2;
+      float *g = sm.G[le][q] + 3 * a, *h = sm.H[le][q] + 3 * a;
+      g[0] = g0;
+      g[1] = g1;
+      g[2] = g2;
+      h[0] = n[0] * g0 + n[3] * g1 + n[5] * g2;
+      h[1] = n[3] * g0 + n[1] * g1 + n[4] * g2;
+      h[2] = n[5] * g0 + n[4] * g1 + n[2] * g2;
     }
   }
 }
@@ -338,26 +340,28 @@ __device__ __forceinline__ void j2_tile_body(Smem& sm, const RefRule& rr, const 
     const int lw = lane / LPE;
     const int le = warp * EPW + lw;
     const int64_t et = e0 + le;
-    if (lw < EPW && et < n_end) {
-      const int a = lane % LPE;
-      float K[NB][3][3], rhs[3] = {0.0f, 0.0f, 0.0f};
+    const bool active = lw < EPW && et < n_end;
+    const int a = lane % LPE;
+    float K[NB][3][3], rhs[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
-      for (int bb = 0; bb < NB; ++bb)
+    for (int bb = 0; bb < NB; ++bb)
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
+      for (int c = 0; c < 3; ++c)
 #pragma unroll
-          for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] = 0.0f;
+        for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] = 0.0f;
+    if (active) {
 #pragma unroll 1
       for (int q = 0; q < NQ; ++q) {
         const float wl = sm.C[le][q][1], wm = sm.C[le][q][2], wb = sm.C[le][q][3];
-        const float ga[3] = {sm.G[le][q][a][0], sm.G[le][q][a][1], sm.G[le][q][a][2]};
+        const float *pg = sm.G[le][q], *ph = sm.H[le][q];
+        const float ga[3] = {pg[3 * a], pg[3 * a + 1], pg[3 * a + 2]};
         const float gl[3] = {wl * ga[0], wl * ga[1], wl * ga[2]};
         const float gm[3] = {wm * ga[0], wm * ga[1], wm * ga[2]};
-        const float hb[3] = {wb * sm.H[le][q][a][0], wb * sm.H[le][q][a][1], wb * sm.H[le][q][a][2]};
+        const float hb[3] = {wb * ph[3 * a], wb * ph[3 * a + 1], wb * ph[3 * a + 2]};
 #pragma unroll
         for (int bb = 0; bb < NB; ++bb) {
-          const float gb[3] = {sm.G[le][q][bb][0], sm.G[le][q][bb][1], sm.G[le][q][bb][2]};
-          const float hh[3] = {sm.H[le][q][bb][0], sm.H[le][q][bb][1], sm.H[le][q][bb][2]};
+          const float gb[3] = {pg[3 * bb], pg[3 * bb + 1], pg[3 * bb + 2]};
+          const float hh[3] = {ph[3 * bb], ph[3 * bb + 1], ph[3 * bb + 2]};
           const float dot = gm[0] * gb[0] + gm[1] * gb[1] + gm[2] * gb[2];
 #pragma unroll
           for (int c = 0; c < 3; ++c)
@@ -371,6 +375,13 @@ __device__ __forceinline__ void j2_tile_body(Smem& sm, const RefRule& rr, const 
         rhs[1] += S[3] * ga[0] + S[1] * ga[1] + S[4] * ga[2];
         rhs[2] += S[5] * ga[0] + S[4] * ga[1] + S[2] * ga[2];
       }
+    }
+    using CS = CoopScatter<NN, SC, sizeof(sm.G) / Cfg::WARPS>;
+    if constexpr (CS::kOn) {
+      // staged in the gradients of the warp's own elements
+      static_assert(sizeof(typename Cfg::Fields) % 16 == 0, "staged entries need 16-byte rows");
+      CS::run(reinterpret_cast<unsigned char*>(sm.G[warp * EPW]), P, active, active ? group_index(P, et) : 0, a, K, rhs);
+    } else if (active) {
       const int64_t g = group_index(P, et);
       const int64_t node = P.tconn[g * NN + a];
       const int64_t id = P.ids ? (int64_t)P.ids[g] : g;

@@ -29,9 +29,11 @@
 // 24 products per pair and point where a row block took 28 per ordered pair.
 // 65,559 hex8, FP64, one GB300: 2.81 -> 1.29 ms.
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <type_traits>
 
+#include "coop_scatter.cuh"
 #include "element.cuh"
 #include "fea_internal.cuh"
 #include "pairs.cuh"
@@ -59,8 +61,8 @@ struct NHCfg {
   struct Smem {
     double X[EPC][NN][3];
     double U[EPC][NN][3];
-    float G[EPC][NQ][NN][3];  // g_a = grad0 N_a
-    float H[EPC][NQ][NN][3];  // h_a = F^-T g_a
+    float G[EPC][NQ][grad_stride(NN)];  // g_a = grad0 N_a [point][node][component]
+    float H[EPC][NQ][grad_stride(NN)];  // h_a = F^-T g_a
     float C[EPC][NQ][4];      // W mu, W lam, W (mu - lam ln J), W m
     float S[EPC][NQ][9];      // W P, row-major
   };
@@ -126,7 +128,7 @@ __device__ __forceinline__ void nh_point(typename Cfg::Smem& sm, const RefRule& 
 #pragma unroll
     for (int a = 0; a < NN; ++a)
 #pragma unroll
-      for (int i = 0; i < 3; ++i) sm.G[le][q][a][i] = sm.H[le][q][a][i] = 0.0f;
+      for (int i = 0; i < 3; ++i) sm.G[le][q][3 * a + i] = sm.H[le][q][3 * a + i] = 0.0f;
     return;
   }
   sm.C[le][q][0] = f64_to_f32_rn(r.W * P.mu);
@@ -170,11 +172,12 @@ __device__ __forceinline__ void nh_point(typename Cfg::Smem& sm, const RefRule& 
 #pragma unroll
   for (int a = 0; a < NN; ++a) {
     const float g0 = gt[a][0], g1 = gt[a][1], g2 = gt[a][2];
-    sm.G[le][q][a][0] = g0;
-    sm.G[le][q][a][1] = g1;
-    sm.G[le][q][a][2] = g2;
+    float *g = sm.G[le][q] + 3 * a, *h = sm.H[le][q] + 3 * a;
+    g[0] = g0;
+    g[1] = g1;
+    g[2] = g2;
 #pragma unroll
-    for (int i = 0; i < 3; ++i) sm.H[le][q][a][i] = Ft[i][0] * g0 + Ft[i][1] * g1 + Ft[i][2] * g2;
+    for (int i = 0; i < 3; ++i) h[i] = Ft[i][0] * g0 + Ft[i][1] * g1 + Ft[i][2] * g2;
   }
 }
 
@@ -212,27 +215,29 @@ __device__ __forceinline__ void nh_tile_body(typename NHCfg<TYPE, SLOT>::Smem& s
   const int lw = lane / LPE;
   const int le = warp * EPW + lw;
   const int64_t et = e0 + le;
-  if (lw < EPW && et < n_end) {
-    const int a = lane % LPE;
-    float K[NB][3][3], rhs[3] = {0.0f, 0.0f, 0.0f};
+  const bool active = lw < EPW && et < n_end;
+  const int a = lane % LPE;
+  float K[NB][3][3], rhs[3] = {0.0f, 0.0f, 0.0f};
 #pragma unroll
-    for (int bb = 0; bb < NB; ++bb)
+  for (int bb = 0; bb < NB; ++bb)
 #pragma unroll
-      for (int c = 0; c < 3; ++c)
+    for (int c = 0; c < 3; ++c)
 #pragma unroll
-        for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] = 0.0f;
+      for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] = 0.0f;
+  if (active) {
 #pragma unroll 1
     for (int q = 0; q < NQ; ++q) {
       const float wm = sm.C[le][q][0], wl = sm.C[le][q][1], wp = sm.C[le][q][2], wn = sm.C[le][q][3];
-      const float ga[3] = {sm.G[le][q][a][0], sm.G[le][q][a][1], sm.G[le][q][a][2]};
+      const float *pg = sm.G[le][q], *ph = sm.H[le][q];
+      const float ga[3] = {pg[3 * a], pg[3 * a + 1], pg[3 * a + 2]};
       const float gm[3] = {wm * ga[0], wm * ga[1], wm * ga[2]};
-      const float hl[3] = {wl * sm.H[le][q][a][0], wl * sm.H[le][q][a][1], wl * sm.H[le][q][a][2]};
-      const float hp[3] = {wp * sm.H[le][q][a][0], wp * sm.H[le][q][a][1], wp * sm.H[le][q][a][2]};
+      const float hl[3] = {wl * ph[3 * a], wl * ph[3 * a + 1], wl * ph[3 * a + 2]};
+      const float hp[3] = {wp * ph[3 * a], wp * ph[3 * a + 1], wp * ph[3 * a + 2]};
       const float mn = wn * rr.Nf[q][a];
 #pragma unroll
       for (int bb = 0; bb < NB; ++bb) {
-        const float gb[3] = {sm.G[le][q][bb][0], sm.G[le][q][bb][1], sm.G[le][q][bb][2]};
-        const float hb[3] = {sm.H[le][q][bb][0], sm.H[le][q][bb][1], sm.H[le][q][bb][2]};
+        const float gb[3] = {pg[3 * bb], pg[3 * bb + 1], pg[3 * bb + 2]};
+        const float hb[3] = {ph[3 * bb], ph[3 * bb + 1], ph[3 * bb + 2]};
         const float diag = gm[0] * gb[0] + gm[1] * gb[1] + gm[2] * gb[2] + mn * rr.Nf[q][bb];
 #pragma unroll
         for (int c = 0; c < 3; ++c)
@@ -245,6 +250,13 @@ __device__ __forceinline__ void nh_tile_body(typename NHCfg<TYPE, SLOT>::Smem& s
 #pragma unroll
       for (int c = 0; c < 3; ++c) rhs[c] += S[3 * c] * ga[0] + S[3 * c + 1] * ga[1] + S[3 * c + 2] * ga[2];
     }
+  }
+  using CS = CoopScatter<NN, SC, sizeof(sm.G) / Cfg::WARPS>;
+  if constexpr (CS::kOn) {
+    // staged in the gradients of the warp's own elements
+    static_assert(offsetof(typename Cfg::Smem, G) % 16 == 0, "staged entries need 16-byte rows");
+    CS::run(reinterpret_cast<unsigned char*>(sm.G[warp * EPW]), P, active, active ? group_index(P, et) : 0, a, K, rhs);
+  } else if (active) {
     const int64_t g = group_index(P, et);
     const int64_t node = P.tconn[g * NN + a];
     const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
