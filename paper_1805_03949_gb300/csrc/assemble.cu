@@ -184,6 +184,16 @@ const RefRule& host_rule(int slot) {
 // ---------------------------------------------------------------------------
 // device
 // ---------------------------------------------------------------------------
+// staging of the cooperative scatter (three dofs per node)
+template <int OP, int NN, int WARPS>
+struct TileStage {
+  using CS = CoopScatter<NN, FEA_SCATTER_ATOMIC>;
+  alignas(16) float vals[WARPS][CS::kVals];
+  typename CS::Rows rows[WARPS];
+};
+template <int NN, int WARPS>
+struct TileStage<FEA_OP_DIFFUSION, NN, WARPS> {};
+
 template <int OP, int NN, int NQ, int EPC>
 struct TileSmem {
   double X[EPC][NN][3];     // node coordinates
@@ -191,15 +201,16 @@ struct TileSmem {
   float S[EPC][NQ];         // w detJ k(x_q)
   float W[EPC][NQ];         // w detJ
   int flag[EPC];            // adaptive mode: element is distorted -> FP64 geometry
+  TileStage<OP, NN, 4> stage;
 };
 
 // Tile values of point q from the cofactors C' and det' of the FP64 Jacobian
 // J' = s J (s a power of two): det J = det'/s^3, grad N_a = J^{-T} grad_xi N_a
 // = s C' grad_xi N_a / det'.  The cofactors and the determinant are rounded
 // once and the gradients formed in FP32.
-template <int OP, int NN, typename Smem>
+template <int OP, int NN, typename Smem, class Params>
 __device__ __forceinline__ void geometry_store(Smem& sm, const RefRule& rr, int le, int q, const double (&C)[3][3],
-                                               double det, double s, double xq, const AsmParams& P) {
+                                               double det, double s, double xq, Params& P) {
   float Cf[3][3];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
@@ -222,9 +233,9 @@ __device__ __forceinline__ void geometry_store(Smem& sm, const RefRule& rr, int 
   }
 }
 
-template <int OP, int NN, typename Smem>
+template <int OP, int NN, typename Smem, class Params>
 __device__ __forceinline__ void geometry_finish(Smem& sm, const RefRule& rr, int le, int q, int64_t elem_id,
-                                                double (&J)[3][3], double s, double xq, const AsmParams& P) {
+                                                double (&J)[3][3], double s, double xq, Params& P) {
   double C[3][3];
   cofactors(J, C);
   const double det = J[0][0] * C[0][0] + J[0][1] * C[0][1] + J[0][2] * C[0][2];
@@ -234,9 +245,9 @@ __device__ __forceinline__ void geometry_finish(Smem& sm, const RefRule& rr, int
 
 // FP64 geometry of point q of element le from the combinations RefMap::prep
 // left in sm.X; with pyramids of point q + 4 too, which shares the Jacobian
-template <int OP, int TYPE, int NN, typename Smem>
+template <int OP, int TYPE, int NN, typename Smem, class Params>
 __device__ __forceinline__ void geometry_fp64(Smem& sm, const RefRule& rr, int le, int q, int64_t elem_id,
-                                              const AsmParams& P) {
+                                              Params& P) {
   using Map = RefMap<TYPE>;
   double J[3][3], C[3][3];
   Map::jac(sm.X[le], rr.m[q], J);
@@ -252,9 +263,9 @@ __device__ __forceinline__ void geometry_fp64(Smem& sm, const RefRule& rr, int l
 }
 
 // FP64 geometry of point q of a distorted hex8 from its node coordinates
-template <int OP, typename Smem>
+template <int OP, typename Smem, class Params>
 __device__ __forceinline__ void geometry_fp64_hex(Smem& sm, const RefRule& rr, int le, int q, int64_t elem_id,
-                                                  const AsmParams& P) {
+                                                  Params& P) {
   double J[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
   double xq = sm.X[le][0][0];
 #pragma unroll
@@ -276,8 +287,8 @@ __device__ __forceinline__ void geometry_fp64_hex(Smem& sm, const RefRule& rr, i
 // FP32 geometry on coordinates relative to node 0; returns false when the
 // element must take the FP64 path (distorted: Frobenius condition number of J
 // above FEA_KAPPA_FP64, or a determinant FP32 cannot trust).
-template <int OP, int NN, typename Smem>
-__device__ __forceinline__ bool geometry_fp32(Smem& sm, const RefRule& rr, int le, int q, const AsmParams& P) {
+template <int OP, int NN, typename Smem, class Params>
+__device__ __forceinline__ bool geometry_fp32(Smem& sm, const RefRule& rr, int le, int q, Params& P) {
   float J[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
   float xr = 0.0f;
 #pragma unroll
@@ -335,15 +346,15 @@ struct TileCfg {
   static constexpr int WARPS = 4;
   static constexpr int THREADS = 32 * WARPS;
   static constexpr int EPC = EPW * WARPS;       // elements per CTA
-  static constexpr int NB = NN;                 // columns per lane
+  static constexpr int NB = column_group(NN, D);  // columns per lane at a time
   static constexpr bool kModal = TYPE == FEA_HEX8 && SLOT == kRuleHex8;
   static_assert(!kModal || (EPC * 8 % 32 == 0 && EPC * 8 <= THREADS), "modal hex geometry needs whole warps");
   using Smem = TileSmem<OP, NN, NQ, EPC>;
 };
 
 // phases 0 and 1 for the tile of elements [e0, e0 + EPC)
-template <class Cfg, int OP>
-__device__ __forceinline__ void tile_geometry(typename Cfg::Smem& sm, const RefRule& rr, const AsmParams& P,
+template <class Cfg, int OP, class Params>
+__device__ __forceinline__ void tile_geometry(typename Cfg::Smem& sm, const RefRule& rr, Params& P,
                                               int64_t e0, int64_t n_end) {
   constexpr int NN = Cfg::NN, NQ = Cfg::NQ, EPC = Cfg::EPC;
   constexpr bool kModal = Cfg::kModal;
@@ -496,10 +507,11 @@ __device__ __forceinline__ void tile_geometry(typename Cfg::Smem& sm, const RefR
   __syncthreads();
 }
 
-// phase 2: row block of node a of element le, and its RHS
-template <class Cfg, int OP>
-__device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const RefRule& rr, const AsmParams& P,
-                                          int le, int a, float (&K)[Cfg::NB][Cfg::D][Cfg::D],
+// phase 2: columns b0 .. b0 + NB of the row block of node a of element le,
+// and with the first columns its RHS
+template <class Cfg, int OP, class Params>
+__device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const RefRule& rr, Params& P,
+                                          int le, int a, int b0, float (&K)[Cfg::NB][Cfg::D][Cfg::D],
                                           float (&rhs)[Cfg::D]) {
   using R = float;
   constexpr int NB = Cfg::NB, D = Cfg::D, NQ = Cfg::NQ;
@@ -509,9 +521,15 @@ __device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const Re
     for (int c = 0; c < D; ++c)
 #pragma unroll
       for (int cc = 0; cc < D; ++cc) K[bb][c][cc] = R(0);
+  R lam = R(0), mu = R(0), src[D];
+  if constexpr (OP == FEA_OP_DIFFUSION) {
+    src[0] = (R)P.src;
+  } else {
+    lam = (R)P.lam;
+    mu = (R)P.mu;
 #pragma unroll
-  for (int c = 0; c < D; ++c) rhs[c] = R(0);
-  const R lam = (R)P.lam, mu = (R)P.mu;
+    for (int c = 0; c < 3; ++c) src[c] = (R)P.f[c];
+  }
 #pragma unroll 1
   for (int q = 0; q < NQ; ++q) {
     const R s = sm.S[le][q];
@@ -521,7 +539,7 @@ __device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const Re
       const R sa0 = s * ga0, sa1 = s * ga1, sa2 = s * ga2;
 #pragma unroll
       for (int bb = 0; bb < NB; ++bb) {
-        const R* gb = sm.G[le][q] + 3 * bb;
+        const R* gb = sm.G[le][q] + 3 * (b0 + bb);
         K[bb][0][0] += sa0 * gb[0] + sa1 * gb[1] + sa2 * gb[2];
       }
     } else {
@@ -529,7 +547,7 @@ __device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const Re
       const R gm[3] = {s * mu * ga0, s * mu * ga1, s * mu * ga2};
 #pragma unroll
       for (int bb = 0; bb < NB; ++bb) {
-        const R* g = sm.G[le][q] + 3 * bb;
+        const R* g = sm.G[le][q] + 3 * (b0 + bb);
         const R gb[3] = {g[0], g[1], g[2]};
         const R dot = gm[0] * gb[0] + gm[1] * gb[1] + gm[2] * gb[2];
 #pragma unroll
@@ -540,27 +558,21 @@ __device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const Re
         for (int c = 0; c < 3; ++c) K[bb][c][c] += dot;
       }
     }
-    const R wN = sm.W[le][q] * rr.Nf[q][a];
-    if constexpr (OP == FEA_OP_DIFFUSION)
-      rhs[0] += wN * (R)P.src;
-    else
+    if (b0 == 0) {
+      const R wN = sm.W[le][q] * rr.Nf[q][a];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) rhs[c] += wN * (R)P.f[c];
+      for (int c = 0; c < D; ++c) rhs[c] += wN * src[c];
+    }
   }
 }
-
-// the cooperative scatter of a tile, staged in the gradients of each warp's elements
-template <class Cfg, int SC>
-using TileCoop =
-    CoopScatter<Cfg::NN, Cfg::D == 3 ? SC : (int)FEA_SCATTER_COLOR, sizeof(((typename Cfg::Smem*)nullptr)->G) / Cfg::WARPS>;
 
 // One tile of EPC elements starting at launch index e0 (elements at or past
 // n_end are skipped): integrate, then scatter each row block,
 // warp-cooperatively when COOP is set.  Every thread of the CTA must call it;
 // it ends with the shared memory free.
-template <int TYPE, int SLOT, int OP, int SC, bool COOP = false>
+template <int TYPE, int SLOT, int OP, int SC, bool COOP, class Params>
 __device__ __forceinline__ void tile_body(typename TileCfg<TYPE, SLOT, OP>::Smem& sm, const RefRule& rr,
-                                          const AsmParams& P, int64_t e0, int64_t n_end) {
+                                          Params& P, int64_t e0, int64_t n_end) {
   using Cfg = TileCfg<TYPE, SLOT, OP>;
   using R = float;
   constexpr int NN = Cfg::NN, D = Cfg::D, NB = Cfg::NB, LPE = Cfg::LPE, EPW = Cfg::EPW;
@@ -570,66 +582,66 @@ __device__ __forceinline__ void tile_body(typename TileCfg<TYPE, SLOT, OP>::Smem
   const int lw = lane / LPE;
   const int le = warp * EPW + lw;
   const int64_t et = e0 + le;
+  const bool active = lw < EPW && et < n_end;
+  const int a = lane % LPE;
+  R K[NB][D][D], rhs[D] = {};
   if constexpr (COOP) {
-    using CS = TileCoop<Cfg, SC>;
-    static_assert(CS::kOn, "no cooperative scatter for this tile");
-    static_assert(offsetof(typename Cfg::Smem, G) % 16 == 0, "staged entries need 16-byte rows");
-    const bool active = lw < EPW && et < n_end;
-    const int a = lane % LPE;
-    R K[NB][D][D], rhs[D];
-    if (active) row_block<Cfg, OP>(sm, rr, P, le, a, K, rhs);
-    CS::run(reinterpret_cast<unsigned char*>(sm.G[warp * EPW]), P, active, active ? group_index(P, et) : 0, a, K, rhs);
-    __syncthreads();
-    return;
-  }
-  if (lw < EPW && et < n_end) {
-    const int a = lane % LPE;
-
-    R K[NB][D][D], rhs[D];
-    row_block<Cfg, OP>(sm, rr, P, le, a, K, rhs);
-
+    using CS = CoopScatter<NN, SC>;
+    CS::begin(sm.stage.rows[warp], P, active, active ? group_index(P, et) : 0, a);
+#pragma unroll 1
+    for (int b0 = 0; b0 < NN; b0 += NB) {
+      if (active) row_block<Cfg, OP>(sm, rr, P, le, a, b0, K, rhs);
+      CS::add(sm.stage.rows[warp], sm.stage.vals[warp], b0, K);
+    }
+    if (active) {
+      const int64_t node = P.tconn[group_index(P, et) * NN + a];
+#pragma unroll
+      for (int c = 0; c < D; ++c) red_add(P.b + D * node + c, widen(rhs[c]));
+    }
+  } else if (active) {
     const int64_t g = group_index(P, et);
     const int64_t node = P.tconn[g * NN + a];
     const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
     const int64_t moff = P.mapoff ? P.mapoff[g] : id * NN * NN;
-    const int32_t* mp = P.node_map + moff + a * NN;
     int64_t rb[D];
 #pragma unroll
     for (int c = 0; c < D; ++c) rb[c] = P.row_ptr[D * node + c];
-    if constexpr (SC == FEA_SCATTER_MULTIDEP) {
-      // this thread is the only writer of these entries (subdomain locks and
-      // a local color class), but CTAs on other SMs wrote them before the
-      // locks changed hands: read them from L2, a column's loads before its
-      // stores (wider groups measured slower: registers)
+#pragma unroll 1
+    for (int b0 = 0; b0 < NN; b0 += NB) {
+      row_block<Cfg, OP>(sm, rr, P, le, a, b0, K, rhs);
+      const int32_t* mp = P.node_map + moff + a * NN + b0;
 #pragma unroll
       for (int bb = 0; bb < NB; ++bb) {
         const int64_t k = mp[bb];
-        double old[D][D];
+        if constexpr (SC == FEA_SCATTER_MULTIDEP) {
+          // this thread is the only writer of these entries (subdomain locks
+          // and a local color class), but CTAs on other SMs wrote them before
+          // the locks changed hands: read them from L2, a column's loads
+          // before its stores (wider groups measured slower: registers)
+          double old[D][D];
 #pragma unroll
-        for (int c = 0; c < D; ++c)
+          for (int c = 0; c < D; ++c)
 #pragma unroll
-          for (int cc = 0; cc < D; ++cc) old[c][cc] = __ldcg(P.A + rb[c] + D * k + cc);
+            for (int cc = 0; cc < D; ++cc) old[c][cc] = __ldcg(P.A + rb[c] + D * k + cc);
 #pragma unroll
-        for (int c = 0; c < D; ++c)
+          for (int c = 0; c < D; ++c)
 #pragma unroll
-          for (int cc = 0; cc < D; ++cc) __stcg(P.A + rb[c] + D * k + cc, old[c][cc] + widen(K[bb][c][cc]));
+            for (int cc = 0; cc < D; ++cc) __stcg(P.A + rb[c] + D * k + cc, old[c][cc] + widen(K[bb][c][cc]));
+        } else {
+#pragma unroll
+          for (int c = 0; c < D; ++c)
+#pragma unroll
+            for (int cc = 0; cc < D; ++cc) scatter_add<SC>(P.A + rb[c] + D * k + cc, widen(K[bb][c][cc]));
+        }
       }
-      double ob[D];
+    }
 #pragma unroll
-      for (int c = 0; c < D; ++c) ob[c] = __ldcg(P.b + D * node + c);
-#pragma unroll
-      for (int c = 0; c < D; ++c) __stcg(P.b + D * node + c, ob[c] + widen(rhs[c]));
-    } else {
-#pragma unroll
-      for (int bb = 0; bb < NB; ++bb) {
-        const int64_t k = mp[bb];
-#pragma unroll
-        for (int c = 0; c < D; ++c)
-#pragma unroll
-          for (int cc = 0; cc < D; ++cc) scatter_add<SC>(P.A + rb[c] + D * k + cc, widen(K[bb][c][cc]));
-      }
-#pragma unroll
-      for (int c = 0; c < D; ++c) scatter_add<SC>(P.b + D * node + c, widen(rhs[c]));
+    for (int c = 0; c < D; ++c) {
+      double* p = P.b + D * node + c;
+      if constexpr (SC == FEA_SCATTER_MULTIDEP)
+        __stcg(p, __ldcg(p) + widen(rhs[c]));
+      else
+        scatter_add<SC>(p, widen(rhs[c]));
     }
   }
   __syncthreads();
@@ -641,13 +653,13 @@ template <int TYPE, int SLOT, int OP, int PREC>
 struct Tile {
   using Cfg = TileCfg<TYPE, SLOT, OP>;
   using Smem = typename Cfg::Smem;
-  template <int SC, bool COOP>
-  __device__ static __forceinline__ void run(unsigned char* raw, const RefRule& rr, const AsmParams& P, int64_t e0,
+  template <int SC, bool COOP, class Params>
+  __device__ static __forceinline__ void run(unsigned char* raw, const RefRule& rr, Params& P, int64_t e0,
                                              int64_t n_end) {
-    tile_body<TYPE, SLOT, OP, SC, COOP && TileCoop<Cfg, SC>::kOn>(*reinterpret_cast<Smem*>(raw), rr, P, e0, n_end);
+    tile_body<TYPE, SLOT, OP, SC, COOP && Cfg::D == 3 && SC == FEA_SCATTER_ATOMIC>(*reinterpret_cast<Smem*>(raw), rr, P, e0, n_end);
   }
   // CTAs per SM its own kernel is compiled for (0: the compiler's choice)
-  static constexpr int min_blocks(int sc) { return sc == FEA_SCATTER_ATOMIC && TileCoop<Cfg, FEA_SCATTER_ATOMIC>::kOn ? 4 : 0; }
+  static constexpr int min_blocks(int sc) { return sc == FEA_SCATTER_ATOMIC && Cfg::D == 3 ? 6 : 0; }
 };
 template <int TYPE, int SLOT, int OP>
 struct Tile<TYPE, SLOT, OP, FEA_FP64> {
@@ -661,14 +673,7 @@ struct Tile<TYPE, SLOT, OP, FEA_FP64> {
   static constexpr int min_blocks(int) { return 0; }
 };
 
-// Tile kernel: one tile per CTA.  Where the scatter is warp-cooperative its
-// staging needs about 15 more registers than the plain one; at four CTAs per
-// SM (128 registers) the hex8 elasticity FP32 atomic tile measured 5.69 ms
-// per 128^3 step on GB300, against 6.83 at three CTAs and 6.20 with the
-// plain scatter.  The other tiles keep the compiler's register choice (a
-// bound of 0), and the persistent kernels the plain scatter: there the
-// staging measured slower (8.22 against 7.48 ms; 256 meshes: 19.0 against
-// 18.4 ms).
+// Tile kernel: one tile per CTA.
 template <int TYPE, int SLOT, int OP, int PREC, int SC>
 __global__ void __launch_bounds__(128, (Tile<TYPE, SLOT, OP, PREC>::min_blocks(SC)))
     k_assemble_tile(const __grid_constant__ RefRule rr, const __grid_constant__ AsmParams P) {
@@ -692,22 +697,14 @@ struct PersistAsmArgs {
 
 template <int OP, int PREC>
 struct PersistCfg {
-  // CTAs per SM the any-type kernel is compiled for.  Its register count is
-  // the largest tile body's plus the call sequence (120 for FP32 diffusion),
-  // while the light types' own tiles need 46-56; measured on GB300 (4.53 M
-  // mixed elements, FP32 diffusion: 4.26 ms with no bound, 4.00 at 5, 3.90 at
-  // 6, 3.86 at 8; 256 elasticity meshes, FP32: 19.5 ms with no bound, 18.4
-  // at 5, 19.9 at 6, where spills start to cost more than the occupancy
-  // gains).  FP64 takes 6 (80 registers; a single tile's kernel needs 40-62,
-  // the compiler's choice here was 116-132).  FP32 elasticity hex items
-  // scatter warp-cooperatively (CoopScatter), which needs 4 CTAs per SM: the
-  // 256 meshes 18.3 ms plain at 5, 19.3 cooperative at 5, 17.1 at 4, 18.8
-  // at 3.  The hex-only kernel (ONLY) keeps the plain scatter: cooperative,
-  // without a bound, it measured 8.56 against 7.46 ms on 2.1 M hexes.
-  static constexpr int kMinBlocks = PREC == FEA_FP64 ? 6 : OP == FEA_OP_DIFFUSION ? 8 : 4;
-  // the hex-only kernel's
-  static constexpr int kMinBlocksHex = PREC == FEA_FP64 ? 6 : 1;
-  static constexpr bool kCoop = true;
+  // CTAs per SM the any-type and the hex-only kernel are compiled for.  FP64:
+  // 80 registers, where a single tile's kernel needs 40-62 and the compiler's
+  // choice here was 116-132.  FP32 diffusion: 64 registers, no spills with the
+  // tiles called one by one.  FP32 elasticity: 96 registers; measured on GB300
+  // (64 meshes: 1.59 ms at 4 and 5, 1.58 at 6; with plain reductions of the
+  // types other than hex8 1.51 at 5, 1.52 at 6; their cooperative scatter,
+  // faster in the per-type kernels, spills in the called tiles).
+  static constexpr int kMinBlocks = PREC == FEA_FP64 ? 6 : OP == FEA_OP_DIFFUSION ? 8 : 5;
   template <int TYPE, int SLOT>
   static constexpr size_t bytes() { return sizeof(typename Tile<TYPE, SLOT, OP, PREC>::Smem); }
   static constexpr size_t mx(size_t a, size_t b) { return a > b ? a : b; }
@@ -719,22 +716,41 @@ struct PersistCfg {
 template <int TYPE, int SLOT, int OP, int PREC, int SC = FEA_SCATTER_ATOMIC, bool COOP = false>
 __device__ __forceinline__ void persist_item(unsigned char* raw, const AsmParams& P, int64_t first, int64_t end) {
   using T = Tile<TYPE, SLOT, OP, PREC>;
-  for (int64_t e0 = first; e0 < end; e0 += T::Cfg::EPC) T::template run<SC, COOP>(raw, c_rules[SLOT], P, e0, end);
+  for (int64_t e0 = first; e0 < end; e0 += T::Cfg::EPC)
+    T::template run<SC, COOP>(raw, c_rules[SLOT + opaque_zero()], P, e0, end);
 }
 
-// One item of the any-type kernel, not inlined: the switch over five inlined
+// Shared memory of the any-type kernel: the item's parameters, then the tile.
+constexpr size_t kParamBytes = (sizeof(AsmParams) + 15) & ~size_t(15);
+
+// One tile of the any-type kernel, not inlined: the switch over five inlined
 // tile bodies made ptxas allocate well above the largest body's registers
-// (FP32 diffusion: 128 against 72), which cut the all-type launch's
-// occupancy; a call keeps the kernel near the largest body (96).
+// (FP32 diffusion: 128 against 72), which cut the all-type launch's occupancy.
+// It is a call per tile, not per item, because the compiler moved what a body
+// computes from its thread index alone out of a loop over tiles, and spilled
+// it (FP32 elasticity: 500-700 bytes per body at 80 registers); and it takes
+// its shared memory and parameters by name, so that they are read as shared
+// memory and not through generic addresses.
+// FP32 tiles read them anew at each use (volatile): kept in registers, the 22
+// words cost more than the loads.
 template <int TYPE, int SLOT, int OP, int PREC>
-__device__ __noinline__ void persist_item_call(unsigned char* raw, const AsmParams& P, int64_t first, int64_t end) {
-  persist_item<TYPE, SLOT, OP, PREC, FEA_SCATTER_ATOMIC, PersistCfg<OP, PREC>::kCoop>(raw, P, first, end);
+__device__ __noinline__ void persist_tile(int64_t e0, int64_t end) {
+  extern __shared__ __align__(16) unsigned char persist_smem[];
+  using Params = std::conditional_t<PREC == FEA_FP64, const AsmParams, const volatile AsmParams>;
+  Tile<TYPE, SLOT, OP, PREC>::template run<FEA_SCATTER_ATOMIC, TYPE == FEA_HEX8>(
+      persist_smem + kParamBytes, c_rules[SLOT], *reinterpret_cast<Params*>(persist_smem), e0, end);
+}
+
+template <int TYPE, int SLOT, int OP, int PREC>
+__device__ __forceinline__ void persist_tiles(int64_t first, int64_t end) {
+  for (int64_t e0 = first; e0 < end; e0 += Tile<TYPE, SLOT, OP, PREC>::Cfg::EPC)
+    persist_tile<TYPE, SLOT, OP, PREC>(e0, end);
 }
 
 // ONLY >= 0: every item uses that rule slot (a single-type mesh), so the
 // kernel holds one tile body and its register budget; -1: any element type
 template <int OP, int PREC, int ONLY>
-__global__ void __launch_bounds__(128, ONLY < 0 ? PersistCfg<OP, PREC>::kMinBlocks : PersistCfg<OP, PREC>::kMinBlocksHex)
+__global__ void __launch_bounds__(128, PersistCfg<OP, PREC>::kMinBlocks)
     k_persistent(const __grid_constant__ PersistAsmArgs A) {
   extern __shared__ __align__(16) unsigned char persist_smem[];
   __shared__ int s_item;
@@ -746,28 +762,21 @@ __global__ void __launch_bounds__(128, ONLY < 0 ? PersistCfg<OP, PREC>::kMinBloc
     const uint64_t t0 = global_ns();
     const WorkItem it = A.S.items[item];
     const int64_t first = it.first, end = (int64_t)it.first + it.count;
-    // single mesh: entry t is type t, read at a constant offset of the
-    // parameter space; batches: the device table
     if constexpr (ONLY == kRuleHex8) {
-      persist_item<FEA_HEX8, kRuleHex8, OP, PREC>(persist_smem, A.table[FEA_HEX8], first, end);
-    } else if (A.tab) {
-      const AsmParams& P = A.tab[it.entry];
-      switch (A.tab_slot[it.entry]) {
-        case kRuleTet1: persist_item_call<FEA_TET4, kRuleTet1, OP, PREC>(persist_smem, P, first, end); break;
-        case kRuleTet4: persist_item_call<FEA_TET4, kRuleTet4, OP, PREC>(persist_smem, P, first, end); break;
-        case kRulePyr8: persist_item_call<FEA_PYR5, kRulePyr8, OP, PREC>(persist_smem, P, first, end); break;
-        case kRulePrism6: persist_item_call<FEA_PRISM6, kRulePrism6, OP, PREC>(persist_smem, P, first, end); break;
-        default: persist_item_call<FEA_HEX8, kRuleHex8, OP, PREC>(persist_smem, P, first, end); break;
-      }
+      persist_item<FEA_HEX8, kRuleHex8, OP, PREC, FEA_SCATTER_ATOMIC, true>(persist_smem, A.table[FEA_HEX8], first, end);
     } else {
-      switch (A.slot[it.entry]) {
-        case kRuleTet1: persist_item_call<FEA_TET4, kRuleTet1, OP, PREC>(persist_smem, A.table[FEA_TET4], first, end); break;
-        case kRuleTet4: persist_item_call<FEA_TET4, kRuleTet4, OP, PREC>(persist_smem, A.table[FEA_TET4], first, end); break;
-        case kRulePyr8: persist_item_call<FEA_PYR5, kRulePyr8, OP, PREC>(persist_smem, A.table[FEA_PYR5], first, end); break;
-        case kRulePrism6:
-          persist_item_call<FEA_PRISM6, kRulePrism6, OP, PREC>(persist_smem, A.table[FEA_PRISM6], first, end);
-          break;
-        default: persist_item_call<FEA_HEX8, kRuleHex8, OP, PREC>(persist_smem, A.table[FEA_HEX8], first, end); break;
+      // the item's parameters: of its type (single mesh) or its (mesh, type)
+      static_assert(sizeof(AsmParams) % 8 == 0 && sizeof(AsmParams) / 8 <= 128, "a thread per word");
+      const AsmParams& P = A.tab ? A.tab[it.entry] : A.table[it.entry];
+      if (threadIdx.x < sizeof(AsmParams) / 8)
+        reinterpret_cast<uint64_t*>(persist_smem)[threadIdx.x] = reinterpret_cast<const uint64_t*>(&P)[threadIdx.x];
+      __syncthreads();
+      switch (A.tab ? A.tab_slot[it.entry] : A.slot[it.entry]) {
+        case kRuleTet1: persist_tiles<FEA_TET4, kRuleTet1, OP, PREC>(first, end); break;
+        case kRuleTet4: persist_tiles<FEA_TET4, kRuleTet4, OP, PREC>(first, end); break;
+        case kRulePyr8: persist_tiles<FEA_PYR5, kRulePyr8, OP, PREC>(first, end); break;
+        case kRulePrism6: persist_tiles<FEA_PRISM6, kRulePrism6, OP, PREC>(first, end); break;
+        default: persist_tiles<FEA_HEX8, kRuleHex8, OP, PREC>(first, end); break;
       }
     }
     sched_record(A.S, item, it.entry, t0);
@@ -958,7 +967,7 @@ static int rule_slot_of(int type, int tet_rule) {
 template <int OP, int PREC, int ONLY>
 static int launch_persistent_k(const PersistAsmArgs& args, int n_ctas, bool dry, cudaStream_t s, int* grid_out) {
   constexpr size_t smem = ONLY == kRuleHex8 ? sizeof(typename Tile<FEA_HEX8, kRuleHex8, OP, PREC>::Smem)
-                                            : PersistCfg<OP, PREC>::smem;
+                                            : kParamBytes + PersistCfg<OP, PREC>::smem;
   auto kern = k_persistent<OP, PREC, ONLY>;
   if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int grid = n_ctas;

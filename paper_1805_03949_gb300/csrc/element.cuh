@@ -52,17 +52,18 @@ const RefRule& host_rule(int slot);
 __device__ __forceinline__ double f32_to_f64_exact(float x) {
   const uint32_t u = __float_as_uint(x);
   const uint32_t mag = u & 0x7fffffffu;
-  if (mag - 0x00800000u < 0x7f000000u) {
-    // a normal number: the exponent field moves 3 bits down and its bias
+  if (mag - 0x00800000u < 0x7f000000u || mag == 0u) {
+    // a normal number (or a zero, which entries of axis-aligned elements often
+    // are: a select, not a branch of the warp): the exponent field moves 3 bits down and its bias
     // grows by 1023 - 127 = 896; the 23 fraction bits split 20 | 3 across
     // the two words
-    return __hiloint2double((int)(((mag >> 3) + (896u << 20)) | (u & 0x80000000u)), (int)(u << 29));
+    const uint32_t hi = mag == 0u ? 0u : (mag >> 3) + (896u << 20);
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
   }
   const uint32_t sign = u & 0x80000000u;
   int e = (int)((u >> 23) & 0xffu);
   uint32_t m = u & 0x7fffffu;
   if (e == 0) {
-    if (m == 0) return __hiloint2double((int)sign, 0);
     const int lz = __clz((int)m) - 8;  // normalise a subnormal: bring the leading bit to position 23
     m = (m << lz) & 0x7fffffu;
     e = 1 - lz;

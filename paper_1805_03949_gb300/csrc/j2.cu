@@ -73,7 +73,7 @@ struct J2Cfg {
   static constexpr int WARPS = 4;
   static constexpr int THREADS = 32 * WARPS;
   static constexpr int EPC = EPW * WARPS;
-  static constexpr int NB = NN;
+  static constexpr int NB = column_group(NN, 3);  // columns per lane at a time
   static constexpr bool kHex = TYPE == FEA_HEX8;
   static_assert(!kHex || (EPC * 8 % 32 == 0 && EPC * 8 <= THREADS), "modal hex geometry needs whole warps");
   // what the Gauss-point update of the element loop needs
@@ -86,6 +86,7 @@ struct J2Cfg {
     float H[EPC][NQ][grad_stride(NN)];  // h_a = n grad N_a
     float C[EPC][NQ][4];      // W, W lam', W mu', W beta
     float S[EPC][NQ][6];      // W sigma (xx, yy, zz, xy, yz, xz)
+    typename CoopScatter<NN, FEA_SCATTER_ATOMIC>::Rows rows[WARPS];  // (the cooperative scatter's)
   };
 };
 
@@ -342,65 +343,75 @@ __device__ __forceinline__ void j2_tile_body(Smem& sm, const RefRule& rr, const 
     const int64_t et = e0 + le;
     const bool active = lw < EPW && et < n_end;
     const int a = lane % LPE;
-    float K[NB][3][3], rhs[3] = {0.0f, 0.0f, 0.0f};
-#pragma unroll
-    for (int bb = 0; bb < NB; ++bb)
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] = 0.0f;
-    if (active) {
-#pragma unroll 1
-      for (int q = 0; q < NQ; ++q) {
-        const float wl = sm.C[le][q][1], wm = sm.C[le][q][2], wb = sm.C[le][q][3];
-        const float *pg = sm.G[le][q], *ph = sm.H[le][q];
-        const float ga[3] = {pg[3 * a], pg[3 * a + 1], pg[3 * a + 2]};
-        const float gl[3] = {wl * ga[0], wl * ga[1], wl * ga[2]};
-        const float gm[3] = {wm * ga[0], wm * ga[1], wm * ga[2]};
-        const float hb[3] = {wb * ph[3 * a], wb * ph[3 * a + 1], wb * ph[3 * a + 2]};
-#pragma unroll
-        for (int bb = 0; bb < NB; ++bb) {
-          const float gb[3] = {pg[3 * bb], pg[3 * bb + 1], pg[3 * bb + 2]};
-          const float hh[3] = {ph[3 * bb], ph[3 * bb + 1], ph[3 * bb + 2]};
-          const float dot = gm[0] * gb[0] + gm[1] * gb[1] + gm[2] * gb[2];
-#pragma unroll
-          for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] += gl[c] * gb[cc] + gm[cc] * gb[c] - hb[c] * hh[cc];
-#pragma unroll
-          for (int c = 0; c < 3; ++c) K[bb][c][c] += dot;
-        }
-        const float* S = sm.S[le][q];
-        rhs[0] += S[0] * ga[0] + S[3] * ga[1] + S[5] * ga[2];
-        rhs[1] += S[3] * ga[0] + S[1] * ga[1] + S[4] * ga[2];
-        rhs[2] += S[5] * ga[0] + S[4] * ga[1] + S[2] * ga[2];
-      }
+    const int64_t g = active ? group_index(P, et) : 0;
+    const int64_t node = active ? (int64_t)P.tconn[g * NN + a] : 0;
+    using CS = CoopScatter<NN, SC>;
+    // the cooperative scatter stages its values where the coordinates and
+    // displacements were
+    float* vals = reinterpret_cast<float*>(&sm) + warp * CS::kVals;
+    constexpr bool kCoop = CS::kOn && Cfg::WARPS * CS::kVals * sizeof(float) <= 2 * sizeof(sm.X);
+    if constexpr (kCoop) {
+      CS::begin(sm.rows[warp], P, active, g, a);
     }
-    using CS = CoopScatter<NN, SC, sizeof(sm.G) / Cfg::WARPS>;
-    if constexpr (CS::kOn) {
-      // staged in the gradients of the warp's own elements
-      static_assert(sizeof(typename Cfg::Fields) % 16 == 0, "staged entries need 16-byte rows");
-      CS::run(reinterpret_cast<unsigned char*>(sm.G[warp * EPW]), P, active, active ? group_index(P, et) : 0, a, K, rhs);
-    } else if (active) {
-      const int64_t g = group_index(P, et);
-      const int64_t node = P.tconn[g * NN + a];
-      const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
-      const int64_t moff = P.mapoff ? P.mapoff[g] : id * NN * NN;
-      const int32_t* mp = P.node_map + moff + a * NN;
-      int64_t rb[3];
+    float rhs[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+    for (int b0 = 0; b0 < NN; b0 += NB) {
+      float K[NB][3][3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) rb[c] = P.row_ptr[3 * node + c];
-#pragma unroll
-      for (int bb = 0; bb < NB; ++bb) {
-        const int64_t k = mp[bb];
+      for (int bb = 0; bb < NB; ++bb)
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
-          for (int cc = 0; cc < 3; ++cc) scatter_add<SC>(P.A + rb[c] + 3 * k + cc, widen(K[bb][c][cc]));
+          for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] = 0.0f;
+      if (active) {
+#pragma unroll 1
+        for (int q = 0; q < NQ; ++q) {
+          const float wl = sm.C[le][q][1], wm = sm.C[le][q][2], wb = sm.C[le][q][3];
+          const float *pg = sm.G[le][q], *ph = sm.H[le][q];
+          const float ga[3] = {pg[3 * a], pg[3 * a + 1], pg[3 * a + 2]};
+          const float gl[3] = {wl * ga[0], wl * ga[1], wl * ga[2]};
+          const float gm[3] = {wm * ga[0], wm * ga[1], wm * ga[2]};
+          const float hb[3] = {wb * ph[3 * a], wb * ph[3 * a + 1], wb * ph[3 * a + 2]};
+#pragma unroll
+          for (int bb = 0; bb < NB; ++bb) {
+            const float gb[3] = {pg[3 * (b0 + bb)], pg[3 * (b0 + bb) + 1], pg[3 * (b0 + bb) + 2]};
+            const float hh[3] = {ph[3 * (b0 + bb)], ph[3 * (b0 + bb) + 1], ph[3 * (b0 + bb) + 2]};
+            const float dot = gm[0] * gb[0] + gm[1] * gb[1] + gm[2] * gb[2];
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+#pragma unroll
+              for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] += gl[c] * gb[cc] + gm[cc] * gb[c] - hb[c] * hh[cc];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) K[bb][c][c] += dot;
+          }
+          if (b0 == 0) {
+            const float* S = sm.S[le][q];
+            rhs[0] += S[0] * ga[0] + S[3] * ga[1] + S[5] * ga[2];
+            rhs[1] += S[3] * ga[0] + S[1] * ga[1] + S[4] * ga[2];
+            rhs[2] += S[5] * ga[0] + S[4] * ga[1] + S[2] * ga[2];
+          }
+        }
       }
+      if constexpr (kCoop) {
+        CS::add(sm.rows[warp], vals, b0, K);
+      } else if (active) {
+        const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
+        const int32_t* mp = P.node_map + (P.mapoff ? P.mapoff[g] : id * NN * NN) + a * NN + b0;
+#pragma unroll
+        for (int bb = 0; bb < NB; ++bb) {
+          const int64_t k = mp[bb];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            double* row = P.A + P.row_ptr[3 * node + c] + 3 * k;
+#pragma unroll
+            for (int cc = 0; cc < 3; ++cc) scatter_add<SC>(row + cc, widen(K[bb][c][cc]));
+          }
+        }
+      }
+    }
+    if (active)
 #pragma unroll
       for (int c = 0; c < 3; ++c) scatter_add<SC>(P.b + 3 * node + c, widen(rhs[c]));
-    }
     __syncthreads();
   }
 }
@@ -563,7 +574,7 @@ struct J2Tile<TYPE, SLOT, FEA_FP64, false> {
 
 // one tile per CTA
 template <int TYPE, int SLOT, int PREC, int SC, bool POINTS>
-__global__ void __launch_bounds__(128) k_j2_tile(const __grid_constant__ RefRule rr, const __grid_constant__ J2Params P) {
+__global__ void __launch_bounds__(128, POINTS || PREC == FEA_FP64 ? 0 : 5) k_j2_tile(const __grid_constant__ RefRule rr, const __grid_constant__ J2Params P) {
   using T = J2Tile<TYPE, SLOT, PREC, POINTS>;
   extern __shared__ __align__(16) unsigned char j2_smem_raw[];
   T::template run<SC>(j2_smem_raw, rr, P, (int64_t)blockIdx.x * T::Cfg::EPC, P.n);
@@ -623,7 +634,7 @@ template <int TYPE, int SLOT, int PREC, bool POINTS>
 __device__ __forceinline__ void persist_j2_item(unsigned char* raw, const J2Params& P, int64_t first, int64_t end) {
   using T = J2Tile<TYPE, SLOT, PREC, POINTS>;
   for (int64_t e0 = first; e0 < end; e0 += T::Cfg::EPC)
-    T::template run<FEA_SCATTER_ATOMIC>(raw, c_rules_j2[SLOT], P, e0, end);
+    T::template run<FEA_SCATTER_ATOMIC>(raw, c_rules_j2[SLOT + opaque_zero()], P, e0, end);
 }
 
 // One item of the any-type kernel, not inlined: four inlined tile bodies take
@@ -633,9 +644,14 @@ __device__ __noinline__ void persist_j2_call(unsigned char* raw, const J2Params&
   persist_j2_item<TYPE, SLOT, PREC, POINTS>(raw, P, first, end);
 }
 
-// ONLY == kRuleHex8: a mesh of hexes only (one tile body); -1: any type
+// ONLY == kRuleHex8: a mesh of hexes only (one tile body); -1: any type.
+// CTAs per SM: what the shared memory (FP64) or the registers without large
+// spills allow.  The element loop could run 8, but with four times as many
+// CTAs as SM sub-partitions an item's time says little about its cost (the
+// network of the cost model explained 2 % of it, 55 % at four).
 template <int PREC, int ONLY, bool POINTS>
-__global__ void __launch_bounds__(128, PREC == FEA_FP64 ? 3 : 4) k_persistent_j2(const __grid_constant__ PersistJ2Args A) {
+__global__ void __launch_bounds__(128, PREC == FEA_FP64 ? 3 : POINTS || ONLY < 0 ? 4 : 5)
+    k_persistent_j2(const __grid_constant__ PersistJ2Args A) {
   extern __shared__ __align__(16) unsigned char persist_j2_smem[];
   __shared__ int s_item;
   sched_start(A.S);

@@ -55,7 +55,7 @@ struct NHCfg {
   static constexpr int WARPS = 4;
   static constexpr int THREADS = 32 * WARPS;
   static constexpr int EPC = EPW * WARPS;
-  static constexpr int NB = NN;
+  static constexpr int NB = column_group(NN, 3);  // columns per lane at a time
   static constexpr bool kHex = TYPE == FEA_HEX8;
   static_assert(!kHex || (EPC * 8 % 32 == 0 && EPC * 8 <= THREADS), "modal hex geometry needs whole warps");
   struct Smem {
@@ -65,6 +65,7 @@ struct NHCfg {
     float H[EPC][NQ][grad_stride(NN)];  // h_a = F^-T g_a
     float C[EPC][NQ][4];      // W mu, W lam, W (mu - lam ln J), W m
     float S[EPC][NQ][9];      // W P, row-major
+    typename CoopScatter<NN, FEA_SCATTER_ATOMIC>::Rows rows[WARPS];  // (the cooperative scatter's)
   };
 };
 
@@ -217,65 +218,75 @@ __device__ __forceinline__ void nh_tile_body(typename NHCfg<TYPE, SLOT>::Smem& s
   const int64_t et = e0 + le;
   const bool active = lw < EPW && et < n_end;
   const int a = lane % LPE;
-  float K[NB][3][3], rhs[3] = {0.0f, 0.0f, 0.0f};
-#pragma unroll
-  for (int bb = 0; bb < NB; ++bb)
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] = 0.0f;
-  if (active) {
-#pragma unroll 1
-    for (int q = 0; q < NQ; ++q) {
-      const float wm = sm.C[le][q][0], wl = sm.C[le][q][1], wp = sm.C[le][q][2], wn = sm.C[le][q][3];
-      const float *pg = sm.G[le][q], *ph = sm.H[le][q];
-      const float ga[3] = {pg[3 * a], pg[3 * a + 1], pg[3 * a + 2]};
-      const float gm[3] = {wm * ga[0], wm * ga[1], wm * ga[2]};
-      const float hl[3] = {wl * ph[3 * a], wl * ph[3 * a + 1], wl * ph[3 * a + 2]};
-      const float hp[3] = {wp * ph[3 * a], wp * ph[3 * a + 1], wp * ph[3 * a + 2]};
-      const float mn = wn * rr.Nf[q][a];
-#pragma unroll
-      for (int bb = 0; bb < NB; ++bb) {
-        const float gb[3] = {pg[3 * bb], pg[3 * bb + 1], pg[3 * bb + 2]};
-        const float hb[3] = {ph[3 * bb], ph[3 * bb + 1], ph[3 * bb + 2]};
-        const float diag = gm[0] * gb[0] + gm[1] * gb[1] + gm[2] * gb[2] + mn * rr.Nf[q][bb];
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-#pragma unroll
-          for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] += hl[c] * hb[cc] + hb[c] * hp[cc];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) K[bb][c][c] += diag;
-      }
-      const float* S = sm.S[le][q];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) rhs[c] += S[3 * c] * ga[0] + S[3 * c + 1] * ga[1] + S[3 * c + 2] * ga[2];
-    }
+  const int64_t g = active ? group_index(P, et) : 0;
+  const int64_t node = active ? (int64_t)P.tconn[g * NN + a] : 0;
+  using CS = CoopScatter<NN, SC>;
+  // the cooperative scatter stages its values where the coordinates and
+  // displacements were
+  float* vals = reinterpret_cast<float*>(&sm) + warp * CS::kVals;
+  constexpr bool kCoop = CS::kOn && Cfg::WARPS * CS::kVals * sizeof(float) <= 2 * sizeof(sm.X);
+  if constexpr (kCoop) {
+    CS::begin(sm.rows[warp], P, active, g, a);
   }
-  using CS = CoopScatter<NN, SC, sizeof(sm.G) / Cfg::WARPS>;
-  if constexpr (CS::kOn) {
-    // staged in the gradients of the warp's own elements
-    static_assert(offsetof(typename Cfg::Smem, G) % 16 == 0, "staged entries need 16-byte rows");
-    CS::run(reinterpret_cast<unsigned char*>(sm.G[warp * EPW]), P, active, active ? group_index(P, et) : 0, a, K, rhs);
-  } else if (active) {
-    const int64_t g = group_index(P, et);
-    const int64_t node = P.tconn[g * NN + a];
-    const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
-    const int64_t moff = P.mapoff ? P.mapoff[g] : id * NN * NN;
-    const int32_t* mp = P.node_map + moff + a * NN;
-    int64_t rb[3];
+  float rhs[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+  for (int b0 = 0; b0 < NN; b0 += NB) {
+    float K[NB][3][3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) rb[c] = P.row_ptr[3 * node + c];
-#pragma unroll
-    for (int bb = 0; bb < NB; ++bb) {
-      const int64_t k = mp[bb];
+    for (int bb = 0; bb < NB; ++bb)
 #pragma unroll
       for (int c = 0; c < 3; ++c)
 #pragma unroll
-        for (int cc = 0; cc < 3; ++cc) scatter_add<SC>(P.A + rb[c] + 3 * k + cc, widen(K[bb][c][cc]));
+        for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] = 0.0f;
+    if (active) {
+#pragma unroll 1
+      for (int q = 0; q < NQ; ++q) {
+        const float wm = sm.C[le][q][0], wl = sm.C[le][q][1], wp = sm.C[le][q][2], wn = sm.C[le][q][3];
+        const float *pg = sm.G[le][q], *ph = sm.H[le][q];
+        const float ga[3] = {pg[3 * a], pg[3 * a + 1], pg[3 * a + 2]};
+        const float gm[3] = {wm * ga[0], wm * ga[1], wm * ga[2]};
+        const float hl[3] = {wl * ph[3 * a], wl * ph[3 * a + 1], wl * ph[3 * a + 2]};
+        const float hp[3] = {wp * ph[3 * a], wp * ph[3 * a + 1], wp * ph[3 * a + 2]};
+        const float mn = wn * rr.Nf[q][a];
+#pragma unroll
+        for (int bb = 0; bb < NB; ++bb) {
+          const float gb[3] = {pg[3 * (b0 + bb)], pg[3 * (b0 + bb) + 1], pg[3 * (b0 + bb) + 2]};
+          const float hb[3] = {ph[3 * (b0 + bb)], ph[3 * (b0 + bb) + 1], ph[3 * (b0 + bb) + 2]};
+          const float diag = gm[0] * gb[0] + gm[1] * gb[1] + gm[2] * gb[2] + mn * rr.Nf[q][b0 + bb];
+#pragma unroll
+          for (int c = 0; c < 3; ++c)
+#pragma unroll
+            for (int cc = 0; cc < 3; ++cc) K[bb][c][cc] += hl[c] * hb[cc] + hb[c] * hp[cc];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) K[bb][c][c] += diag;
+        }
+        if (b0 == 0) {
+          const float* S = sm.S[le][q];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) rhs[c] += S[3 * c] * ga[0] + S[3 * c + 1] * ga[1] + S[3 * c + 2] * ga[2];
+        }
+      }
     }
+    if constexpr (kCoop) {
+      CS::add(sm.rows[warp], vals, b0, K);
+    } else if (active) {
+      const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
+      const int32_t* mp = P.node_map + (P.mapoff ? P.mapoff[g] : id * NN * NN) + a * NN + b0;
+#pragma unroll
+      for (int bb = 0; bb < NB; ++bb) {
+        const int64_t k = mp[bb];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          double* row = P.A + P.row_ptr[3 * node + c] + 3 * k;
+#pragma unroll
+          for (int cc = 0; cc < 3; ++cc) scatter_add<SC>(row + cc, widen(K[bb][c][cc]));
+        }
+      }
+    }
+  }
+  if (active)
 #pragma unroll
     for (int c = 0; c < 3; ++c) scatter_add<SC>(P.b + 3 * node + c, widen(rhs[c]));
-  }
   __syncthreads();
 }
 
@@ -416,7 +427,7 @@ struct NHTile<TYPE, SLOT, FEA_FP64> {
 };
 
 template <int TYPE, int SLOT, int PREC, int SC>
-__global__ void __launch_bounds__(128, PREC == FEA_FP64 ? 0 : 4) k_nh_tile(const __grid_constant__ RefRule rr, const __grid_constant__ NHParams P) {
+__global__ void __launch_bounds__(128, PREC == FEA_FP64 ? 0 : 5) k_nh_tile(const __grid_constant__ RefRule rr, const __grid_constant__ NHParams P) {
   using T = NHTile<TYPE, SLOT, PREC>;
   extern __shared__ __align__(16) unsigned char nh_smem_raw[];
   T::template run<SC>(*reinterpret_cast<typename T::Cfg::Smem*>(nh_smem_raw), rr, P,

@@ -31,10 +31,14 @@ struct ElemParams {
   DevStatus* st;
 };
 
-__device__ __forceinline__ int64_t group_index(const ElemParams& P, int64_t et) {
+// (Params: const ElemParams or a derived struct, volatile where its fields are
+// to be read from shared memory at each use instead of kept in registers)
+template <class Params>
+__device__ __forceinline__ int64_t group_index(Params& P, int64_t et) {
   return P.list ? (int64_t)P.list[et] : et;
 }
-__device__ __forceinline__ int64_t original_id(const ElemParams& P, int64_t et) {
+template <class Params>
+__device__ __forceinline__ int64_t original_id(Params& P, int64_t et) {
   const int64_t g = group_index(P, et);
   return P.ids ? (int64_t)P.ids[g] : g;
 }

@@ -49,6 +49,16 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 
+// 0, unknown to the compiler.  The persistent kernels add it to the index of a
+// tile's quadrature tables: they are constant memory, and the compiler
+// otherwise moves their loads out of the loop over tiles, which fills the
+// registers and spills.
+__device__ __forceinline__ int opaque_zero() {
+  int z;
+  asm volatile("mov.u32 %0, 0;" : "=r"(z));
+  return z;
+}
+
 // The next item of this CTA (-1: done).  Every thread of the CTA calls it; k
 // is the CTA's position in its own queue.  s_item is a shared slot.
 //  STEAL          next position of a global counter, into the item list or,
