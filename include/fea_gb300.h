@@ -474,8 +474,8 @@ int fea_batch_latency(fea_batch* batch, uint64_t* mesh_ns_h, void* stream);
  * a library allocate device memory -- applications that reserve all of the
  * GPU's memory for their own pool at start-up, or that run this step where an
  * allocation would have to go through their allocator or would synchronize
- * the device.  The same scan inside fea_pattern_size takes its scratch from a
- * stream-ordered allocation; this entry point instead uses a fixed 128 KB
+ * the device.  The same scan inside fea_pattern_size takes its scratch from the
+ * mesh handle's allocation; this entry point instead uses a fixed 128 KB
  * array compiled into the library, which every GPU that loads the library
  * holds until the process exits.
  *  counts_d   int32 [n] row lengths (device)

@@ -15,6 +15,7 @@
 //   phase 2  n_e lanes per element: lane a accumulates the row block A^e_(a, b)
 //            for every column b over the points
 //   phase 3  the same lane scatters its row block through the rank map.
+#include <algorithm>
 #include <cmath>
 #include <cstddef>
 #include <cstdio>
@@ -577,6 +578,7 @@ __device__ __forceinline__ void tile_body(typename TileCfg<TYPE, SLOT, OP>::Smem
   using R = float;
   constexpr int NN = Cfg::NN, D = Cfg::D, NB = Cfg::NB, LPE = Cfg::LPE, EPW = Cfg::EPW;
   tile_geometry<Cfg, OP>(sm, rr, P, e0, n_end);
+  if constexpr (SC == FEA_SCATTER_ATOMIC) wait_for_previous();
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int lw = lane / LPE;
@@ -679,6 +681,7 @@ __global__ void __launch_bounds__(128, (Tile<TYPE, SLOT, OP, PREC>::min_blocks(S
     k_assemble_tile(const __grid_constant__ RefRule rr, const __grid_constant__ AsmParams P) {
   using T = Tile<TYPE, SLOT, OP, PREC>;
   extern __shared__ __align__(16) unsigned char tile_smem[];
+  let_next_start();
   T::template run<SC, true>(tile_smem, rr, P, (int64_t)blockIdx.x * T::Cfg::EPC, P.n);
 }
 
@@ -1143,8 +1146,9 @@ static int launch_tile(const AsmParams& P, cudaStream_t s) {
   constexpr size_t smem = sizeof(typename T::Smem);
   auto kern = k_assemble_tile<TYPE, SLOT, OP, PREC, SC>;
   if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<grid, T::Cfg::THREADS, smem, s>>>(host_rule(SLOT), P);
-  FEA_CUDA(cudaGetLastError());
+  constexpr bool kLight = TYPE == FEA_TET4 && (OP == FEA_OP_DIFFUSION || PREC != FEA_FP64);
+  const bool early = P.early && starts_early(grid, P.early == 1, kLight);
+  FEA_CUDA(launch_tiles(kern, grid, T::Cfg::THREADS, smem, s, early, host_rule(SLOT), P));
   return FEA_OK;
 }
 
@@ -1199,8 +1203,8 @@ int assemble(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, const 
     cudaEvent_t* ev = (cudaEvent_t*)op->events;
     const int nev = ev ? op->n_events : 0;
     if (nev > 0) FEA_CUDA(cudaEventRecord(ev[0], s));
-    FEA_CUDA(cudaMemsetAsync(A, 0, (int64_t)D * D * m->nnz_node * sizeof(double), s));
-    FEA_CUDA(cudaMemsetAsync(b, 0, m->n_nodes * D * sizeof(double), s));
+    rc = zero_system(A, (int64_t)D * D * m->nnz_node, b, m->n_nodes * D, nullptr, s);
+    if (rc) return rc;
     if (nev > 1) FEA_CUDA(cudaEventRecord(ev[1], s));
     rc = launch_multidep(op, m, *plan, row_ptr, node_map, A, b, s);
     if (rc) return rc;
@@ -1250,10 +1254,11 @@ int assemble(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, const 
     // block boundaries, which they add to: only those rows are cleared
     int rc = zero_block_rows(*bplan, row_ptr, A, s);
     if (rc) return rc;
+    FEA_CUDA(cudaMemsetAsync(b, 0, m->n_nodes * D * sizeof(double), s));
   } else {
-    FEA_CUDA(cudaMemsetAsync(A, 0, nnz * sizeof(double), s));
+    int rc = zero_system(A, nnz, b, m->n_nodes * D, nullptr, s);
+    if (rc) return rc;
   }
-  FEA_CUDA(cudaMemsetAsync(b, 0, m->n_nodes * D * sizeof(double), s));
   if (nev > 1) FEA_CUDA(cudaEventRecord(ev[1], s));
   if (op->scatter == FEA_SCATTER_BLOCK) {
     // geometry records (computed by the task kernel itself for hex meshes in
@@ -1289,6 +1294,7 @@ int assemble(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, const 
   P.mu = E / (2.0 * (1.0 + nu));
   for (int c = 0; c < 3; ++c) P.f[c] = op->body_force[c];
   P.geo64 = op->precision != FEA_FP32_ADAPTIVE;
+  P.early = op->scatter == FEA_SCATTER_ATOMIC && small_system(nnz);
   auto run = [&](int t) -> int {
     int rc;
     if (op->kind == FEA_OP_DIFFUSION)
@@ -1300,6 +1306,7 @@ int assemble(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, const 
     if (rc) return rc;
     if (2 + launched < nev) FEA_CUDA(cudaEventRecord(ev[2 + launched], s));
     ++launched;
+    if (P.early) P.early = 2;
     return FEA_OK;
   };
   if (op->scatter == FEA_SCATTER_COLOR) {
@@ -1333,6 +1340,30 @@ int assemble(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, const 
     int rc = run(t);
     if (rc) return rc;
   }
+  for (int k = 2 + launched; k < nev; ++k) FEA_CUDA(cudaEventRecord(ev[k], s));
+  return FEA_OK;
+}
+
+__global__ void __launch_bounds__(256) k_zero_system(double* A, int64_t nnz, double* b, int64_t nb, int32_t* counter) {
+  let_next_start();
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, n = (int64_t)gridDim.x * blockDim.x;
+  // A is 16-byte aligned
+  for (int64_t i = t; i < nnz / 2; i += n) reinterpret_cast<double2*>(A)[i] = make_double2(0.0, 0.0);
+  if (t == 0 && (nnz & 1)) A[nnz - 1] = 0.0;
+  for (int64_t i = t; i < nb; i += n) b[i] = 0.0;
+  if (t == 0 && counter) *counter = 0;
+}
+
+int zero_system(double* A, int64_t nnz, double* b, int64_t nb, int32_t* counter, cudaStream_t s) {
+  if (small_system(nnz)) {
+    const unsigned grid = (unsigned)std::min<int64_t>((nnz / 2 + nb) / 1024 + 1, 4 * 152);
+    k_zero_system<<<grid, 256, 0, s>>>(A, nnz, b, nb, counter);
+    FEA_CUDA(cudaGetLastError());
+    return FEA_OK;
+  }
+  FEA_CUDA(cudaMemsetAsync(A, 0, nnz * sizeof(double), s));
+  FEA_CUDA(cudaMemsetAsync(b, 0, nb * sizeof(double), s));
+  if (counter) FEA_CUDA(cudaMemsetAsync(counter, 0, sizeof(int32_t), s));
   return FEA_OK;
 }
 
@@ -1360,7 +1391,9 @@ int assemble_launches(const fea_operator* op, const fea_mesh* m, int* n) {
   }
   int k = 0;
   for (int t = 0; t < kNumTypes; ++t) k += m->group[t].n > 0;
-  *n = k;
+  // small systems are cleared by a kernel
+  const int D = op->kind == FEA_OP_DIFFUSION ? 1 : 3;
+  *n = k + (small_system((int64_t)D * D * m->nnz_node) ? 1 : 0);
   return FEA_OK;
 }
 

@@ -399,6 +399,11 @@ __device__ __forceinline__ void red_add(double* p, double v) {
 }
 
 
+// 32 zero bytes at a 32-byte aligned address
+__device__ __forceinline__ void zero32(double* p) {
+  asm volatile("st.global.v4.f64 [%0], {%1, %1, %1, %1};" ::"l"(__cvta_generic_to_global(p)), "d"(0.0) : "memory");
+}
+
 // add into A or b: FP64 atomic (ATOMIC, Alg. "no coloring"), or a plain
 // read-modify-write when no other element of the launch touches the entry
 // (COLOR: the launch holds one color class, Alg. "coloring")

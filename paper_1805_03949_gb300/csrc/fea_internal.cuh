@@ -149,7 +149,6 @@ void scan_tile_sums(int64_t* tile_sums, int64_t n, cudaStream_t s);  // exclusiv
 int build_node_graph(fea_mesh* m, cudaStream_t s);
 int write_csr_pattern(fea_mesh* m, int ndof, int64_t* row_ptr, int32_t* col_idx, int32_t* node_map,
                       cudaStream_t s);
-int exclusive_scan_i32(const int32_t* in, int64_t n, int64_t* out, cudaStream_t s);
 
 // assemble.cu
 int assemble(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, const int32_t* node_map,

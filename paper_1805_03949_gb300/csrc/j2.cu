@@ -334,6 +334,7 @@ __device__ __forceinline__ void j2_tile_body(Smem& sm, const RefRule& rr, const 
       });
   __syncthreads();
   if constexpr (!SCATTER) return;
+  if constexpr (SC == FEA_SCATTER_ATOMIC) wait_for_previous();
 
   // phase 2: lane a accumulates its row block
   if constexpr (SCATTER) {
@@ -544,6 +545,7 @@ __device__ __forceinline__ void j2_pair_body(typename J2PairCfg<TYPE, SLOT>::Sme
         j2_pair_point<Cfg>(sm, rr, P, le, q, et, J, Ju, s);
       });
   __syncthreads();
+  if constexpr (SC == FEA_SCATTER_ATOMIC) wait_for_previous();
   pair_rounds<Cfg>(
       sm, e0, n_end, [&](int le, int u, int v) { j2_pair_task<Cfg, SC, false>(sm, P, le, u, v); },
       [&](int le, int u) { j2_pair_task<Cfg, SC, true>(sm, P, le, u, u); });
@@ -577,6 +579,7 @@ template <int TYPE, int SLOT, int PREC, int SC, bool POINTS>
 __global__ void __launch_bounds__(128, POINTS || PREC == FEA_FP64 ? 0 : 5) k_j2_tile(const __grid_constant__ RefRule rr, const __grid_constant__ J2Params P) {
   using T = J2Tile<TYPE, SLOT, PREC, POINTS>;
   extern __shared__ __align__(16) unsigned char j2_smem_raw[];
+  if constexpr (!POINTS) let_next_start();
   T::template run<SC>(j2_smem_raw, rr, P, (int64_t)blockIdx.x * T::Cfg::EPC, P.n);
 }
 
@@ -587,8 +590,9 @@ static int launch_j2(const J2Params& P, cudaStream_t s) {
   static_assert(smem <= 227 * 1024, "J2 tile exceeds shared memory");
   auto kern = k_j2_tile<TYPE, SLOT, PREC, SC, POINTS>;
   if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<grid_for(P.n, T::Cfg::EPC), T::Cfg::THREADS, smem, s>>>(host_rule(SLOT), P);
-  FEA_CUDA(cudaGetLastError());
+  const unsigned grid = grid_for(P.n, T::Cfg::EPC);
+  const bool early = P.early && starts_early(grid, P.early == 1, false);
+  FEA_CUDA(launch_tiles(kern, grid, T::Cfg::THREADS, smem, s, early, host_rule(SLOT), P));
   return FEA_OK;
 }
 
@@ -801,17 +805,19 @@ int assemble_j2(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, con
   const int nev = ev ? op->n_events : 0;
   const int64_t nnz = 9 * m->nnz_node;
   if (nev > 0) FEA_CUDA(cudaEventRecord(ev[0], s));
-  FEA_CUDA(cudaMemsetAsync(A, 0, nnz * sizeof(double), s));
-  FEA_CUDA(cudaMemsetAsync(b, 0, m->n_nodes * 3 * sizeof(double), s));
+  int zrc = zero_system(A, nnz, b, m->n_nodes * 3, nullptr, s);
+  if (zrc) return zrc;
   if (nev > 1) FEA_CUDA(cudaEventRecord(ev[1], s));
 
   J2Params P = j2_base_params(op, m, row_ptr, node_map, A, b);
+  P.early = op->scatter == FEA_SCATTER_ATOMIC && small_system(nnz);
   int launched = 0;
   auto run = [&](int t) -> int {
     int rc = launch_j2_any(t, op->precision, op->scatter == FEA_SCATTER_COLOR, P, s);
     if (rc) return rc;
     if (2 + launched < nev) FEA_CUDA(cudaEventRecord(ev[2 + launched], s));
     ++launched;
+    if (P.early) P.early = 2;
     return FEA_OK;
   };
   if (op->scatter == FEA_SCATTER_COLOR) {
@@ -843,6 +849,7 @@ int assemble_j2(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, con
     int rc = run(t);
     if (rc) return rc;
   }
+  for (int k = 2 + launched; k < nev; ++k) FEA_CUDA(cudaEventRecord(ev[k], s));
   return FEA_OK;
 }
 
@@ -872,6 +879,7 @@ int element_loop_j2(const fea_operator* op, fea_mesh* m, double* stress, cudaStr
     if (rc) return rc;
     if (2 + launched < nev) FEA_CUDA(cudaEventRecord(ev[2 + launched], s));
     ++launched;
+    if (P.early) P.early = 2;
   }
   return FEA_OK;
 }

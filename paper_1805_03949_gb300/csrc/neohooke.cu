@@ -210,6 +210,7 @@ __device__ __forceinline__ void nh_tile_body(typename NHCfg<TYPE, SLOT>::Smem& s
         nh_point<Cfg>(sm, rr, P, le, q, et, J, Ju, s);
       });
   __syncthreads();
+  if constexpr (SC == FEA_SCATTER_ATOMIC) wait_for_previous();
 
   // phase 2: lane a accumulates its row block
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -402,6 +403,7 @@ __device__ __forceinline__ void nh_pair_body(typename NHPairCfg<TYPE, SLOT>::Sme
         nh_pair_point<Cfg>(sm, rr, P, le, q, et, J, Ju, s);
       });
   __syncthreads();
+  if constexpr (SC == FEA_SCATTER_ATOMIC) wait_for_previous();
   pair_rounds<Cfg>(
       sm, e0, n_end, [&](int le, int u, int v) { nh_pair_task<Cfg, SC, false>(sm, rr, P, le, u, v); },
       [&](int le, int u) { nh_pair_task<Cfg, SC, true>(sm, rr, P, le, u, u); });
@@ -430,6 +432,7 @@ template <int TYPE, int SLOT, int PREC, int SC>
 __global__ void __launch_bounds__(128, PREC == FEA_FP64 ? 0 : 5) k_nh_tile(const __grid_constant__ RefRule rr, const __grid_constant__ NHParams P) {
   using T = NHTile<TYPE, SLOT, PREC>;
   extern __shared__ __align__(16) unsigned char nh_smem_raw[];
+  let_next_start();
   T::template run<SC>(*reinterpret_cast<typename T::Cfg::Smem*>(nh_smem_raw), rr, P,
                       (int64_t)blockIdx.x * T::Cfg::EPC);
 }
@@ -441,8 +444,9 @@ static int launch_nh(const NHParams& P, cudaStream_t s) {
   static_assert(smem <= 227 * 1024, "finite-strain tile exceeds shared memory");
   auto kern = k_nh_tile<TYPE, SLOT, PREC, SC>;
   if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  kern<<<grid_for(P.n, Cfg::EPC), Cfg::THREADS, smem, s>>>(host_rule(SLOT), P);
-  FEA_CUDA(cudaGetLastError());
+  const unsigned grid = grid_for(P.n, Cfg::EPC);
+  const bool early = P.early && starts_early(grid, P.early == 1, false);
+  FEA_CUDA(launch_tiles(kern, grid, Cfg::THREADS, smem, s, early, host_rule(SLOT), P));
   return FEA_OK;
 }
 
@@ -472,8 +476,8 @@ int assemble_nh(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, con
   cudaEvent_t* ev = (cudaEvent_t*)op->events;
   const int nev = ev ? op->n_events : 0;
   if (nev > 0) FEA_CUDA(cudaEventRecord(ev[0], s));
-  FEA_CUDA(cudaMemsetAsync(A, 0, 9 * m->nnz_node * sizeof(double), s));
-  FEA_CUDA(cudaMemsetAsync(b, 0, m->n_nodes * 3 * sizeof(double), s));
+  const int zrc = zero_system(A, 9 * m->nnz_node, b, m->n_nodes * 3, nullptr, s);
+  if (zrc) return zrc;
   if (nev > 1) FEA_CUDA(cudaEventRecord(ev[1], s));
 
   NHParams P;
@@ -490,6 +494,7 @@ int assemble_nh(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, con
   P.mu = E / (2.0 * (1.0 + nu));
   P.mass = op->mass;
   const bool color = op->scatter == FEA_SCATTER_COLOR;
+  P.early = !color && small_system(9 * m->nnz_node);
   int launched = 0;
   auto run = [&](int t) -> int {
     int rc;
@@ -502,6 +507,7 @@ int assemble_nh(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, con
     if (rc) return rc;
     if (2 + launched < nev) FEA_CUDA(cudaEventRecord(ev[2 + launched], s));
     ++launched;
+    if (P.early) P.early = 2;
     return FEA_OK;
   };
   if (color) {
@@ -533,6 +539,7 @@ int assemble_nh(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, con
     int rc = run(t);
     if (rc) return rc;
   }
+  for (int k = 2 + launched; k < nev; ++k) FEA_CUDA(cudaEventRecord(ev[k], s));
   return FEA_OK;
 }
 

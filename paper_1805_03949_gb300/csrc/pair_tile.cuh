@@ -233,6 +233,7 @@ __device__ __forceinline__ void pair_tile_body(typename PairCfg<TYPE, SLOT, OP>:
                                                const AsmParams& P, int64_t e0, int64_t n_end) {
   using Cfg = PairCfg<TYPE, SLOT, OP>;
   pair_geometry<Cfg, OP>(sm, rr, P, e0, n_end);
+  if constexpr (SC == FEA_SCATTER_ATOMIC) wait_for_previous();
   pair_rounds<Cfg>(
       sm, e0, n_end, [&](int le, int u, int v) { pair_task<Cfg, OP, SC, false>(sm, rr, P, le, u, v); },
       [&](int le, int u) { pair_task<Cfg, OP, SC, true>(sm, rr, P, le, u, u); });

@@ -13,6 +13,7 @@
 #pragma once
 
 #include "element.cuh"
+#include "zero.cuh"
 
 namespace fea {
 
@@ -29,6 +30,7 @@ struct ElemParams {
   double* A;
   double* b;
   DevStatus* st;
+  int early;                // host: tile kernels may start early (zero.cuh): 1 after the clearing, 2 after a type
 };
 
 // (Params: const ElemParams or a derived struct, volatile where its fields are

@@ -18,6 +18,7 @@
 // decide the order of the incidence lists, which no output depends on, and
 // those of step 2 the order in which the distinct nodes are found, which the
 // ranking removes.
+#include <algorithm>
 #include <cstdio>
 #include <mutex>
 #include <string>
@@ -114,16 +115,15 @@ void scan_tile_sums(int64_t* tile_sums, int64_t n, cudaStream_t s) {
   k_scan_tiles<<<1, kScanBlock, 0, s>>>(tile_sums, n);
 }
 
-int exclusive_scan_i32(const int32_t* in, int64_t n, int64_t* out, cudaStream_t s) {
-  int64_t ntiles = (n + kScanTile - 1) / kScanTile;
-  if (ntiles < 1) ntiles = 1;
-  int64_t* tiles = nullptr;
-  FEA_CUDA(cudaMallocAsync(&tiles, ntiles * sizeof(int64_t), s));
+// tiles: scratch of scan_tiles(n) values
+static int64_t scan_tiles(int64_t n) { return std::max<int64_t>((n + kScanTile - 1) / kScanTile, 1); }
+
+static int exclusive_scan_i32(const int32_t* in, int64_t n, int64_t* out, int64_t* tiles, cudaStream_t s) {
+  const int64_t ntiles = scan_tiles(n);
   k_scan_reduce<<<(unsigned)ntiles, kScanBlock, 0, s>>>(in, n, tiles);
   k_scan_tiles<<<1, kScanBlock, 0, s>>>(tiles, ntiles);
   k_scan_apply<<<(unsigned)ntiles, kScanBlock, 0, s>>>(in, n, tiles, out);
   FEA_CUDA(cudaGetLastError());
-  FEA_CUDA(cudaFreeAsync(tiles, s));
   return FEA_OK;
 }
 
@@ -356,25 +356,27 @@ static void drop_graph(fea_mesh* m) {
 
 static int node_graph(fea_mesh* m, cudaStream_t s) {
   const int64_t N = m->n_nodes, E = m->n_elems, L = m->conn_len;
-  // one allocation: incidence offsets and lists, row pointers, and two
-  // int32 work arrays (counts, then row lengths; the nodes of many elements)
-  const size_t a_inc = (size_t)(N + 1) * 8, a_rp = a_inc + (size_t)L * 8, a_cnt = a_rp + (size_t)(N + 1) * 8,
-               a_todo = a_cnt + (size_t)N * 4;
+  // one allocation: incidence offsets and lists, row pointers, the scans'
+  // scratch, and two int32 work arrays (counts, then row lengths; the nodes of
+  // many elements)
+  const size_t a_inc = (size_t)(N + 1) * 8, a_rp = a_inc + (size_t)L * 8, a_tiles = a_rp + (size_t)(N + 1) * 8,
+               a_cnt = a_tiles + (size_t)scan_tiles(N) * 8, a_todo = a_cnt + (size_t)N * 4;
   FEA_CUDA(cudaMalloc((void**)&m->graph, a_todo + (size_t)(N + 1) * 4));
   m->inc_off = reinterpret_cast<int64_t*>(m->graph);
   m->inc = reinterpret_cast<int64_t*>(m->graph + a_inc);
   m->rp_node = reinterpret_cast<int64_t*>(m->graph + a_rp);
+  int64_t* tiles = reinterpret_cast<int64_t*>(m->graph + a_tiles);
   int32_t* cnt = reinterpret_cast<int32_t*>(m->graph + a_cnt);
   int32_t* todo = reinterpret_cast<int32_t*>(m->graph + a_todo);
   FEA_CUDA(cudaMemsetAsync(cnt, 0, N * sizeof(int32_t), s));
   k_inc_count<<<grid_for(L, 256), 256, 0, s>>>(m->conn, L, cnt);
-  int rc = exclusive_scan_i32(cnt, N, m->inc_off, s);
+  int rc = exclusive_scan_i32(cnt, N, m->inc_off, tiles, s);
   if (rc) return rc;
   k_inc_fill<<<grid_for(E, 256), 256, 0, s>>>(m->conn_off, m->conn, E, m->inc_off, cnt, m->inc);
   const RowMesh M = row_mesh(m);
   rc = launch_rows<false>(m, M, cnt, todo, s);
   if (rc) return rc;
-  rc = exclusive_scan_i32(cnt, N, m->rp_node, s);
+  rc = exclusive_scan_i32(cnt, N, m->rp_node, tiles, s);
   if (rc) return rc;
   FEA_CUDA(cudaMemcpyAsync(&m->nnz_node, m->rp_node + N, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   int code = 0;
@@ -419,7 +421,7 @@ int write_csr_pattern(fea_mesh* m, int ndof, int64_t* row_ptr, int32_t* col_idx,
 // ---------------------------------------------------------------------------
 // Row pointers from row lengths without any device allocation.
 //
-// The scan above takes its per-tile partial sums from a stream-ordered
+// The scan above takes its per-tile partial sums from the mesh handle's
 // allocation.  Callers that hand all device memory to their own pool up
 // front, or that must not let a library allocate on their behalf, use
 // fea_row_ptr_from_counts_noalloc instead: the tile sums live in the

@@ -650,11 +650,6 @@ int assemble_rows(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, d
   return rc;
 }
 
-// 32 zero bytes at a 32-byte aligned address
-__device__ __forceinline__ void zero32(double* p) {
-  asm volatile("st.global.v4.f64 [%0], {%1, %1, %1, %1};" ::"l"(__cvta_generic_to_global(p)), "d"(0.0) : "memory");
-}
-
 // A warp per run of nodes: their rows of A, [row_ptr[D first], row_ptr[D
 // (first + count)]), are contiguous; zeroed with 32-byte stores from the
 // first 32-byte boundary on, single values before it and after the last one.
