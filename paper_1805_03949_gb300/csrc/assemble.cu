@@ -26,6 +26,7 @@
 #include "coop_scatter.cuh"
 #include "element.cuh"
 #include "fea_internal.cuh"
+#include "hex_diffusion.cuh"
 #include "pair_tile.cuh"
 #include "sched.cuh"
 
@@ -671,6 +672,17 @@ struct Tile<TYPE, SLOT, OP, FEA_FP64> {
   __device__ static __forceinline__ void run(unsigned char* raw, const RefRule& rr, const AsmParams& P, int64_t e0,
                                              int64_t n_end) {
     pair_tile_body<TYPE, SLOT, OP, SC>(*reinterpret_cast<Smem*>(raw), rr, P, e0, n_end);
+  }
+  static constexpr int min_blocks(int) { return 0; }
+};
+template <>
+struct Tile<FEA_HEX8, kRuleHex8, FEA_OP_DIFFUSION, FEA_FP64> {
+  using Cfg = HexDiffusionCfg;
+  using Smem = Cfg::Smem;
+  template <int SC, bool COOP>
+  __device__ static __forceinline__ void run(unsigned char* raw, const RefRule& rr, const AsmParams& P, int64_t e0,
+                                             int64_t n_end) {
+    hex_diffusion_body<SC>(*reinterpret_cast<Smem*>(raw), rr, P, e0, n_end);
   }
   static constexpr int min_blocks(int) { return 0; }
 };

@@ -14,7 +14,8 @@
 //    pairs) make one set of gradients, with their weights summed first.
 // Measured on one GB300, before and after: 250,047 hex8, elasticity 8.82 ->
 // 1.95 ms; 162,000 tet4, elasticity 0.776 -> 0.137 ms; 412,500 mixed elements,
-// diffusion 1.53 -> 0.94 ms.
+// diffusion 1.53 -> 0.94 ms (0.85 with RefMap; hex8 diffusion has its own tile,
+// hex_diffusion.cuh).
 #pragma once
 
 #include "pairs.cuh"
