@@ -348,7 +348,6 @@ struct TileCfg {
   static constexpr int WARPS = 4;
   static constexpr int THREADS = 32 * WARPS;
   static constexpr int EPC = EPW * WARPS;       // elements per CTA
-  static constexpr int NB = column_group(NN, D);  // columns per lane at a time
   static constexpr bool kModal = TYPE == FEA_HEX8 && SLOT == kRuleHex8;
   static_assert(!kModal || (EPC * 8 % 32 == 0 && EPC * 8 <= THREADS), "modal hex geometry needs whole warps");
   using Smem = TileSmem<OP, NN, NQ, EPC>;
@@ -511,12 +510,12 @@ __device__ __forceinline__ void tile_geometry(typename Cfg::Smem& sm, const RefR
 
 // phase 2: columns b0 .. b0 + NB of the row block of node a of element le,
 // and with the first columns its RHS
-template <class Cfg, int OP, class Params>
+template <class Cfg, int OP, int NB, class Params>
 __device__ __forceinline__ void row_block(const typename Cfg::Smem& sm, const RefRule& rr, Params& P,
-                                          int le, int a, int b0, float (&K)[Cfg::NB][Cfg::D][Cfg::D],
+                                          int le, int a, int b0, float (&K)[NB][Cfg::D][Cfg::D],
                                           float (&rhs)[Cfg::D]) {
   using R = float;
-  constexpr int NB = Cfg::NB, D = Cfg::D, NQ = Cfg::NQ;
+  constexpr int D = Cfg::D, NQ = Cfg::NQ;
 #pragma unroll
   for (int bb = 0; bb < NB; ++bb)
 #pragma unroll
@@ -577,7 +576,7 @@ __device__ __forceinline__ void tile_body(typename TileCfg<TYPE, SLOT, OP>::Smem
                                           Params& P, int64_t e0, int64_t n_end) {
   using Cfg = TileCfg<TYPE, SLOT, OP>;
   using R = float;
-  constexpr int NN = Cfg::NN, D = Cfg::D, NB = Cfg::NB, LPE = Cfg::LPE, EPW = Cfg::EPW;
+  constexpr int NN = Cfg::NN, D = Cfg::D, NB = column_group(NN, D, SC), LPE = Cfg::LPE, EPW = Cfg::EPW;
   tile_geometry<Cfg, OP>(sm, rr, P, e0, n_end);
   if constexpr (SC == FEA_SCATTER_ATOMIC) wait_for_previous();
 
@@ -638,13 +637,15 @@ __device__ __forceinline__ void tile_body(typename TileCfg<TYPE, SLOT, OP>::Smem
         }
       }
     }
+    if constexpr (SC == FEA_SCATTER_MULTIDEP) {
+      double ob[D];
 #pragma unroll
-    for (int c = 0; c < D; ++c) {
-      double* p = P.b + D * node + c;
-      if constexpr (SC == FEA_SCATTER_MULTIDEP)
-        __stcg(p, __ldcg(p) + widen(rhs[c]));
-      else
-        scatter_add<SC>(p, widen(rhs[c]));
+      for (int c = 0; c < D; ++c) ob[c] = __ldcg(P.b + D * node + c);
+#pragma unroll
+      for (int c = 0; c < D; ++c) __stcg(P.b + D * node + c, ob[c] + widen(rhs[c]));
+    } else {
+#pragma unroll
+      for (int c = 0; c < D; ++c) scatter_add<SC>(P.b + D * node + c, widen(rhs[c]));
     }
   }
   __syncthreads();
@@ -890,7 +891,7 @@ __device__ int mdep_next(const MdepArgs& A, int& cursor) {
 }
 
 template <int OP, int PREC, int ONLY>
-__global__ void __launch_bounds__(128) k_multidep(const __grid_constant__ MdepArgs A) {
+__global__ void __launch_bounds__(128, PREC == FEA_FP64 ? 0 : OP == FEA_OP_DIFFUSION ? 5 : 3) k_multidep(const __grid_constant__ MdepArgs A) {
   constexpr int MD = FEA_SCATTER_MULTIDEP;
   extern __shared__ __align__(16) unsigned char mdep_smem[];
   __shared__ int s_sub;
@@ -1087,6 +1088,9 @@ static int launch_multidep_k(const MdepArgs& args, int n_ctas, cudaStream_t s) {
     FEA_CUDA(cudaGetDevice(&dev));
     FEA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     FEA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128, smem));
+    // more CTAs than these only try for locks that others hold (2.1 M hex8,
+    // FP32 elasticity: 14.6 ms with three per SM, 16.0 with four)
+    if (PREC != FEA_FP64) per_sm = std::min(per_sm, OP == FEA_OP_DIFFUSION ? 5 : 3);
     grid = sms * (per_sm > 0 ? per_sm : 1);
   }
   if (grid > args.n_sub) grid = args.n_sub;
@@ -1215,8 +1219,8 @@ int assemble(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, const 
     cudaEvent_t* ev = (cudaEvent_t*)op->events;
     const int nev = ev ? op->n_events : 0;
     if (nev > 0) FEA_CUDA(cudaEventRecord(ev[0], s));
-    rc = zero_system(A, (int64_t)D * D * m->nnz_node, b, m->n_nodes * D, nullptr, s);
-    if (rc) return rc;
+    FEA_CUDA(cudaMemsetAsync(A, 0, (int64_t)D * D * m->nnz_node * sizeof(double), s));
+    FEA_CUDA(cudaMemsetAsync(b, 0, m->n_nodes * D * sizeof(double), s));
     if (nev > 1) FEA_CUDA(cudaEventRecord(ev[1], s));
     rc = launch_multidep(op, m, *plan, row_ptr, node_map, A, b, s);
     if (rc) return rc;

@@ -20,9 +20,12 @@ __host__ __device__ constexpr int grad_stride(int nn) { return (3 * nn) | 1; }
 // taking turns.  In groups of four (prisms three) the tiles fit six CTAs
 // (elasticity: 682 us per step of 258,048 hex8 at 4, 614 at 5, 564 at 6, 590 at
 // 7) or five (J2, finite strain: more would not fit the shared memory), at the
-// cost of reading the row's own gradient once per group.
-__host__ __device__ constexpr int column_group(int nn, int dofs) {
-  return dofs == 1 ? nn : nn == 8 ? 4 : nn == 6 ? 3 : nn;
+// cost of reading the row's own gradient once per group.  Only with
+// reductions: a coloring or multidependence launch waits for the
+// read-modify-writes of each group (hex8, FP32, grouped: elasticity 1.29
+// against 1.20 ms, finite strain 0.93 against 0.62).
+__host__ __device__ constexpr int column_group(int nn, int dofs, int sc) {
+  return dofs == 1 || sc != FEA_SCATTER_ATOMIC ? nn : nn == 8 ? 4 : nn == 6 ? 3 : nn;
 }
 
 // Warp-cooperative reduction of FP32 row blocks.  A lane's row block holds, for
@@ -40,7 +43,7 @@ __host__ __device__ constexpr int column_group(int nn, int dofs) {
 template <int NN, int SC>
 struct CoopScatter {
   static constexpr bool kOn = SC == FEA_SCATTER_ATOMIC;
-  static constexpr int NB = column_group(NN, 3);
+  static constexpr int NB = column_group(NN, 3, FEA_SCATTER_ATOMIC);
   static constexpr int kVals = 32 * 3 * NB;  // floats a warp stages (16-byte aligned)
   // what a warp knows of its lanes' rows
   struct Rows {

@@ -73,7 +73,6 @@ struct J2Cfg {
   static constexpr int WARPS = 4;
   static constexpr int THREADS = 32 * WARPS;
   static constexpr int EPC = EPW * WARPS;
-  static constexpr int NB = column_group(NN, 3);  // columns per lane at a time
   static constexpr bool kHex = TYPE == FEA_HEX8;
   static_assert(!kHex || (EPC * 8 % 32 == 0 && EPC * 8 <= THREADS), "modal hex geometry needs whole warps");
   // what the Gauss-point update of the element loop needs
@@ -311,7 +310,8 @@ template <int TYPE, int SLOT, int SC, bool SCATTER, class Smem>
 __device__ __forceinline__ void j2_tile_body(Smem& sm, const RefRule& rr, const J2Params& P, int64_t e0,
                                              int64_t n_end) {
   using Cfg = J2Cfg<TYPE, SLOT>;
-  constexpr int NN = Cfg::NN, NQ = Cfg::NQ, EPC = Cfg::EPC, NB = Cfg::NB, LPE = Cfg::LPE, EPW = Cfg::EPW;
+  constexpr int NN = Cfg::NN, NQ = Cfg::NQ, EPC = Cfg::EPC, LPE = Cfg::LPE, EPW = Cfg::EPW;
+  constexpr int NB = column_group(NN, 3, SC);  // columns a lane accumulates at a time
   // phase 0: coordinates and displacements of the tile's nodes
   for (int t = threadIdx.x; t < EPC * NN; t += Cfg::THREADS) {
     const int le = t / NN, a = t % NN;
@@ -398,12 +398,15 @@ __device__ __forceinline__ void j2_tile_body(Smem& sm, const RefRule& rr, const 
       } else if (active) {
         const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
         const int32_t* mp = P.node_map + (P.mapoff ? P.mapoff[g] : id * NN * NN) + a * NN + b0;
+        int64_t rb[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) rb[c] = P.row_ptr[3 * node + c];
 #pragma unroll
         for (int bb = 0; bb < NB; ++bb) {
           const int64_t k = mp[bb];
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
-            double* row = P.A + P.row_ptr[3 * node + c] + 3 * k;
+            double* row = P.A + rb[c] + 3 * k;
 #pragma unroll
             for (int cc = 0; cc < 3; ++cc) scatter_add<SC>(row + cc, widen(K[bb][c][cc]));
           }
@@ -576,7 +579,8 @@ struct J2Tile<TYPE, SLOT, FEA_FP64, false> {
 
 // one tile per CTA
 template <int TYPE, int SLOT, int PREC, int SC, bool POINTS>
-__global__ void __launch_bounds__(128, POINTS || PREC == FEA_FP64 ? 0 : 5) k_j2_tile(const __grid_constant__ RefRule rr, const __grid_constant__ J2Params P) {
+__global__ void __launch_bounds__(128, POINTS || PREC == FEA_FP64 || SC != FEA_SCATTER_ATOMIC ? 0 : 5)
+    k_j2_tile(const __grid_constant__ RefRule rr, const __grid_constant__ J2Params P) {
   using T = J2Tile<TYPE, SLOT, PREC, POINTS>;
   extern __shared__ __align__(16) unsigned char j2_smem_raw[];
   if constexpr (!POINTS) let_next_start();

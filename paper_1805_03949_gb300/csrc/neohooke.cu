@@ -55,7 +55,6 @@ struct NHCfg {
   static constexpr int WARPS = 4;
   static constexpr int THREADS = 32 * WARPS;
   static constexpr int EPC = EPW * WARPS;
-  static constexpr int NB = column_group(NN, 3);  // columns per lane at a time
   static constexpr bool kHex = TYPE == FEA_HEX8;
   static_assert(!kHex || (EPC * 8 % 32 == 0 && EPC * 8 <= THREADS), "modal hex geometry needs whole warps");
   struct Smem {
@@ -65,7 +64,11 @@ struct NHCfg {
     float H[EPC][NQ][grad_stride(NN)];  // h_a = F^-T g_a
     float C[EPC][NQ][4];      // W mu, W lam, W (mu - lam ln J), W m
     float S[EPC][NQ][9];      // W P, row-major
-    typename CoopScatter<NN, FEA_SCATTER_ATOMIC>::Rows rows[WARPS];  // (the cooperative scatter's)
+  };
+  // with the cooperative scatter's rows (a plain read-modify-write scatter has
+  // the L1 cache that they would take)
+  struct CoopSmem : Smem {
+    typename CoopScatter<NN, FEA_SCATTER_ATOMIC>::Rows rows[WARPS];
   };
 };
 
@@ -184,11 +187,12 @@ __device__ __forceinline__ void nh_point(typename Cfg::Smem& sm, const RefRule& 
 
 // One FP32 tile of EPC elements from launch index e0 (elements at or past
 // n_end are skipped).  Every thread of the CTA calls it; it ends with a barrier.
-template <int TYPE, int SLOT, int SC>
-__device__ __forceinline__ void nh_tile_body(typename NHCfg<TYPE, SLOT>::Smem& sm, const RefRule& rr,
-                                             const NHParams& P, int64_t e0, int64_t n_end) {
+template <int TYPE, int SLOT, int SC, class Smem>
+__device__ __forceinline__ void nh_tile_body(Smem& sm, const RefRule& rr, const NHParams& P, int64_t e0,
+                                             int64_t n_end) {
   using Cfg = NHCfg<TYPE, SLOT>;
-  constexpr int NN = Cfg::NN, NQ = Cfg::NQ, EPC = Cfg::EPC, NB = Cfg::NB, LPE = Cfg::LPE, EPW = Cfg::EPW;
+  constexpr int NN = Cfg::NN, NQ = Cfg::NQ, EPC = Cfg::EPC, LPE = Cfg::LPE, EPW = Cfg::EPW;
+  constexpr int NB = column_group(NN, 3, SC);  // columns a lane accumulates at a time
   // phase 0: coordinates and displacements of the tile's nodes
   for (int t = threadIdx.x; t < EPC * NN; t += Cfg::THREADS) {
     const int le = t / NN, a = t % NN;
@@ -273,12 +277,15 @@ __device__ __forceinline__ void nh_tile_body(typename NHCfg<TYPE, SLOT>::Smem& s
     } else if (active) {
       const int64_t id = P.ids ? (int64_t)P.ids[g] : g;
       const int32_t* mp = P.node_map + (P.mapoff ? P.mapoff[g] : id * NN * NN) + a * NN + b0;
+      int64_t rb[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) rb[c] = P.row_ptr[3 * node + c];
 #pragma unroll
       for (int bb = 0; bb < NB; ++bb) {
         const int64_t k = mp[bb];
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-          double* row = P.A + P.row_ptr[3 * node + c] + 3 * k;
+          double* row = P.A + rb[c] + 3 * k;
 #pragma unroll
           for (int cc = 0; cc < 3; ++cc) scatter_add<SC>(row + cc, widen(K[bb][c][cc]));
         }
@@ -415,7 +422,9 @@ template <int TYPE, int SLOT, int PREC>
 struct NHTile {
   using Cfg = NHCfg<TYPE, SLOT>;
   template <int SC>
-  __device__ static __forceinline__ void run(typename Cfg::Smem& sm, const RefRule& rr, const NHParams& P, int64_t e0) {
+  using Smem = std::conditional_t<SC == FEA_SCATTER_ATOMIC, typename Cfg::CoopSmem, typename Cfg::Smem>;
+  template <int SC>
+  __device__ static __forceinline__ void run(Smem<SC>& sm, const RefRule& rr, const NHParams& P, int64_t e0) {
     nh_tile_body<TYPE, SLOT, SC>(sm, rr, P, e0, P.n);
   }
 };
@@ -423,24 +432,27 @@ template <int TYPE, int SLOT>
 struct NHTile<TYPE, SLOT, FEA_FP64> {
   using Cfg = NHPairCfg<TYPE, SLOT>;
   template <int SC>
-  __device__ static __forceinline__ void run(typename Cfg::Smem& sm, const RefRule& rr, const NHParams& P, int64_t e0) {
+  using Smem = typename Cfg::Smem;
+  template <int SC>
+  __device__ static __forceinline__ void run(Smem<SC>& sm, const RefRule& rr, const NHParams& P, int64_t e0) {
     nh_pair_body<TYPE, SLOT, SC>(sm, rr, P, e0, P.n);
   }
 };
 
 template <int TYPE, int SLOT, int PREC, int SC>
-__global__ void __launch_bounds__(128, PREC == FEA_FP64 ? 0 : 5) k_nh_tile(const __grid_constant__ RefRule rr, const __grid_constant__ NHParams P) {
+__global__ void __launch_bounds__(128, PREC == FEA_FP64 || SC != FEA_SCATTER_ATOMIC ? 0 : 5)
+    k_nh_tile(const __grid_constant__ RefRule rr, const __grid_constant__ NHParams P) {
   using T = NHTile<TYPE, SLOT, PREC>;
   extern __shared__ __align__(16) unsigned char nh_smem_raw[];
   let_next_start();
-  T::template run<SC>(*reinterpret_cast<typename T::Cfg::Smem*>(nh_smem_raw), rr, P,
+  T::template run<SC>(*reinterpret_cast<typename T::template Smem<SC>*>(nh_smem_raw), rr, P,
                       (int64_t)blockIdx.x * T::Cfg::EPC);
 }
 
 template <int TYPE, int SLOT, int PREC, int SC>
 static int launch_nh(const NHParams& P, cudaStream_t s) {
   using Cfg = typename NHTile<TYPE, SLOT, PREC>::Cfg;
-  constexpr size_t smem = sizeof(typename Cfg::Smem);
+  constexpr size_t smem = sizeof(typename NHTile<TYPE, SLOT, PREC>::template Smem<SC>);
   static_assert(smem <= 227 * 1024, "finite-strain tile exceeds shared memory");
   auto kern = k_nh_tile<TYPE, SLOT, PREC, SC>;
   if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));

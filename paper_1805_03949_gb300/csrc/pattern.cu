@@ -359,10 +359,17 @@ static int node_graph(fea_mesh* m, cudaStream_t s) {
   // one allocation: incidence offsets and lists, row pointers, the scans'
   // scratch, and two int32 work arrays (counts, then row lengths; the nodes of
   // many elements)
-  const size_t a_inc = (size_t)(N + 1) * 8, a_rp = a_inc + (size_t)L * 8, a_tiles = a_rp + (size_t)(N + 1) * 8,
-               a_cnt = a_tiles + (size_t)scan_tiles(N) * 8, a_todo = a_cnt + (size_t)N * 4;
-  FEA_CUDA(cudaMalloc((void**)&m->graph, a_todo + (size_t)(N + 1) * 4));
-  m->inc_off = reinterpret_cast<int64_t*>(m->graph);
+  size_t bytes = 0;
+  auto place = [&](size_t n) {
+    const size_t at = bytes;
+    bytes += (n + 255) & ~(size_t)255;
+    return at;
+  };
+  const size_t a_off = place((size_t)(N + 1) * 8), a_inc = place((size_t)L * 8), a_rp = place((size_t)(N + 1) * 8),
+               a_tiles = place((size_t)scan_tiles(N) * 8), a_cnt = place((size_t)N * 4),
+               a_todo = place((size_t)(N + 1) * 4);
+  FEA_CUDA(cudaMalloc((void**)&m->graph, bytes));
+  m->inc_off = reinterpret_cast<int64_t*>(m->graph + a_off);
   m->inc = reinterpret_cast<int64_t*>(m->graph + a_inc);
   m->rp_node = reinterpret_cast<int64_t*>(m->graph + a_rp);
   int64_t* tiles = reinterpret_cast<int64_t*>(m->graph + a_tiles);

@@ -47,6 +47,10 @@ __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontr
 template <class Kernel, class... Args>
 cudaError_t launch_tiles(Kernel kern, unsigned grid, unsigned threads, size_t smem, cudaStream_t s, bool early,
                          const Args&... args) {
+  if (!early) {
+    kern<<<grid, threads, smem, s>>>(args...);
+    return cudaGetLastError();
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(threads);
@@ -56,7 +60,7 @@ cudaError_t launch_tiles(Kernel kern, unsigned grid, unsigned threads, size_t sm
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
-  cfg.numAttrs = early ? 1 : 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
