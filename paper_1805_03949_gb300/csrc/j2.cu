@@ -33,8 +33,8 @@
 //  * reciprocals of det J, of the Newton slope and of the norm are rcp64, and
 //    constant divisors are the host's factors;
 //  * the element loop forms no tile factors (they go nowhere there).
-// 499,200 hex8, element loop, one GB300: 2.24 -> 1.63 ms; 373,248 hex8, FP32
-// assembly: 2.20 -> 1.96 ms.
+// 499,200 hex8, element loop, one GB300: 2.18 -> 1.58 ms; 373,248 hex8, FP32
+// assembly: 2.24 -> 1.75 ms with the scatter of coop_scatter.cuh.
 #include <cmath>
 #include <cstring>
 #include <type_traits>
