@@ -163,6 +163,18 @@ def variant_operators(fea) -> dict:
             for name, (prec, sc) in VARIANTS.items()}
 
 
+def kernels_after_zeroing(fea, system, name, launches):
+    """Of a variant's `launches` per step on a hex8 mesh, those after the zeroing interval of the events: block-task
+    plans clear the rows of A they add to, and the launches per element type a small system, with one kernel inside
+    that interval."""
+    kind = name.split("_", 1)[1]
+    if kind == "atomic":
+        return 1                                        # one element type, one tile launch
+    if kind == "color":
+        return fea.fea_color_info(system.handle, system.n_elems)[0]
+    return launches - 1 if kind == "block" else launches
+
+
 def hex_cube_mesh(n=128):
     """The headline workload's mesh: n^3 hex8 cube, interior nodes jittered by +-0.2h (PCG64 seed 2)."""
     from paper_1805_03949_gb300 import meshgen as mg
@@ -466,9 +478,7 @@ def run_ours(args, rank, world, local_rank):
             tuned[name] = fea.fea_autotune(op, sysm.handle, sysm.row_ptr, sysm.node_map, sysm.A, sysm.b, 5)
             tuned[name]["seconds"] = time.perf_counter() - t0
         nk = fea.fea_assemble_launches(op, sysm.handle)     # every kernel of the step
-        # block-task plans clear the rows of A they add to with one kernel,
-        # inside the zeroing interval of the events below
-        post = nk - 1 if name.endswith("block") else nk
+        post = kernels_after_zeroing(fea, sysm, name, nk)
         steps = args.steps if name.startswith("fp32") else max(3, min(args.steps, 5))
         # one set of profiling events per timed step: events[0] before zeroing, [1] after,
         # [2 + j] after the j-th kernel after the zeroing

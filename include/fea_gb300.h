@@ -167,7 +167,7 @@ typedef struct {
  *  events     optional profiling hook (NULL to skip): cudaEvent_t handles the
  *             call records on its stream -- events[0] before zeroing A and b,
  *             events[1] after zeroing, events[2 + j] after the j-th kernel it
- *             launches (only those with index < n_events are recorded).
+ *             launches after that (only those with index < n_events are recorded).
  *  schedule   fea_schedule (FEA_SCATTER_ATOMIC only for the persistent ones)
  *  chunk      elements per work item (persistent schedules) and per subdomain
  *             (FEA_SCATTER_MULTIDEP); 0 = 128
@@ -569,7 +569,11 @@ int fea_multidep_hold(fea_mesh* mesh, int subdomain, int held);
 int fea_color_info(const fea_mesh* mesh, int32_t* colors_h, int* n_colors);
 
 /* Number of kernels one fea_assemble call with this operator launches on this
- * mesh (after its pattern is built).  Service; host call. */
+ * mesh (after its pattern is built).  The kernel that clears the rows of A of a
+ * FEA_SCATTER_BLOCK plan, or A and b of a small system (A up to 32 MB) under
+ * FEA_SCATTER_ATOMIC and FEA_SCATTER_COLOR with FEA_SCHED_PER_TYPE, is one of
+ * them, though it runs between events[0] and events[1]; elsewhere memsets
+ * clear.  Service; host call. */
 int fea_assemble_launches(const fea_operator* op, const fea_mesh* mesh, int* n_kernels);
 
 /* Wait for the stream and return the mesh's latched device status (and clear

@@ -1272,7 +1272,7 @@ int assemble(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, const 
     if (rc) return rc;
     FEA_CUDA(cudaMemsetAsync(b, 0, m->n_nodes * D * sizeof(double), s));
   } else {
-    int rc = zero_system(A, nnz, b, m->n_nodes * D, nullptr, s);
+    int rc = zero_system(A, nnz, b, m->n_nodes * D, s);
     if (rc) return rc;
   }
   if (nev > 1) FEA_CUDA(cudaEventRecord(ev[1], s));
@@ -1360,26 +1360,24 @@ int assemble(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, const 
   return FEA_OK;
 }
 
-__global__ void __launch_bounds__(256) k_zero_system(double* A, int64_t nnz, double* b, int64_t nb, int32_t* counter) {
+__global__ void __launch_bounds__(256) k_zero_system(double* A, int64_t nnz, double* b, int64_t nb) {
   let_next_start();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, n = (int64_t)gridDim.x * blockDim.x;
   // A is 16-byte aligned
   for (int64_t i = t; i < nnz / 2; i += n) reinterpret_cast<double2*>(A)[i] = make_double2(0.0, 0.0);
   if (t == 0 && (nnz & 1)) A[nnz - 1] = 0.0;
   for (int64_t i = t; i < nb; i += n) b[i] = 0.0;
-  if (t == 0 && counter) *counter = 0;
 }
 
-int zero_system(double* A, int64_t nnz, double* b, int64_t nb, int32_t* counter, cudaStream_t s) {
+int zero_system(double* A, int64_t nnz, double* b, int64_t nb, cudaStream_t s) {
   if (small_system(nnz)) {
     const unsigned grid = (unsigned)std::min<int64_t>((nnz / 2 + nb) / 1024 + 1, 4 * 152);
-    k_zero_system<<<grid, 256, 0, s>>>(A, nnz, b, nb, counter);
+    k_zero_system<<<grid, 256, 0, s>>>(A, nnz, b, nb);
     FEA_CUDA(cudaGetLastError());
     return FEA_OK;
   }
   FEA_CUDA(cudaMemsetAsync(A, 0, nnz * sizeof(double), s));
   FEA_CUDA(cudaMemsetAsync(b, 0, nb * sizeof(double), s));
-  if (counter) FEA_CUDA(cudaMemsetAsync(counter, 0, sizeof(int32_t), s));
   return FEA_OK;
 }
 
@@ -1400,16 +1398,16 @@ int assemble_launches(const fea_operator* op, const fea_mesh* m, int* n) {
     if (op->scatter == FEA_SCATTER_BLOCK && !(m->blocks && m->blocks->n_zero_runs == 0)) *n += 1;
     return FEA_OK;
   }
+  // the tile launches, and the kernel that clears a small system before them
+  const int D = op->kind == FEA_OP_DIFFUSION ? 1 : 3;
+  int k = small_system((int64_t)D * D * m->nnz_node) ? 1 : 0;
   if (op->scatter == FEA_SCATTER_COLOR) {
     if (!m->color) return fail(FEA_ERR_ARG, "fea_assemble_launches: the coloring is built by the first COLOR call");
-    *n = color_launches(m);
-    return FEA_OK;
+    k += color_launches(m);
+  } else {
+    for (int t = 0; t < kNumTypes; ++t) k += m->group[t].n > 0;
   }
-  int k = 0;
-  for (int t = 0; t < kNumTypes; ++t) k += m->group[t].n > 0;
-  // small systems are cleared by a kernel
-  const int D = op->kind == FEA_OP_DIFFUSION ? 1 : 3;
-  *n = k + (small_system((int64_t)D * D * m->nnz_node) ? 1 : 0);
+  *n = k;
   return FEA_OK;
 }
 

@@ -809,7 +809,7 @@ int assemble_j2(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, con
   const int nev = ev ? op->n_events : 0;
   const int64_t nnz = 9 * m->nnz_node;
   if (nev > 0) FEA_CUDA(cudaEventRecord(ev[0], s));
-  int zrc = zero_system(A, nnz, b, m->n_nodes * 3, nullptr, s);
+  int zrc = zero_system(A, nnz, b, m->n_nodes * 3, s);
   if (zrc) return zrc;
   if (nev > 1) FEA_CUDA(cudaEventRecord(ev[1], s));
 

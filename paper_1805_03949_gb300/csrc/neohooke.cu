@@ -488,7 +488,7 @@ int assemble_nh(const fea_operator* op, fea_mesh* m, const int64_t* row_ptr, con
   cudaEvent_t* ev = (cudaEvent_t*)op->events;
   const int nev = ev ? op->n_events : 0;
   if (nev > 0) FEA_CUDA(cudaEventRecord(ev[0], s));
-  const int zrc = zero_system(A, 9 * m->nnz_node, b, m->n_nodes * 3, nullptr, s);
+  const int zrc = zero_system(A, 9 * m->nnz_node, b, m->n_nodes * 3, s);
   if (zrc) return zrc;
   if (nev > 1) FEA_CUDA(cudaEventRecord(ev[1], s));
 

@@ -5,7 +5,6 @@
 #include <cstring>
 
 #include "fea_internal.cuh"
-#include "zero.cuh"
 
 namespace fea {
 
@@ -61,8 +60,7 @@ static int ensure_items(fea_mesh* m, int chunk, cudaStream_t s) {
 static int chunk_of(const fea_operator* op) { return op->chunk > 0 ? op->chunk : kDefaultChunk; }
 
 // scheduler state of one persistent launch: items of the operator's chunk,
-// and the queue heads, reset on the stream (the stealing counter is left to
-// the caller, which clears it with the system)
+// the stealing counter and the queue heads, reset on the stream
 static int prepare_sched(const fea_operator* op, fea_mesh* m, cudaStream_t s, SchedArgs* S) {
   if (op->chunk < 0 || op->chunk > (1 << 24)) return fail(FEA_ERR_ARG, "fea_assemble: chunk must be in [0, 2^24]");
   const bool queues = op->schedule == FEA_SCHED_QUEUES || op->schedule == FEA_SCHED_QUEUES_STEAL;
@@ -71,6 +69,7 @@ static int prepare_sched(const fea_operator* op, fea_mesh* m, cudaStream_t s, Sc
   if (op->n_ctas < 0) return fail(FEA_ERR_ARG, "fea_assemble: n_ctas must be >= 0");
   int rc = ensure_items(m, chunk_of(op), s);
   if (rc) return rc;
+  FEA_CUDA(cudaMemsetAsync(m->sched_counter, 0, sizeof(int32_t), s));
   if (op->schedule == FEA_SCHED_QUEUES_STEAL) {
     if (m->sched_heads_n < op->n_ctas) {
       cudaFree(m->sched_heads);
@@ -106,8 +105,10 @@ int assemble_persistent(const fea_operator* op, fea_mesh* m, const int64_t* row_
   SchedArgs S;
   int rc = prepare_sched(op, m, s, &S);
   if (rc) return rc;
-  rc = zero_system(A, (int64_t)D * D * m->nnz_node, b, m->n_nodes * D, m->sched_counter, s);
-  if (rc) return rc;
+  // memsets, not the clearing kernel of zero.cuh: the persistent kernel does not
+  // overlap it, and the call launches one kernel (fea_assemble_launches)
+  FEA_CUDA(cudaMemsetAsync(A, 0, (size_t)D * D * m->nnz_node * sizeof(double), s));
+  FEA_CUDA(cudaMemsetAsync(b, 0, (size_t)m->n_nodes * D * sizeof(double), s));
   if (nev > 1) FEA_CUDA(cudaEventRecord(ev[1], s));
   if (S.n_items > 0) {
     rc = op->kind == FEA_OP_J2
@@ -126,7 +127,6 @@ int element_loop_persistent(const fea_operator* op, fea_mesh* m, double* stress,
   SchedArgs S;
   int rc = prepare_sched(op, m, s, &S);
   if (rc) return rc;
-  FEA_CUDA(cudaMemsetAsync(m->sched_counter, 0, sizeof(int32_t), s));
   if (nev > 1) FEA_CUDA(cudaEventRecord(ev[1], s));
   if (S.n_items > 0) {
     rc = launch_persistent_j2(op, m, nullptr, nullptr, nullptr, nullptr, S, op->n_ctas, false, s, nullptr, stress,

@@ -9,11 +9,12 @@
 
 namespace fea {
 
-// Systems up to this size are cleared by one kernel (A, b and the scheduler's
-// counter), and the tile kernel that follows may start while it runs and wait
-// for it only before its first addition: on small meshes the launches and the
-// tiles' gathers take longer than the work (22,950 tet4, Poisson: 16.4 us per
-// step with two memsets, 14.0 with the kernel, 12.7 with the early start).
+// Systems up to this size are cleared by one kernel in the launches per
+// element type, which fea_assemble_launches counts, and the tile kernel that
+// follows may start while it runs and wait for it only before its first
+// addition: on small meshes the launches and the tiles' gathers take longer
+// than the work (22,950 tet4, Poisson: 16.4 us per step with two memsets, 14.0
+// with the kernel, 12.7 with the early start).
 // Larger ones keep cudaMemsetAsync, which writes at 7.5 TB/s where the kernel
 // reaches 5.8.
 constexpr int64_t kSmallSystemBytes = 32ll << 20;
@@ -33,8 +34,8 @@ inline bool starts_early(unsigned grid, bool after_clearing, bool light) {
   return grid <= 64 || (after_clearing && (light || grid >= 1024));
 }
 
-// Clear A [nnz] and b [nb]; counter (may be nullptr): an int32 to set to 0.
-int zero_system(double* A, int64_t nnz, double* b, int64_t nb, int32_t* counter, cudaStream_t s);
+// Clear A [nnz] and b [nb].
+int zero_system(double* A, int64_t nnz, double* b, int64_t nb, cudaStream_t s);
 
 // Device side of the early start: let the next kernel of the stream start; wait
 // until the kernels before have finished and their writes are visible (nothing
