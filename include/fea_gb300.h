@@ -126,8 +126,9 @@ typedef enum {
  * cut into ceil(n_t / chunk) items (fea_work_items lists them). */
 typedef enum {
   FEA_SCHED_PER_TYPE = 0, /* one launch per element type (per color class for FEA_SCATTER_COLOR) */
-  FEA_SCHED_STEAL = 1,    /* one persistent launch over every type: n_ctas CTAs take items from a
-                             global counter (dynamic work stealing), in list order, or in the order
+  FEA_SCHED_STEAL = 1,    /* one persistent launch over every type: n_ctas CTAs (if the items are at
+                             most 3/4 of them, one per item) take items from a global counter
+                             (dynamic work stealing), in list order, or in the order
                              queue_d gives when queue_d is set and queue_off_d is NULL (a permutation
                              of all items, e.g. by decreasing predicted cost) */
   FEA_SCHED_QUEUES = 2,   /* one persistent launch: CTA c processes exactly the items

@@ -996,7 +996,7 @@ static int launch_persistent_k(const PersistAsmArgs& args, int n_ctas, bool dry,
   }
   if (grid_out) *grid_out = grid;
   if (!dry) {
-    kern<<<grid, 128, smem, s>>>(args);
+    kern<<<sched_ctas(args.S, grid), 128, smem, s>>>(args);
     FEA_CUDA(cudaGetLastError());
   }
   return FEA_OK;

@@ -754,7 +754,7 @@ static int launch_persistent_j2_t(const PersistJ2Args& args, int n_ctas, bool dr
   }
   if (grid_out) *grid_out = grid;
   if (!dry) {
-    kern<<<grid, 128, smem, s>>>(args);
+    kern<<<sched_ctas(args.S, grid), 128, smem, s>>>(args);
     FEA_CUDA(cudaGetLastError());
   }
   return FEA_OK;

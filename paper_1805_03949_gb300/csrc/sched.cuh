@@ -43,6 +43,21 @@ struct SchedArgs {
   unsigned long long* start_ns;
 };
 
+// CTAs to launch of a persistent grid: under STEAL one per item if the items are
+// at most three quarters of it.  The CTAs of an SM reach the counter together,
+// so with few items those of the SMs that got there first took several each,
+// and ran them side by side while other SMs had none; one CTA per item starts
+// on an SM of its own.  The more CTAs fit an SM, the worse (FP32 J2, 750 tet4,
+// 6 items: 103 us with three per SM, 200 with four, 94 with one per item; 4,096
+// hex8: 361, 419, 229; FP64 elasticity, 13,824 hex8, 108 items of 912 CTAs: 456
+// -> 234).  Near a full grid the free choice balances items of several types
+// better (FP32 diffusion, 1,216 CTAs: 778 mixed items equal, 864 hex8 items 161
+// -> 135 us, but 1,160 mixed items 153 -> 165).
+inline int sched_ctas(const SchedArgs& S, int grid) {
+  if (S.mode != FEA_SCHED_STEAL || S.n_items > grid - grid / 4) return grid;
+  return S.n_items > 0 ? S.n_items : 1;
+}
+
 __device__ __forceinline__ uint64_t global_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
