@@ -890,8 +890,13 @@ __device__ int mdep_next(const MdepArgs& A, int& cursor) {
   }
 }
 
+// CTAs per SM (launch_multidep_k): the FP32 kernels' bounds, except that the
+// any-type diffusion kernel is left to the compiler, whose registers it is
+// faster with (99,408 mixed elements: 8.54 -> 7.85 ms, FP32-adaptive 7.74 ->
+// 7.06; the hex-only kernel loses: 262,144 hex8 1.73 -> 1.80 ms).
 template <int OP, int PREC, int ONLY>
-__global__ void __launch_bounds__(128, PREC == FEA_FP64 ? 0 : OP == FEA_OP_DIFFUSION ? 5 : 3) k_multidep(const __grid_constant__ MdepArgs A) {
+__global__ void __launch_bounds__(128, PREC == FEA_FP64 ? 0 : OP == FEA_OP_ELASTICITY ? 3 : ONLY < 0 ? 0 : 5)
+    k_multidep(const __grid_constant__ MdepArgs A) {
   constexpr int MD = FEA_SCATTER_MULTIDEP;
   extern __shared__ __align__(16) unsigned char mdep_smem[];
   __shared__ int s_sub;
