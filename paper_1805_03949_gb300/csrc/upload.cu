@@ -7,10 +7,12 @@
 // counts each type per tile of elements, a scan of the counts (type-major, so
 // that an element's position among all elements of its type is one offset plus
 // its rank in the tile), and a pass that writes the lists.  The counts of the
-// types before an element give its node_map offset too.  One allocation holds
-// every array of the handle: cudaMalloc and cudaFree cost more than the
-// kernels on small meshes.  Upload and pattern of 412,500 mixed elements from
-// device arrays, one GB300: 18.1 -> 1.44 ms (with the row builder of pattern.cu).
+// types before an element give its node_map offset too.  Two allocations hold
+// every array of the handle (cudaMalloc and cudaFree cost more than the kernels
+// on small meshes): one sized by nodes and elements, and one, sized by the
+// check, for the connectivity and, with several types, their lists.  Upload and
+// pattern of 412,500 mixed elements from device arrays, one GB300: 18.1 -> 1.44
+// ms (with the row builder of pattern.cu).
 #include <algorithm>
 #include <cstring>
 #include <string>
@@ -27,6 +29,7 @@ struct UploadInfo {
   unsigned long long bad_elem;  // smallest 2 e + (0: unknown type, 1: wrong node count), or ~0
   unsigned long long bad_conn;  // smallest t with conn[t] out of range, or ~0
   int64_t off0, len;            // conn_offsets[0], conn_offsets[E]
+  unsigned types;               // bit t: elements of type t
   int64_t base[kNumTypes + 1];  // elements of the types before t
 };
 
@@ -59,7 +62,10 @@ __global__ void __launch_bounds__(kUpThreads) k_upload_count(const uint8_t* type
     }
   }
   __syncthreads();
-  if (threadIdx.x < kNumTypes) tile_cnt[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = cnt[threadIdx.x];
+  if (threadIdx.x < kNumTypes) {
+    tile_cnt[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = cnt[threadIdx.x];
+    if (cnt[threadIdx.x]) atomicOr(&info->types, 1u << threadIdx.x);
+  }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     info->off0 = off[0];
     info->len = off[E];
@@ -171,7 +177,7 @@ int upload_mesh(const fea_mesh_desc* d, cudaStream_t s, fea_mesh** out) {
     return fail(FEA_ERR_OOM, "fea_mesh_upload: cudaMalloc of " + std::to_string(bytes) + " bytes failed");
   };
   const size_t a_coords = place(3 * N * 8), a_off = place((E + 1) * 8), a_moff = place((E + 1) * 8),
-               a_gmoff = place(E * 8), a_ids = place(E * 4), a_types = place(E), a_status = place(sizeof(DevStatus)),
+               a_types = place(E), a_status = place(sizeof(DevStatus)),
                a_info = place(sizeof(UploadInfo)), a_tiles = place(kNumTypes * tiles * 8);
   int rc = alloc(&m->arena);
   if (rc) return leave(rc);
@@ -183,8 +189,6 @@ int upload_mesh(const fea_mesh_desc* d, cudaStream_t s, fea_mesh** out) {
   UploadInfo* info = reinterpret_cast<UploadInfo*>(base + a_info);
   int64_t* tile_cnt = reinterpret_cast<int64_t*>(base + a_tiles);
   uint8_t* types = base + a_types;
-  int32_t* ids = reinterpret_cast<int32_t*>(base + a_ids);
-  int64_t* gmoff = reinterpret_cast<int64_t*>(base + a_gmoff);
 
   const cudaMemcpyKind kind = d->on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   FEA_UP(cudaMemcpyAsync(m->conn_off, d->conn_offsets, (E + 1) * 8, kind, s));
@@ -210,11 +214,17 @@ int upload_mesh(const fea_mesh_desc* d, cudaStream_t s, fea_mesh** out) {
   const int64_t L = got.len;
   m->conn_len = L;
   bytes = 0;
-  const size_t a_conn = place(L * 4), a_packed = place(L * 4);
+  // the lists per type only where there are several types
+  const bool lists = (got.types & (got.types - 1)) != 0;
+  const size_t a_conn = place(L * 4), a_gmoff = place(lists ? E * 8 : 0), a_ids = place(lists ? E * 4 : 0),
+               a_packed = place(lists ? L * 4 : 0);
   rc = alloc(&m->arena_conn);
   if (rc) return leave(rc);
-  m->conn = reinterpret_cast<int32_t*>(m->arena_conn + a_conn);
-  int32_t* packed = reinterpret_cast<int32_t*>(m->arena_conn + a_packed);
+  base = m->arena_conn;
+  m->conn = reinterpret_cast<int32_t*>(base + a_conn);
+  int32_t* packed = reinterpret_cast<int32_t*>(base + a_packed);
+  int32_t* ids = reinterpret_cast<int32_t*>(base + a_ids);
+  int64_t* gmoff = reinterpret_cast<int64_t*>(base + a_gmoff);
   FEA_UP(cudaMemcpyAsync(m->coords, d->coords, 3 * N * 8, kind, s));
   FEA_UP(cudaMemcpyAsync(m->conn, d->conn, L * 4, kind, s));
   k_conn_check<<<grid_for(L, 256), 256, 0, s>>>(m->conn, L, (int32_t)N, info);
