@@ -163,6 +163,44 @@ def variant_operators(fea) -> dict:
             for name, (prec, sc) in VARIANTS.items()}
 
 
+def summary_line(report, path):
+    """The printed line of a run: the report without its tables, which stay in the file `path`.  Of them the line keeps
+    each variant's time, roofline fraction and error verdict, and each workload's times, the fraction of its fastest
+    one and whether every error is within its bar."""
+    tables = ("variants", "errors", "workloads", "spmv", "neohooke", "first_call_s", "autotuned", "rows_plan")
+
+    def short(x):
+        return float(f"{x:.4g}")
+
+    def within(err):
+        return err["within_bar"] if "within_bar" in err else all(within(e) for e in err.values())
+
+    def workload(w):
+        ms, roof = w["ms"], w["roofline"]
+        if isinstance(ms, dict):
+            out = {"ms": {k: short(v) for k, v in ms.items()}, "frac": short(roof[min(ms, key=ms.get)]["frac"])}
+        else:
+            out = {"ms": short(ms), "frac": short(roof["frac"])}
+        if "error" in w:
+            out["within_bar"] = within(w["error"])
+        if "element_loop" in w:
+            out["element_loop"] = workload(w["element_loop"])
+        return out
+
+    line = {k: v for k, v in report.items() if k not in tables}
+    line["variants"] = {k: {"ms": short(v["ms_per_step"]), "frac": short(v["step_roofline"]["frac"])}
+                        for k, v in report["variants"].items()}
+    for k, e in report.get("errors", {}).items():
+        line["variants"][k]["within_bar"] = e["within_bar"]
+    if report.get("spmv"):
+        line["spmv"] = {k: short(report["spmv"][k]) for k in ("ms", "frac", "fp64_frac")}
+    if report.get("neohooke"):
+        line["neohooke"] = {k: short(v["ms"]) for k, v in report["neohooke"].items() if isinstance(v, dict)}
+    line["workloads"] = {k: workload(w) for k, w in report.get("workloads", {}).items()}
+    line["report"] = path
+    return line
+
+
 def kernels_after_zeroing(fea, system, name, launches):
     """Of a variant's `launches` per step on a hex8 mesh, those after the zeroing interval of the events: block-task
     plans clear the rows of A they add to, and the launches per element type a small system, with one kernel inside
@@ -742,7 +780,14 @@ def run_ours(args, rank, world, local_rank):
             sysm.close()
             torch.cuda.empty_cache()
             line["workloads"] = other_workloads(args, dev, pk)
-        print(json.dumps(line), flush=True)
+        path = args.report
+        try:
+            os.makedirs(os.path.dirname(os.path.abspath(path)), exist_ok=True)
+            with open(path, "w") as f:
+                json.dump(line, f, indent=1)
+        except OSError as e:
+            path = f"not written: {e}"
+        print(json.dumps(summary_line(line, path)), flush=True)
     sysm.close()
     if dist is not None:
         dist.barrier()
@@ -1364,6 +1409,8 @@ def make_parser() -> argparse.ArgumentParser:
                     help="skip every oracle step: the CPU baseline and the error of each result")
     ap.add_argument("--clocks-dir", default=tempfile.gettempdir(),
                     help="where the raw nvidia-smi clock samples of the timed region are written")
+    ap.add_argument("--report", default=os.path.join(ROOT, "_build", "bench_report.json"),
+                    help="file for the whole report (the printed line leaves out its tables)")
     ap.add_argument("--workloads", "--configs", dest="workloads", default="poisson,hybrid,j2,batch",
                     help="other workloads timed after the headline one (comma list of poisson, hybrid, j2, "
                          "batch; '' for none)")
