@@ -5,11 +5,11 @@
 // Every SM runs warps of independent fused multiply-add chains long enough
 // that launch and tail costs vanish; the rate is the FMA count x 2 over the
 // kernel's CUDA-event time.  The chains are x <- x m + c with |m| < 1, so the
-// values stay normal and finite whatever the length.  m and c are arguments, so
-// that the loop keeps them in registers: as literals they became constant
-// operands, with which an FP64 instruction of a warp takes 19.9 cycles of the
-// SM's FP64 unit instead of 16.7 (1.01 to 1.06 against 1.20 TFLOP/s), below what the
-// assembly kernels reach.
+// values stay normal and finite whatever the length.  Their two factors are the
+// kernel's last arguments, side by side on a 16-byte boundary: an FP64
+// instruction of a warp then takes 16 cycles of the SM's FP64 unit.  As literals,
+// or with the pointer after them, the same loop took 19 (measured; 1.05 against
+// 1.25 TFLOP/s at 2,070 MHz), slower than the assembly kernels run the unit.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -36,7 +36,7 @@ constexpr int kProbeChains = 8;
 constexpr int kProbeThreads = 256;
 
 template <typename T>
-__global__ void __launch_bounds__(kProbeThreads) k_fma_probe(int64_t iters, T m, T c, T* out) {
+__global__ void __launch_bounds__(kProbeThreads) k_fma_probe(int64_t iters, T* out, T m, T c) {
   T x[kProbeChains];
 #pragma unroll
   for (int k = 0; k < kProbeChains; ++k) x[k] = (T)(threadIdx.x + 1 + k) * (T)1e-3;
@@ -68,9 +68,9 @@ static int run_probe(int64_t iters, double* flops, cudaStream_t s) {
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) {
     rc = fail(FEA_ERR_CUDA, "fea_peak_probe: cudaEventCreate failed");
   } else {
-    k_fma_probe<T><<<grid, kProbeThreads, 0, s>>>(iters / 8 + 4, m, c, out);  // warm-up (clocks, caches)
+    k_fma_probe<T><<<grid, kProbeThreads, 0, s>>>(iters / 8 + 4, out, m, c);  // warm-up (clocks, caches)
     cudaEventRecord(e0, s);
-    k_fma_probe<T><<<grid, kProbeThreads, 0, s>>>(iters, m, c, out);
+    k_fma_probe<T><<<grid, kProbeThreads, 0, s>>>(iters, out, m, c);
     cudaEventRecord(e1, s);
     cudaError_t e = cudaEventSynchronize(e1);
     if (e == cudaSuccess) e = cudaGetLastError();
