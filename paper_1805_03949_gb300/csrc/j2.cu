@@ -85,7 +85,13 @@ struct J2Cfg {
     float H[EPC][NQ][grad_stride(NN)];  // h_a = n grad N_a
     float C[EPC][NQ][4];      // W, W lam', W mu', W beta
     float S[EPC][NQ][6];      // W sigma (xx, yy, zz, xy, yz, xz)
-    typename CoopScatter<NN, FEA_SCATTER_ATOMIC>::Rows rows[WARPS];  // (the cooperative scatter's)
+  };
+  // with the cooperative scatter's rows, where its staging fits the place of the
+  // coordinates and displacements (every type but pyramids)
+  using CS = CoopScatter<NN, FEA_SCATTER_ATOMIC>;
+  static constexpr bool kCoop = WARPS * CS::kVals * sizeof(float) <= sizeof(Fields);
+  struct CoopSmem : Smem {
+    typename CS::Rows rows[WARPS];
   };
 };
 
@@ -350,7 +356,7 @@ __device__ __forceinline__ void j2_tile_body(Smem& sm, const RefRule& rr, const 
     // the cooperative scatter stages its values where the coordinates and
     // displacements were
     float* vals = reinterpret_cast<float*>(&sm) + warp * CS::kVals;
-    constexpr bool kCoop = CS::kOn && Cfg::WARPS * CS::kVals * sizeof(float) <= 2 * sizeof(sm.X);
+    constexpr bool kCoop = CS::kOn && Cfg::kCoop;
     if constexpr (kCoop) {
       CS::begin(sm.rows[warp], P, active, g, a);
     }
@@ -559,21 +565,25 @@ __device__ __forceinline__ void j2_pair_body(typename J2PairCfg<TYPE, SLOT>::Sme
 template <int TYPE, int SLOT, int PREC, bool POINTS = false>
 struct J2Tile {
   using Cfg = J2Cfg<TYPE, SLOT>;
-  using Smem = std::conditional_t<POINTS, typename Cfg::Fields, typename Cfg::Smem>;
+  template <int SC>
+  using Smem = std::conditional_t<POINTS, typename Cfg::Fields,
+                                  std::conditional_t<SC == FEA_SCATTER_ATOMIC && Cfg::kCoop, typename Cfg::CoopSmem,
+                                                     typename Cfg::Smem>>;
   template <int SC>
   __device__ static __forceinline__ void run(unsigned char* raw, const RefRule& rr, const J2Params& P, int64_t e0,
                                              int64_t n_end) {
-    j2_tile_body<TYPE, SLOT, SC, !POINTS>(*reinterpret_cast<Smem*>(raw), rr, P, e0, n_end);
+    j2_tile_body<TYPE, SLOT, SC, !POINTS>(*reinterpret_cast<Smem<SC>*>(raw), rr, P, e0, n_end);
   }
 };
 template <int TYPE, int SLOT>
 struct J2Tile<TYPE, SLOT, FEA_FP64, false> {
   using Cfg = J2PairCfg<TYPE, SLOT>;
+  template <int SC>
   using Smem = typename Cfg::Smem;
   template <int SC>
   __device__ static __forceinline__ void run(unsigned char* raw, const RefRule& rr, const J2Params& P, int64_t e0,
                                              int64_t n_end) {
-    j2_pair_body<TYPE, SLOT, SC>(*reinterpret_cast<Smem*>(raw), rr, P, e0, n_end);
+    j2_pair_body<TYPE, SLOT, SC>(*reinterpret_cast<Smem<SC>*>(raw), rr, P, e0, n_end);
   }
 };
 
@@ -590,7 +600,7 @@ __global__ void __launch_bounds__(128, POINTS || PREC == FEA_FP64 || SC != FEA_S
 template <int TYPE, int SLOT, int PREC, int SC, bool POINTS = false>
 static int launch_j2(const J2Params& P, cudaStream_t s) {
   using T = J2Tile<TYPE, SLOT, PREC, POINTS>;
-  constexpr size_t smem = sizeof(typename T::Smem);
+  constexpr size_t smem = sizeof(typename T::template Smem<SC>);
   static_assert(smem <= 227 * 1024, "J2 tile exceeds shared memory");
   auto kern = k_j2_tile<TYPE, SLOT, PREC, SC, POINTS>;
   if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -632,7 +642,7 @@ struct PersistJ2Args {
 template <int PREC, bool POINTS>
 struct PersistJ2Cfg {
   template <int TYPE, int SLOT>
-  static constexpr size_t bytes() { return sizeof(typename J2Tile<TYPE, SLOT, PREC, POINTS>::Smem); }
+  static constexpr size_t bytes() { return sizeof(typename J2Tile<TYPE, SLOT, PREC, POINTS>::template Smem<FEA_SCATTER_ATOMIC>); }
   static constexpr size_t mx(size_t a, size_t b) { return a > b ? a : b; }
   static constexpr size_t smem = mx(mx(bytes<FEA_TET4, kRuleTet4>(), bytes<FEA_PYR5, kRulePyr8>()),
                                     mx(bytes<FEA_PRISM6, kRulePrism6>(), bytes<FEA_HEX8, kRuleHex8>()));
@@ -740,7 +750,7 @@ static J2Params j2_base_params(const fea_operator* op, fea_mesh* m, const int64_
 template <int PREC, int ONLY, bool POINTS = false>
 static int launch_persistent_j2_t(const PersistJ2Args& args, int n_ctas, bool dry, cudaStream_t s, int* grid_out) {
   constexpr size_t smem = ONLY == kRuleHex8
-                              ? sizeof(typename J2Tile<FEA_HEX8, kRuleHex8, PREC, POINTS>::Smem)
+                              ? sizeof(typename J2Tile<FEA_HEX8, kRuleHex8, PREC, POINTS>::template Smem<FEA_SCATTER_ATOMIC>)
                               : PersistJ2Cfg<PREC, POINTS>::smem;
   auto kern = k_persistent_j2<PREC, ONLY, POINTS>;
   if (smem > 48 * 1024) FEA_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -883,7 +893,6 @@ int element_loop_j2(const fea_operator* op, fea_mesh* m, double* stress, cudaStr
     if (rc) return rc;
     if (2 + launched < nev) FEA_CUDA(cudaEventRecord(ev[2 + launched], s));
     ++launched;
-    if (P.early) P.early = 2;
   }
   return FEA_OK;
 }

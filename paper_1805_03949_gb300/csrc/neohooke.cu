@@ -65,10 +65,13 @@ struct NHCfg {
     float C[EPC][NQ][4];      // W mu, W lam, W (mu - lam ln J), W m
     float S[EPC][NQ][9];      // W P, row-major
   };
-  // with the cooperative scatter's rows (a plain read-modify-write scatter has
-  // the L1 cache that they would take)
+  // with the cooperative scatter's rows, where its staging fits the place of the
+  // coordinates and displacements (every type but pyramids; a plain
+  // read-modify-write scatter has the L1 cache that they would take)
+  using CS = CoopScatter<NN, FEA_SCATTER_ATOMIC>;
+  static constexpr bool kCoop = WARPS * CS::kVals * sizeof(float) <= 2 * sizeof(double[EPC][NN][3]);
   struct CoopSmem : Smem {
-    typename CoopScatter<NN, FEA_SCATTER_ATOMIC>::Rows rows[WARPS];
+    typename CS::Rows rows[WARPS];
   };
 };
 
@@ -229,7 +232,7 @@ __device__ __forceinline__ void nh_tile_body(Smem& sm, const RefRule& rr, const 
   // the cooperative scatter stages its values where the coordinates and
   // displacements were
   float* vals = reinterpret_cast<float*>(&sm) + warp * CS::kVals;
-  constexpr bool kCoop = CS::kOn && Cfg::WARPS * CS::kVals * sizeof(float) <= 2 * sizeof(sm.X);
+  constexpr bool kCoop = CS::kOn && Cfg::kCoop;
   if constexpr (kCoop) {
     CS::begin(sm.rows[warp], P, active, g, a);
   }
@@ -422,7 +425,7 @@ template <int TYPE, int SLOT, int PREC>
 struct NHTile {
   using Cfg = NHCfg<TYPE, SLOT>;
   template <int SC>
-  using Smem = std::conditional_t<SC == FEA_SCATTER_ATOMIC, typename Cfg::CoopSmem, typename Cfg::Smem>;
+  using Smem = std::conditional_t<SC == FEA_SCATTER_ATOMIC && Cfg::kCoop, typename Cfg::CoopSmem, typename Cfg::Smem>;
   template <int SC>
   __device__ static __forceinline__ void run(Smem<SC>& sm, const RefRule& rr, const NHParams& P, int64_t e0) {
     nh_tile_body<TYPE, SLOT, SC>(sm, rr, P, e0, P.n);
