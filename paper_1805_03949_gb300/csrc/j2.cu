@@ -664,9 +664,10 @@ __device__ __noinline__ void persist_j2_call(unsigned char* raw, const J2Params&
 
 // ONLY == kRuleHex8: a mesh of hexes only (one tile body); -1: any type.
 // CTAs per SM: what the shared memory (FP64) or the registers without large
-// spills allow.  The element loop could run 8, but with four times as many
-// CTAs as SM sub-partitions an item's time says little about its cost (the
-// network of the cost model explained 2 % of it, 55 % at four).
+// spills allow.  The element loop could run 8, but is no faster (512,000 hex8,
+// stealing: 2.39 ms at four, 2.42 at eight), and with that many CTAs on an SM an
+// item's time says little about its cost (the network of the cost model
+// explained 2 % of it, 55 % at four).
 template <int PREC, int ONLY, bool POINTS>
 __global__ void __launch_bounds__(128, PREC == FEA_FP64 ? 3 : POINTS || ONLY < 0 ? 4 : 5)
     k_persistent_j2(const __grid_constant__ PersistJ2Args A) {
